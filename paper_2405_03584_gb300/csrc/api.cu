@@ -268,6 +268,7 @@ void carve_state(Carver& cv, Dev& d, int64_t n, int64_t m, int64_t nR, int stiff
   d.p = cv.take<double>(n + m); d.q = cv.take<double>(n + m); d.rhs = cv.take<double>(n + m);
   d.ds = cv.take<double>(m); d.dy = cv.take<double>(m); d.dzl = cv.take<double>(n); d.dzu = cv.take<double>(n);
   d.ratio = cv.take<double>(m); d.slotR = cv.take<int32_t>(nR); d.stiff_k = cv.take<int32_t>(stiff_cap);
+  d.st_beg = cv.take<int64_t>(stiff_cap); d.st_end = cv.take<int64_t>(stiff_cap);
   d.rowk = cv.take<int32_t>(nR);
   d.sc_cnt = cv.take<int32_t>(n); d.sc_ptr = cv.take<int64_t>(n + 1);
   d.sc_slot = cv.take<int32_t>(sc_cap); d.sc_val = cv.take<double>(sc_cap); d.sc_cap = sc_cap;
@@ -786,8 +787,7 @@ cudaError_t emit_step(ipm_handle* h, int pc, bool full, cudaStream_t st, cudaStr
   if (!lowp) {
     cudaGraphConditionalHandle hp = 0;
     chk(new_handle(st, &hp));
-    chk(launch_set_cond(hp, 1u, st));
-    chk(launch_cg_init(d, g, pc, st));
+    chk(launch_cg_init(d, g, pc, st, hp));
     if (e == cudaSuccess)
       chk(add_while(st, s2, [&](cudaGraphConditionalHandle ch, cudaStream_t bs) {
             return launch_cg_body(d, g, pc, ch, bs, true, false);
@@ -798,8 +798,7 @@ cudaError_t emit_step(ipm_handle* h, int pc, bool full, cudaStream_t st, cudaStr
     chk(new_handle(st, &hp));
     chk(new_handle(st, &hf));
     chk(launch_ru_start(d, st));
-    chk(launch_set_cond(hp, 1u, st));
-    chk(launch_cg_init(d, g, pc, st));
+    chk(launch_cg_init(d, g, pc, st, hp));
     c->ru = 1;
     if (e == cudaSuccess)
       chk(add_while(st, s2, [&](cudaGraphConditionalHandle ch, cudaStream_t bs) {
@@ -807,8 +806,7 @@ cudaError_t emit_step(ipm_handle* h, int pc, bool full, cudaStream_t st, cudaStr
           }, &c->pcg, &hp));
     chk(launch_ru_end(d, g, st));
     chk(launch_refine_fallback(d, g, st));
-    chk(launch_set_cond(hf, 1u, st));
-    chk(launch_cg_init(d, g, pc, st));
+    chk(launch_cg_init(d, g, pc, st, hf));
     if (e == cudaSuccess)
       chk(add_while(st, s2, [&](cudaGraphConditionalHandle ch, cudaStream_t bs) {
             return launch_cg_body(d, g, pc, ch, bs, true, false);
@@ -835,8 +833,7 @@ cudaError_t emit_step(ipm_handle* h, int pc, bool full, cudaStream_t st, cudaStr
           }, &c->refine, &hr));
     // FP64 fallback for a step the refinement could not finish (exits at once otherwise)
     chk(launch_refine_fallback(d, g, st));
-    chk(launch_set_cond(hf, 1u, st));
-    chk(launch_cg_init(d, g, pc, st));
+    chk(launch_cg_init(d, g, pc, st, hf));
     if (e == cudaSuccess)
       chk(add_while(st, s2, [&](cudaGraphConditionalHandle ch, cudaStream_t bs) {
             return launch_cg_body(d, g, pc, ch, bs, true, false);
@@ -1110,6 +1107,11 @@ int ipm_create(const ipm_options* opt, ipm_handle** out) {
     if (h->st4) cudaStreamDestroy(h->st4);
     if (h->ev) cudaEventDestroy(h->ev);
     delete h;
+    return IPM_ERR_CUDA;
+  }
+  if (prepare_tail() != cudaSuccess) {   // a per-device attribute: cheap to set again
+    cudaGetLastError();
+    ipm_destroy(h);
     return IPM_ERR_CUDA;
   }
   std::memset(h->hs, 0, sizeof(Scal));

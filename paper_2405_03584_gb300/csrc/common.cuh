@@ -117,6 +117,20 @@ __device__ __forceinline__ double block_reduce(double v, double* sh /* >= 32 dou
   return r;
 }
 
+// Sum over the block (at most 32 warps) into thread 0, one barrier; every thread calls it.
+__device__ __forceinline__ double block_sum0(double v, double* sh /* >= 32 doubles */) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+  v = warp_sum(v);
+  if (lane == 0) sh[wid] = v;
+  __syncthreads();
+  if (wid == 0) {
+    v = lane < nw ? sh[lane] : 0.0;
+    for (int o = 16; o > 0; o >>= 1)
+      if (o < nw) v += __shfl_xor_sync(0xffffffffu, v, o);
+  }
+  return v;
+}
+
 // Last-block-done grid reduction.  Each block stores its partial for each of NQ quantities
 // at partials[q * kMaxRedBlocks + blockIdx.x]; the last block to arrive reduces them in
 // block-index order and returns true (in all of its threads) with the totals in out[].

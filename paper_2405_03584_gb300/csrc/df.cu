@@ -162,23 +162,7 @@ __global__ void __launch_bounds__(256, 6) k_op_cols_df(Dev d) {
   if (d.aug)
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < d.m; k += (int64_t)gridDim.x * blockDim.x)
       pq = fma(d.p[d.n + k], d.q[d.n + k], pq);
-  double v[1] = {pq};
-  const int ops[1] = {0};
-  double out[1];
-  if (grid_reduce<1>(v, ops, d.partials + 16 * kMaxRedBlocks, &d.sc->ticket[T_PQ], out, sh)) {
-    if (threadIdx.x == 0) {
-      Scal* sc = d.sc;
-      const double pqv = out[0];
-      if (!(pqv > 0.0) || !isfinite(pqv)) {
-        sc->cg_done = 1;
-        if (!isfinite(pqv)) sc->status = DS_NUMERICAL;
-        sc->alpha = 0.0;
-      } else {
-        sc->alpha = sc->rz / pqv;
-      }
-      sc->pq = pqv;
-    }
-  }
+  store_pq_part(d, pq, sh);
 }
 
 cudaError_t launch_op_rows_df(const Dev& d, const Geo& g, int mode, cudaStream_t st) {

@@ -819,6 +819,8 @@ __global__ void k_stiff_compact(Dev d) {
     const int32_t row = d.arow[k];
     if (v && off < cap) {
       d.stiff_k[off] = (int32_t)k;
+      d.st_beg[off] = d.R_ptr[row];
+      d.st_end[off] = d.R_ptr[row + 1];
       d.slotR[row] = (int32_t)off;
       d.thR[row] = 0.0;
     } else {
@@ -1111,7 +1113,7 @@ cudaError_t launch_op_rows_runs(const Dev& d, const Geo& g, int mode, cudaStream
   return cudaGetLastError();
 }
 
-// q = R^T v + Hs p + (h0 + sigma) o p; p^T q -> alpha = rz / p^T q (last block).
+// q = R^T v + Hs p + (h0 + sigma) o p; p^T q by blocks.
 // MODE 0: inside PCG; MODE 1: a single operator apply (no scalars touched); MODE 2: as 1,
 // when the reduced-precision PCG asks for a residual replacement.
 template <int MODE, int G>
@@ -1139,34 +1141,23 @@ __global__ void __launch_bounds__(256, kOpColsMinBlocks) k_op_cols(Dev d) {
   if (d.aug)   // p^T q over the bottom block too (q's bottom written by the rows pass)
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < d.m; k += (int64_t)gridDim.x * blockDim.x)
       pq = fma(d.p[d.n + k], d.q[d.n + k], pq);
-  double v[1] = {pq};
-  const int ops[1] = {0};
-  double out[1];
-  if (grid_reduce<1>(v, ops, d.partials + 16 * kMaxRedBlocks, &d.sc->ticket[T_PQ], out, sh)) {
-    if (threadIdx.x == 0) {
-      Scal* sc = d.sc;
-      const double pqv = out[0];
-      if (!(pqv > 0.0) || !isfinite(pqv)) {
-        sc->cg_done = 1;                       // breakdown: keep the last iterate
-        if (!isfinite(pqv)) sc->status = DS_NUMERICAL;
-        sc->alpha = 0.0;
-      } else {
-        sc->alpha = sc->rz / pqv;
-      }
-      sc->pq = pqv;
-    }
-  }
+  store_pq_part(d, pq, sh);
 }
 
-// dx += alpha p; r -= alpha q; ||r||^2 -> convergence test.
+// The whole-chip form of the iteration's vector half (pcg.cu's cluster kernel where that does
+// not run: BLOCK32 and DENSE preconditioners, systems beyond its size).
+// alpha = rz / p^T q (npart block parts); dx += alpha p; r -= alpha q; ||r||^2 -> convergence test.
 // ZM 0 (Jacobi): z = r / M, r^T z, beta.  ZM 1 (Jacobi + low rank): z0 = r / M only.
 // ZM 2 (dense): z is left to the dense apply.
 template <int ZM>
-__global__ void k_cg_update(Dev d) {
+__global__ void k_cg_update(Dev d, int npart) {
   __shared__ double sh[32];
   if (d.sc->cg_done) return;
-  const double alpha = d.sc->alpha;
+  const double pq = sum_pq_parts(d, npart, sh);
+  const bool good = pq > 0.0 && isfinite(pq);      // else breakdown: keep the last iterate
+  const double alpha = good ? d.sc->rz / pq : 0.0;
   double rr = 0.0, rz = 0.0;
+  if (good)
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < d.nsys; j += (int64_t)gridDim.x * blockDim.x) {
     d.dx[j] = fma(alpha, d.p[j], d.dx[j]);
     const double rj = fma(-alpha, d.q[j], d.r[j]);
@@ -1184,6 +1175,13 @@ __global__ void k_cg_update(Dev d) {
   if (grid_reduce<2>(v, ops, d.partials + 17 * kMaxRedBlocks, &d.sc->ticket[T_UPD], out, sh)) {
     if (threadIdx.x == 0) {
       Scal* sc = d.sc;
+      sc->pq = pq;
+      sc->alpha = alpha;
+      if (!good) {
+        sc->cg_done = 1;
+        if (!isfinite(pq)) sc->status = DS_NUMERICAL;
+        return;
+      }
       sc->cg_iter += 1;
       sc->rr = out[0];
       if (!isfinite(out[0])) {
@@ -1368,6 +1366,7 @@ __global__ void k_cg_init_diag(Dev d) {
     const double zj = d.r[j] * d.Minv[j];
     d.z[j] = zj;
     d.p[j] = zj;
+    if (d.p32) d.p32[j] = (float)zj;
     if (d.p_df && j < d.n) d.p_df[j] = df_split(zj);
     rz = fma(d.r[j], zj, rz);
   }
@@ -1394,26 +1393,33 @@ __global__ void k_cg_p(Dev d, cudaGraphConditionalHandle h, int set_cond) {
   }
 }
 
-cudaError_t launch_cg_init(const Dev& d, const Geo& g, int precond, cudaStream_t st) {
+cudaError_t launch_cg_init(const Dev& d, const Geo& g, int precond, cudaStream_t st, cudaGraphConditionalHandle h) {
+  if (tail_runs(d, precond)) return launch_tail_init(d, precond, h, st);
+  if (h) {
+    const cudaError_t e = launch_set_cond(h, 1u, st);
+    if (e != cudaSuccess) return e;
+  }
   if (precond == PC_BLOCK32) return launch_block_apply(d, 1, st);
   if (precond == PC_DENSE) {
     k_dense_trsv<<<1, 1024, sizeof(float2) * d.n, st>>>(d, 1);
-  } else if (precond == PC_JACOBI_LR) {
-    k_cg_init_diag<<<g.eN, kBlock, 0, st>>>(d);
-    const int gs = (d.stiff_cap + 7) / 8;
-    k_stiff_u<<<gs, kBlock, 0, st>>>(d, 1);
-    k_stiff_t<<<gs, kBlock, 0, st>>>(d, 1);
-    k_stiff_corr<<<g.eN, kBlock, 0, st>>>(d, 1);
   } else {
     k_cg_init_diag<<<g.eN, kBlock, 0, st>>>(d);
+    if (precond == PC_JACOBI_LR && d.m) {
+      const int gs = (d.stiff_cap + 7) / 8;
+      k_stiff_u<<<gs, kBlock, 0, st>>>(d, 1);
+      k_stiff_t<<<gs, kBlock, 0, st>>>(d, 1);
+      k_stiff_corr<<<g.eN, kBlock, 0, st>>>(d, 1);
+    }
   }
   return cudaGetLastError();
 }
 
 cudaError_t launch_cg_body(const Dev& d, const Geo& g, int precond, cudaGraphConditionalHandle h, cudaStream_t st,
                            bool in_graph, bool lowp) {
+  const bool tail = tail_runs(d, precond);
+  int npart = g.gNc;
   if (lowp) {
-    cudaError_t e = launch_op_lp(d, g, st);
+    cudaError_t e = launch_op_lp(d, g, !tail, st);
     if (e != cudaSuccess) return e;
   } else if (d.mx) {
     launch_op_rows_mx(d, g, 0, st);
@@ -1428,21 +1434,23 @@ cudaError_t launch_cg_body(const Dev& d, const Geo& g, int precond, cudaGraphCon
     else if (d.nR) DISPATCH_G(d.g_rows, k_op_rows<0, G><<<g.gR64, kBlock, 0, st>>>(d));
     launch_lr(d, d.p, 0, st);
     DISPATCH_G(d.g_cols, k_op_cols<0, G><<<g.gN64, kBlock, 0, st>>>(d));
+    npart = g.gN64;
   }
+  if (tail) return launch_tail_iter(d, precond, npart, h, in_graph, st);
   if (precond == PC_BLOCK32) {
-    k_cg_update<2><<<g.eN, kBlock, 0, st>>>(d);
+    k_cg_update<2><<<g.eN, kBlock, 0, st>>>(d, npart);
     launch_block_apply(d, 0, st);
   } else if (precond == PC_DENSE) {
-    k_cg_update<2><<<g.eN, kBlock, 0, st>>>(d);
+    k_cg_update<2><<<g.eN, kBlock, 0, st>>>(d, npart);
     k_dense_trsv<<<1, 1024, sizeof(float2) * d.n, st>>>(d, 0);
-  } else if (precond == PC_JACOBI_LR) {
-    k_cg_update<1><<<g.eN, kBlock, 0, st>>>(d);
+  } else if (precond == PC_JACOBI_LR && d.m) {
+    k_cg_update<1><<<g.eN, kBlock, 0, st>>>(d, npart);
     const int gs = (d.stiff_cap + 7) / 8;
     k_stiff_u<<<gs, kBlock, 0, st>>>(d, 0);
     k_stiff_t<<<gs, kBlock, 0, st>>>(d, 0);
     k_stiff_corr<<<g.eN, kBlock, 0, st>>>(d, 0);
   } else {
-    k_cg_update<0><<<g.eN, kBlock, 0, st>>>(d);
+    k_cg_update<0><<<g.eN, kBlock, 0, st>>>(d, npart);
   }
   k_cg_p<<<g.eN, kBlock, 0, st>>>(d, h, in_graph ? 1 : 0);
   return cudaGetLastError();

@@ -341,7 +341,7 @@ __device__ __forceinline__ float group_gap_dot_lp(const Dev& d, const int64_t j,
   return a;
 }
 
-// q_j = sum_i q_ij w_i + Hs p + (h0 + sigma) p;  p^T q -> alpha (last block), as k_op_cols.
+// q_j = sum_i q_ij w_i + Hs p + (h0 + sigma) p;  p^T q by blocks, as k_op_cols.
 // GAP: R^T read in the gap layout (16-bit row gaps) instead of CSR.
 template <int S, int G, bool GAP>
 __global__ void __launch_bounds__(256, 6) k_op_cols_lp(Dev d, int standalone) {
@@ -377,23 +377,7 @@ __global__ void __launch_bounds__(256, 6) k_op_cols_lp(Dev d, int standalone) {
     }
   }
   if (standalone) return;
-  double v[1] = {pq};
-  const int ops[1] = {0};
-  double out[1];
-  if (grid_reduce<1>(v, ops, d.partials + 16 * kMaxRedBlocks, &d.sc->ticket[T_PQ], out, sh)) {
-    if (threadIdx.x == 0) {
-      Scal* sc = d.sc;
-      const double pqv = out[0];
-      if (!(pqv > 0.0) || !isfinite(pqv)) {
-        sc->cg_done = 1;
-        if (!isfinite(pqv)) sc->status = DS_NUMERICAL;
-        sc->alpha = 0.0;
-      } else {
-        sc->alpha = sc->rz / pqv;
-      }
-      sc->pq = pqv;
-    }
-  }
+  store_pq_part(d, pq, sh);
 }
 
 #define DISPATCH_SG(s, g, ...)                                                                   \
@@ -446,8 +430,9 @@ cudaError_t launch_op_rows_lp_runs(const Dev& d, const Geo& g, int standalone, c
   return cudaGetLastError();
 }
 
-cudaError_t launch_op_lp(const Dev& d, const Geo& g, cudaStream_t st) {
-  k_stiff_op_u<<<(d.stiff_cap + 7) / 8, kBlock, 0, st>>>(d);
+// stiff_u: the stiff rows' product with p is still to be formed (pcg.cu forms it with p).
+cudaError_t launch_op_lp(const Dev& d, const Geo& g, bool stiff_u, cudaStream_t st) {
+  if (stiff_u) k_stiff_op_u<<<(d.stiff_cap + 7) / 8, kBlock, 0, st>>>(d);
   launch_lr(d, d.p, 0, st);
   launch_rows_lp(d, g, 0, st);
   if (d.gap) DISPATCH_SG(d.storage, d.g_cols, k_op_cols_lp<S, G, true><<<g.gNc, kBlock, 0, st>>>(d, 0));
@@ -623,11 +608,14 @@ __global__ void k_ru_start(Dev d) {
 
 // dx += alpha p; r -= alpha q; ||r||^2; a replacement is asked for when ||r|| fell by
 // refine_eta since the last one, met the tolerance, or the iteration limit is reached.
-__global__ void k_ru_update(Dev d) {
+__global__ void k_ru_update(Dev d, int npart) {
   __shared__ double sh[32];
   if (d.sc->cg_done) return;
-  const double alpha = d.sc->alpha;
+  const double pq = sum_pq_parts(d, npart, sh);
+  const bool good = pq > 0.0 && isfinite(pq);      // else breakdown: keep the last iterate
+  const double alpha = good ? d.sc->rz / pq : 0.0;
   double rr = 0.0;
+  if (good)
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < d.n; j += (int64_t)gridDim.x * blockDim.x) {
     d.dx[j] = fma(alpha, d.p[j], d.dx[j]);
     const double rj = fma(-alpha, d.q[j], d.r[j]);
@@ -640,6 +628,13 @@ __global__ void k_ru_update(Dev d) {
   if (grid_reduce<1>(v, ops, d.partials + 17 * kMaxRedBlocks, &d.sc->ticket[T_UPD], out, sh)) {
     if (threadIdx.x == 0) {
       Scal* sc = d.sc;
+      sc->pq = pq;
+      sc->alpha = alpha;
+      if (!good) {
+        sc->cg_done = 1;
+        if (!isfinite(pq)) sc->status = DS_NUMERICAL;
+        return;
+      }
       sc->cg_iter += 1;
       sc->rr = out[0];
       if (!isfinite(out[0])) {
@@ -745,13 +740,19 @@ cudaError_t launch_apply_ru(const Dev& d, const Geo& g, cudaStream_t st);   // k
 // the preconditioner, the next direction (k_cg_p sets the loop condition).
 cudaError_t launch_ru_body(const Dev& d, const Geo& g, int precond, cudaGraphConditionalHandle h, cudaStream_t st,
                            bool in_graph) {
-  cudaError_t e = launch_op_lp(d, g, st);
+  const bool tail = tail_runs(d, precond);
+  cudaError_t e = launch_op_lp(d, g, !tail, st);
   if (e != cudaSuccess) return e;
-  k_ru_update<<<g.eN, kBlock, 0, st>>>(d);
+  if (tail) {
+    e = launch_tail_ru(d, precond, g.gNc, st);
+    if (e == cudaSuccess) e = launch_apply_ru(d, g, st);
+    return e == cudaSuccess ? launch_tail_ru2(d, precond, h, in_graph, st) : e;
+  }
+  k_ru_update<<<g.eN, kBlock, 0, st>>>(d, g.gNc);
   e = launch_apply_ru(d, g, st);
   if (e != cudaSuccess) return e;
   k_ru_resid<<<g.eN, kBlock, 0, st>>>(d);
-  if (precond == PC_JACOBI_LR) {
+  if (precond == PC_JACOBI_LR && d.m) {
     k_ru_z<1><<<g.eN, kBlock, 0, st>>>(d);
     e = launch_stiff_apply(d, g, st);
     if (e != cudaSuccess) return e;

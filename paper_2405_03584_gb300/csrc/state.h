@@ -54,6 +54,7 @@ struct Dev {
   int32_t* slotR;              // nR: slot of a stiff row, -1 otherwise
   int32_t* rowk;               // nR: constraint index of a row of R, -1 for the factor's rows
   int32_t* stiff_k;            // stiff_cap: constraint index of each slot
+  int64_t *st_beg, *st_end;    // stiff_cap: entries of each slot's row of R
   int32_t* sc_cnt;             // n
   int64_t* sc_ptr;             // n+1: stiff entries per variable (CSC of the stiff rows)
   int32_t* sc_slot; double* sc_val;  // sc_cap
@@ -194,6 +195,20 @@ __device__ __forceinline__ void for_row_pieces(const Dev& d, const int64_t r, co
   }
 }
 
+// p^T q of a column pass: the block's part (slot 16 of the partials); whoever updates the PCG
+// vectors next adds the parts in block order.
+__device__ __forceinline__ void store_pq_part(const Dev& d, double pq, double* sh) {
+  pq = block_sum0(pq, sh);
+  if (threadIdx.x == 0) d.partials[16 * kMaxRedBlocks + blockIdx.x] = pq;
+}
+
+// The total of npart such parts, in every thread of the block.
+__device__ __forceinline__ double sum_pq_parts(const Dev& d, int npart, double* sh) {
+  double t = 0.0;
+  for (int b = threadIdx.x; b < npart; b += blockDim.x) t += __ldcg(d.partials + 16 * kMaxRedBlocks + b);
+  return block_reduce<0>(t, sh);
+}
+
 // Launch geometry shared by the host code and the final reduction kernel.
 struct Geo {
   int gR, gM, gN;              // blocks of the row-group kernels over R rows, constraint rows, R^T rows
@@ -237,12 +252,21 @@ cudaError_t launch_precond_build(const Dev& d, const Geo& g, int precond, cudaSt
 cudaError_t launch_precond_finish(const Dev& d, const Geo& g, int precond, cudaStream_t st);  // after rhs
 // ---- right-hand side and PCG ----
 cudaError_t launch_rhs(const Dev& d, const Geo& g, int precond, cudaStream_t st);  // + Jacobi diagonal
-cudaError_t launch_cg_init(const Dev& d, const Geo& g, int precond, cudaStream_t st);
+// (h != 0: also arms the loop condition h)
+cudaError_t launch_cg_init(const Dev& d, const Geo& g, int precond, cudaStream_t st, cudaGraphConditionalHandle h = 0);
 cudaError_t launch_cg_body(const Dev& d, const Geo& g, int precond, cudaGraphConditionalHandle h, cudaStream_t st,
                            bool in_graph = true, bool lowp = false);
+// ---- the vector half of a PCG iteration as one cluster kernel (pcg.cu) ----
+bool tail_runs(const Dev& d, int precond);   // the cluster kernel covers this system
+cudaError_t prepare_tail();                  // once per process and device
+cudaError_t launch_tail_init(const Dev& d, int precond, cudaGraphConditionalHandle h, cudaStream_t st);
+cudaError_t launch_tail_iter(const Dev& d, int precond, int npart, cudaGraphConditionalHandle h, bool in_graph,
+                             cudaStream_t st);
+cudaError_t launch_tail_ru(const Dev& d, int precond, int npart, cudaStream_t st);
+cudaError_t launch_tail_ru2(const Dev& d, int precond, cudaGraphConditionalHandle h, bool in_graph, cudaStream_t st);
 // ---- reduced-precision operator and FP64 refinement (lowp.cu) ----
 cudaError_t launch_quantize(const Dev& d, cudaStream_t st);
-cudaError_t launch_op_lp(const Dev& d, const Geo& g, cudaStream_t st);
+cudaError_t launch_op_lp(const Dev& d, const Geo& g, bool stiff_u, cudaStream_t st);
 cudaError_t launch_op_rows_lp_only(const Dev& d, const Geo& g, cudaStream_t st);   // measurement
 cudaError_t launch_op_cols_lp_only(const Dev& d, const Geo& g, cudaStream_t st);
 cudaError_t launch_mirror_p32(const Dev& d, const Geo& g, cudaStream_t st);
