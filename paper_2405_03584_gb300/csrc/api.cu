@@ -414,6 +414,24 @@ int heuristic_group(double avg_nnz) {
   return g;
 }
 
+// The same for the float64 operator passes, measured on GB300 at every width over RT, dense and
+// VMAT-shaped matrices.  Two costs pull apart: a row's sum takes log2 G float64 instructions a
+// warp (each holds a quarter of an SM for 64 cycles), and few rows times few lanes leave the
+// chip without loads in flight.
+//  * rows of R (many, short): 4 lanes up to 64 entries (n = 7001, 42 a row: 7.4 us at 4, 8.0 at
+//    8, 10.9 at 16), 8 beyond (RT n = 50000, 250 a row: 141 us at 4, 121 at 8, 143 at 16; VMAT
+//    134 a row: 37.6, 31.9, 35.2);
+//  * columns (few, long): 16 lanes from 32 entries (n = 7001, 168 a column: 13.0 us at 4, 8.4 at
+//    8, 8.3 at 16, 11.7 at 32; n = 50000, 1000 a column: 207, 137, 123, 149), else 8;
+//  * so few rows that 32768 lanes are not reached: wider while 8 entries a lane remain (dense n =
+//    500, m = 1000: rows 13.8 us at 8, 5.8 at 32; columns 17.0 at 16, 12.9 at 32).
+// Reduced storages keep heuristic_group's widths: their float32 sums depend on it.
+int operator_group(double avg_nnz, int64_t rows, bool columns) {
+  int g = columns ? (avg_nnz >= 32.0 ? 16 : 8) : (avg_nnz > 64.0 ? 8 : 4);
+  while (g < 32 && rows * g < 32768 && avg_nnz >= 16.0 * g) g *= 2;
+  return g;
+}
+
 // Autotuner results per matrix signature (n, rows of R, non-zeros), process-wide, so that a
 // QP loaded again in the same process runs the same schedule (and gives the same bits).
 std::mutex g_tune_mu;
@@ -844,8 +862,7 @@ cudaError_t emit_step(ipm_handle* h, int pc, bool full, cudaStream_t st, cudaStr
   if (full) {
     chk(launch_ratio(d, g, st));
     chk(launch_update(d, g, st));
-    chk(launch_residual_summary(d, g, st));
-    chk(launch_control(d, st, ipm_loop));
+    chk(launch_residual_summary(d, g, st, RSM_CONTROL, ipm_loop));
   }
   return e;
 }
@@ -963,8 +980,7 @@ int run_iteration_direct(ipm_handle* h, int pc, int64_t* launches) {
   CUDA_TRY(h, launch_recover(d, g, st));
   CUDA_TRY(h, launch_ratio(d, g, st));
   CUDA_TRY(h, launch_update(d, g, st));
-  CUDA_TRY(h, launch_residual_summary(d, g, st));
-  CUDA_TRY(h, launch_control(d, st));
+  CUDA_TRY(h, launch_residual_summary(d, g, st, RSM_CONTROL));
   *launches += lc.ipm;
   return IPM_OK;
 }
@@ -1402,8 +1418,11 @@ static int load_qp(ipm_handle* h, const ipm_qp* qp, int64_t m_ar, void* stream) 
   carve_matrix(cvm, dv, n, m, q.nR, nnzR, nnzAT, nnzHs, h->opt.storage, want_df);
   carve_state(cvs, dv, n, m, q.nR, stiff_cap, sc_cap, dense, h->opt.storage, h->opt.max_ipm, want_df, nblk);
   dv.n = n; dv.m = m; dv.nR = q.nR; dv.nnzR = nnzR; dv.nnzHs = nnzHs; dv.nnzA = nnzAT;
-  dv.g_rows = heuristic_group(q.nR ? (double)nnzR / (double)q.nR : 0.0);
-  dv.g_cols = heuristic_group((double)nnzR / (double)n);
+  const double row_len = q.nR ? (double)nnzR / (double)q.nR : 0.0, col_len = (double)nnzR / (double)n;
+  const bool f64 = h->opt.storage == IPM_STORAGE_F64;
+  dv.g_rows = f64 ? operator_group(row_len, q.nR, false) : heuristic_group(row_len);
+  // (without a matrix the column pass is the low-rank term's rows, measured fastest at 4 lanes)
+  dv.g_cols = f64 && nnzR + nnzHs ? operator_group(col_len + (double)nnzHs / (double)n, n, true) : heuristic_group(col_len);
   dv.g_at = heuristic_group((double)nnzAT / (double)n);
   if (h->opt.lanes_rows) dv.g_rows = h->opt.lanes_rows;
   if (h->opt.lanes_cols) dv.g_cols = h->opt.lanes_cols;

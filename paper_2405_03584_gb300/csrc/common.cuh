@@ -46,7 +46,6 @@ struct Scal {
   int n_stiff, stiff_max, max_stiff_seen, chol_fail;
   // FP64 refinement of a reduced-precision Newton step
   double tol2_outer, rr_outer, refine_eta;
-  double lr_quad;               // x^T U W U^T x of the last residual summary
   // primal infeasibility certificate (Farkas): with (y, z) scaled by its largest entry,
   // |A^T y - z_l + z_u|_inf and b^T y - l^T z_l + u^T z_u
   double cert_res, cert_gap, mult_inf;
@@ -261,6 +260,31 @@ __device__ __forceinline__ double group_row_dot(const int64_t beg, const int64_t
   }
 #pragma unroll
   for (int o = G / 2; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  return a;
+}
+
+// A lane's part of group_row_dot (the same additions, not yet summed over the group).
+template <int G>
+__device__ __forceinline__ double group_row_part(const int64_t beg, const int64_t end, const int gl,
+                                                 const int32_t* __restrict__ idx, const double* __restrict__ val,
+                                                 const double* __restrict__ x) {
+  double a = 0.0;
+  int64_t e = beg + gl;
+  for (; e + 7 * G < end; e += 8 * G) {
+    double v[8];
+    int i[8];
+    double xv[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      v[k] = __ldg(val + e + k * G);
+      i[k] = __ldg(idx + e + k * G);
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) xv[k] = __ldg(x + i[k]);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) a = fma(v[k], xv[k], a);
+  }
+  for (; e < end; e += G) a = fma(__ldg(val + e), __ldg(x + __ldg(idx + e)), a);
   return a;
 }
 

@@ -144,20 +144,10 @@ __global__ void k_lr_final(Dev d, int quad) {
   }
 }
 
-// v^T U W U^T v = sum_r lrq_r (one block, fixed order) into the device scalars.
-__global__ void k_lr_quad(Dev d) {
-  __shared__ double sh[32];
-  double q = 0.0;
-  for (int64_t r = threadIdx.x; r < d.ucols; r += blockDim.x) q += d.lrq[r];
-  q = block_reduce<0>(q, sh);
-  if (threadIdx.x == 0) d.sc->lr_quad = q;
-}
-
 cudaError_t launch_lr(const Dev& d, const double* v, int quad, cudaStream_t st) {
   if (!d.ucols) return cudaSuccess;
   k_lr_part<<<d.ublocks, 256, 0, st>>>(d, v);
   k_lr_final<<<(int)std::min<int64_t>((d.ucols + 7) / 8, 4096), 256, 0, st>>>(d, quad);
-  if (quad) k_lr_quad<<<1, 1024, 0, st>>>(d);
   return cudaGetLastError();
 }
 
@@ -213,7 +203,8 @@ cudaError_t launch_diagH(const Dev& d, cudaStream_t st) {
 
 // ------------------------------------------------------------------------------ residuals
 
-// t = R x; v = w_R o t; partial sum of w_R t^2 (the factor part of x^T H x).
+// t = R x; v = w_R o t; y placed on the constraint rows of R (0 on the others); partial sum of
+// w_R t^2 (the factor part of x^T H x).
 template <int G>
 __global__ void k_rows_resid(Dev d, double* part) {
   __shared__ double sh[32];
@@ -223,179 +214,313 @@ __global__ void k_rows_resid(Dev d, double* part) {
     const double t = group_row_dot<G, false>(beg, end, glane<G>(), d.R_idx, d.R_val, d.x);
     if (ok && glane<G>() == 0) {
       const double w = d.wR[r];
+      const int32_t k = d.rowk[r];
       d.tR[r] = t;
       d.vR[r] = w * t;
+      d.vR2[r] = k >= 0 ? d.y[k] : 0.0;
       acc = fma(w * t, t, acc);
     }
   }
-  acc = block_reduce<0>(acc, sh);
+  acc = block_sum0(acc, sh);
   if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
 
-// Constraint rows: r_p = A x + s - b, r_s = s o y - mu, and y placed on R rows (vR2).
-__global__ void k_cons_resid(Dev d, double* part) {
-  __shared__ double sh[32];
-  const double mu = d.sc->mu;
-  double rp_inf = 0.0, viol = 0.0, rs_inf = 0.0, by = 0.0, sy = 0.0, ymax = 0.0;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < d.m; k += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t row = d.arow[k];
-    const double ax = d.tR[row];
-    const double rp = ax + d.s[k] - d.b[k];
-    const double rs = d.s[k] * d.y[k] - mu;
-    d.rp[k] = rp;
-    d.vR2[row] = d.y[k];
-    rp_inf = fmax(rp_inf, fabs(rp));
-    viol = fmax(viol, ax - d.b[k]);
-    rs_inf = fmax(rs_inf, fabs(rs));
-    by = fma(d.b[k], d.y[k], by);
-    ymax = fmax(ymax, fabs(d.y[k]));
-    sy = fma(d.s[k], d.y[k], sy);
+// A running maximum of numbers >= 0 kept as the bits of the float64 (their order is the
+// numbers'), so that its reductions run on the integer pipe; negative numbers and NaN are
+// passed over, as fmax does.
+__device__ __forceinline__ void keep_max(long long& m, double v) {
+  const long long b = __double_as_longlong(v);
+  if (b > m && b <= 0x7ff0000000000000ll) m = b;
+}
+__device__ __forceinline__ void keep_abs_max(long long& m, double v) { keep_max(m, fabs(v)); }
+__device__ __forceinline__ long long warp_imax(long long m) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long t = __shfl_xor_sync(0xffffffffu, m, o);
+    m = t > m ? t : m;
   }
-  const int K = kMaxRedBlocks;
-  double v;
-  v = block_reduce<1>(rp_inf, sh); if (threadIdx.x == 0) part[1 * K + blockIdx.x] = v;
-  v = block_reduce<1>(viol, sh);   if (threadIdx.x == 0) part[2 * K + blockIdx.x] = v;
-  v = block_reduce<1>(rs_inf, sh); if (threadIdx.x == 0) part[3 * K + blockIdx.x] = v;
-  v = block_reduce<0>(by, sh);     if (threadIdx.x == 0) part[4 * K + blockIdx.x] = v;
-  v = block_reduce<0>(sy, sh);     if (threadIdx.x == 0) part[5 * K + blockIdx.x] = v;
-  v = block_reduce<1>(ymax, sh);   if (threadIdx.x == 0) part[28 * K + blockIdx.x] = v;
+  return m;
+}
+
+// Slots of the partials of a residual summary: rows (RS_XFX), constraint rows, variables.
+enum ResidSlot { RS_XFX = 0, RS_RP = 1, RS_VIOL = 2, RS_RS = 3, RS_BY = 4, RS_SY = 5, RS_RD = 6, RS_HX = 7,
+                 RS_ATY = 8, RS_RC = 9, RS_XHX = 10, RS_CX = 11, RS_LU = 12, RS_TZ = 14, RS_BVIOL = 15,
+                 RS_YMAX = 28, RS_CERT = 29, RS_ZMAX = 30 };
+
+// Constraint rows (block b of nb): r_p = A x + s - b, r_s = s o y - mu and their scalar parts.
+__device__ void cons_resid(const Dev& d, double* part, int b, int nb) {
+  __shared__ long long sm[4][8];
+  __shared__ double sh[2][8];
+  const double mu = d.sc->mu;
+  long long rp_inf = 0, viol = 0, rs_inf = 0, ymax = 0;
+  double by = 0.0, sy = 0.0;
+  for (int64_t k = b * (int64_t)kBlock + threadIdx.x; k < d.m; k += (int64_t)nb * kBlock) {
+    const double ax = d.tR[d.arow[k]], s = d.s[k], y = d.y[k], bk = d.b[k];
+    const double rp = ax + s - bk;
+    d.rp[k] = rp;
+    keep_abs_max(rp_inf, rp);
+    keep_max(viol, ax - bk);
+    keep_abs_max(rs_inf, s * y - mu);
+    by = fma(bk, y, by);
+    keep_abs_max(ymax, y);
+    sy = fma(s, y, sy);
+  }
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  rp_inf = warp_imax(rp_inf);
+  viol = warp_imax(viol);
+  rs_inf = warp_imax(rs_inf);
+  ymax = warp_imax(ymax);
+  by = warp_sum(by);
+  sy = warp_sum(sy);
+  if (lane == 0) {
+    sm[0][w] = rp_inf; sm[1][w] = viol; sm[2][w] = rs_inf; sm[3][w] = ymax;
+    sh[0][w] = by; sh[1][w] = sy;
+  }
+  __syncthreads();
+  if (w == 0) {
+    const int q = lane >> 3, i = lane & 7;
+    long long m = sm[q][i];
+    double v = q < 2 ? sh[q][i] : 0.0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+      const long long t = __shfl_xor_sync(0xffffffffu, m, o);
+      m = t > m ? t : m;
+      v += __shfl_xor_sync(0xffffffffu, v, o);
+    }
+    const int mslot[4] = {RS_RP, RS_VIOL, RS_RS, RS_YMAX}, sslot[2] = {RS_BY, RS_SY};
+    if (i == 0) {
+      part[mslot[q] * kMaxRedBlocks + b] = __longlong_as_double(m);
+      if (q < 2) part[sslot[q] * kMaxRedBlocks + b] = v;
+    }
+  }
 }
 
 // Variables: Hx = R^T vR + Hs x + h0 o x, A^T y (over the stored A^T, y placed on R rows in
-// vR2), r_d, r_l, r_u and the scalar parts
-// of the objective, the dual objective and the complementarity sum.
+// vR2), r_d and the scalar parts of the objective, the dual objective and the complementarity
+// sum; the blocks from gcols on take the constraint rows.
+//
+// A float64 instruction holds a quarter of an SM for 64 cycles whatever its lanes do, so the
+// per-variable arithmetic (some 20 instructions) is not done by one lane in G: the groups leave
+// their sums in shared memory and the block's 256 / G variables are finished by that many
+// neighbouring threads.  The two dot products share one tree (each half of a group carries one
+// of them after the first exchange).  The maxima are reduced as integers.  n = 7001 at 16 lanes:
+// 31 us as one kernel of one-lane epilogues and twelve float64 block reductions (and 7 us for
+// the constraint rows), 11 us now for both.
 template <int G>
-__global__ void __launch_bounds__(256, 4) k_cols_resid(Dev d, double* part) {
-  __shared__ double sh[32];
+__global__ void __launch_bounds__(256, 4) k_cols_resid(Dev d, double* part, int gcols) {
+  if ((int)blockIdx.x >= gcols) {
+    cons_resid(d, part, (int)blockIdx.x - gcols, (int)gridDim.x - gcols);
+    return;
+  }
+  constexpr int C = kBlock / G;        // variables a block handles per trip
+  constexpr int S = 32 / G;            // of them per warp
+  __shared__ double st[2][4][C];
+  __shared__ double sw[4][8];
+  __shared__ long long sm[7][2];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, gl = glane<G>(), c = tid / G;
   const double mu = d.sc->mu;
-  double rd_inf = 0.0, hx_inf = 0.0, aty_inf = 0.0, rc_inf = 0.0, xHsx = 0.0, cx = 0.0, lzl = 0.0,
-         uzu = 0.0, tz = 0.0, bviol = 0.0, cert = 0.0, zmax = 0.0;
-  FOR_GROUP_ROWS(G, j, ok, d.n) {
-    const int64_t beg = ok ? d.RT_ptr[j] : 0, end = ok ? d.RT_ptr[j + 1] : 0;
-    const double hx_f = group_row_dot<G, false>(beg, end, glane<G>(), d.RT_idx, d.RT_val, d.vR);
-    const int64_t ab = ok ? d.AT_ptr[j] : 0, ae = ok ? d.AT_ptr[j + 1] : 0;
-    const double aty = group_row_dot<G, false>(ab, ae, glane<G>(), d.AT_idx, d.AT_val, d.vR2);
-    double hs = 0.0;
+  long long rd_inf = 0, hx_inf = 0, aty_inf = 0, rc_inf = 0, bviol = 0, cert = 0, zmax = 0;
+  double xHsx = 0.0, cx = 0.0, lu = 0.0, tz = 0.0;
+  int buf = 0;
+  for (int64_t j0 = (int64_t)blockIdx.x * C; j0 < d.n; j0 += (int64_t)gcols * C, buf ^= 1) {
+    const int64_t j = j0 + c;
+    const bool ok = j < d.n;
+    double a = group_row_part<G>(ok ? d.RT_ptr[j] : 0, ok ? d.RT_ptr[j + 1] : 0, gl, d.RT_idx, d.RT_val, d.vR);
+    double b = group_row_part<G>(ok ? d.AT_ptr[j] : 0, ok ? d.AT_ptr[j + 1] : 0, gl, d.AT_idx, d.AT_val, d.vR2);
+    // lower half of the group: the sum of a, upper half: of b
+    const bool up = gl & (G / 2);
+    const double keep = up ? b : a, give = up ? a : b;
+    double t = keep + __shfl_xor_sync(0xffffffffu, give, G / 2);
+#pragma unroll
+    for (int o = G / 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (gl == 0) st[buf][0][c] = t;
+    if (gl == G / 2) st[buf][1][c] = t;
     if (d.Hs_ptr) {
-      const int64_t hb = ok ? d.Hs_ptr[j] : 0, he = ok ? d.Hs_ptr[j + 1] : 0;
-      hs = group_row_dot<G, false>(hb, he, glane<G>(), d.Hs_idx, d.Hs_val, d.x);
+      const double hs = group_row_dot<G, false>(ok ? d.Hs_ptr[j] : 0, ok ? d.Hs_ptr[j + 1] : 0, gl, d.Hs_idx, d.Hs_val, d.x);
+      if (gl == 0) st[buf][2][c] = hs;
     }
-    const double lr = d.ucols ? lr_row<G>(d, j, ok, glane<G>()) : 0.0;
-    if (ok && glane<G>() == 0) {
-      const double xj = d.x[j];
-      const double hsx = hs + d.h0[j] * xj;
-      const double hx = hx_f + hsx + lr;
-      const double zl = d.zl[j], zu = d.zu[j];
-      const double rd = hx + d.c[j] + aty - zl + zu;
-      d.Hx[j] = hx;
-      d.Aty[j] = aty;
-      d.rd[j] = rd;
-      cert = fmax(cert, fabs(aty - zl + zu));
-      zmax = fmax(zmax, fmax(fabs(zl), fabs(zu)));
-      rd_inf = fmax(rd_inf, fabs(rd));
-      hx_inf = fmax(hx_inf, fabs(hx));
-      aty_inf = fmax(aty_inf, fabs(aty));
+    if (d.ucols) {
+      const double lr = lr_row<G>(d, j, ok, gl);
+      if (gl == 0) st[buf][3][c] = lr;
+    }
+    __syncthreads();
+    const int64_t jj = j0 + tid;
+    if (tid < C && jj < d.n) {
+      const double xj = d.x[jj], zl = d.zl[jj], zu = d.zu[jj], cj = d.c[jj];
+      const double hsx = (d.Hs_ptr ? st[buf][2][tid] : 0.0) + d.h0[jj] * xj;
+      const double hx = st[buf][0][tid] + hsx + (d.ucols ? st[buf][3][tid] : 0.0);
+      const double aty = st[buf][1][tid];
+      const double rd = hx + cj + aty - zl + zu;
+      d.Hx[jj] = hx;
+      d.Aty[jj] = aty;
+      d.rd[jj] = rd;
+      keep_abs_max(cert, aty - zl + zu);
+      keep_abs_max(zmax, zl);
+      keep_abs_max(zmax, zu);
+      keep_abs_max(rd_inf, rd);
+      keep_abs_max(hx_inf, hx);
+      keep_abs_max(aty_inf, aty);
       xHsx = fma(xj, hsx, xHsx);
-      cx = fma(d.c[j], xj, cx);
-      if (d.fl[j]) {
-        const double tl = xj - d.l[j];
-        rc_inf = fmax(rc_inf, fabs(tl * zl - mu));
-        lzl = fma(d.l[j], zl, lzl);
+      cx = fma(cj, xj, cx);
+      if (d.fl[jj]) {
+        const double l = d.l[jj], tl = xj - l;
+        keep_abs_max(rc_inf, tl * zl - mu);
+        lu = fma(l, zl, lu);
         tz = fma(tl, zl, tz);
-        bviol = fmax(bviol, -tl);
+        keep_max(bviol, -tl);
       }
-      if (d.fu[j]) {
-        const double tu = d.u[j] - xj;
-        rc_inf = fmax(rc_inf, fabs(tu * zu - mu));
-        uzu = fma(d.u[j], zu, uzu);
+      if (d.fu[jj]) {
+        const double u = d.u[jj], tu = u - xj;
+        keep_abs_max(rc_inf, tu * zu - mu);
+        lu = fma(-u, zu, lu);
         tz = fma(tu, zu, tz);
-        bviol = fmax(bviol, -tu);
+        keep_max(bviol, -tu);
       }
     }
   }
-  const int K = kMaxRedBlocks;
-  double v;
-  v = block_reduce<1>(rd_inf, sh);  if (threadIdx.x == 0) part[6 * K + blockIdx.x] = v;
-  v = block_reduce<1>(hx_inf, sh);  if (threadIdx.x == 0) part[7 * K + blockIdx.x] = v;
-  v = block_reduce<1>(aty_inf, sh); if (threadIdx.x == 0) part[8 * K + blockIdx.x] = v;
-  v = block_reduce<1>(rc_inf, sh);  if (threadIdx.x == 0) part[9 * K + blockIdx.x] = v;
-  v = block_reduce<0>(xHsx, sh);    if (threadIdx.x == 0) part[10 * K + blockIdx.x] = v;
-  v = block_reduce<0>(cx, sh);      if (threadIdx.x == 0) part[11 * K + blockIdx.x] = v;
-  v = block_reduce<0>(lzl, sh);     if (threadIdx.x == 0) part[12 * K + blockIdx.x] = v;
-  v = block_reduce<0>(uzu, sh);     if (threadIdx.x == 0) part[13 * K + blockIdx.x] = v;
-  v = block_reduce<0>(tz, sh);      if (threadIdx.x == 0) part[14 * K + blockIdx.x] = v;
-  v = block_reduce<1>(bviol, sh);   if (threadIdx.x == 0) part[15 * K + blockIdx.x] = v;
-  v = block_reduce<1>(cert, sh);    if (threadIdx.x == 0) part[29 * K + blockIdx.x] = v;
-  v = block_reduce<1>(zmax, sh);    if (threadIdx.x == 0) part[30 * K + blockIdx.x] = v;
+  // sums over the block in the order of a 256-thread block whose groups' first lanes hold the
+  // values: over the S groups of a warp, then over the 8 warps
+  constexpr int NW = (C + 31) / 32;    // warps that hold values
+  if (w < NW) {
+    double v[4] = {xHsx, cx, lu, tz};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+#pragma unroll
+      for (int o = S / 2; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+      if (tid < C && (tid & (S - 1)) == 0) sw[q][tid / S] = v[q];
+    }
+    long long m[7] = {rd_inf, hx_inf, aty_inf, rc_inf, bviol, cert, zmax};
+#pragma unroll
+    for (int q = 0; q < 7; ++q) {
+      m[q] = warp_imax(m[q]);
+      if (lane == 0) sm[q][w] = m[q];
+    }
+  }
+  __syncthreads();
+  if (w == 0) {
+    double v = sw[lane >> 3][lane & 7];
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    const int sslot[4] = {RS_XHX, RS_CX, RS_LU, RS_TZ};
+    if ((lane & 7) == 0) part[sslot[lane >> 3] * kMaxRedBlocks + blockIdx.x] = v;
+    const int mslot[7] = {RS_RD, RS_HX, RS_ATY, RS_RC, RS_BVIOL, RS_CERT, RS_ZMAX};
+    if (lane < 7) {
+      const long long m = NW > 1 && sm[lane][1] > sm[lane][0] ? sm[lane][1] : sm[lane][0];
+      part[mslot[lane] * kMaxRedBlocks + blockIdx.x] = __longlong_as_double(m);
+    }
+  }
 }
 
-// One block: totals of the partials, then the relative KKT residual (primal, dual, gap), the
-// objective values and the norm of the mu test.
+static __device__ void set_eta(Scal* sc);
+static __device__ void control_step(const Dev& d, double cg_rel, cudaGraphConditionalHandle h, int set_cond);
+
+// One block: totals of the partials, one warp per quantity, then the relative KKT residual
+// (primal, dual, gap), the objective values and the norm of the mu test.
 //   primal = max(viol_A, viol_bounds) / (1 + ||b||), dual = ||r_d|| / (1 + max(||c||, ||Hx||, ||A^T y||)),
 //   gap = |pobj - dobj| / (1 + |pobj| + |dobj|),
 //   ||r||_mu = max(||r_s, r_l, r_u||, (1 + |pobj|) / N_c * max(||r_p|| / (1 + ||b||), ||r_d|| / (1 + ||c||))).
-__global__ void k_resid_final(Dev d, int gR, int gM, int gN, const double* part) {
-  // all 19 block partials reduced in one pass: per thread over its blocks, then per warp by
-  // shuffles, then across warps (fixed order); sums (op 0) and maxima (op 1)
-  constexpr int NQ = 19;
-  const int slot[NQ] = {0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 28, 29, 30};
-  const int opq[NQ] = {0, 1, 1, 1, 0, 0, 1, 1, 1, 1, 0, 0, 0, 0, 0, 1, 1, 1, 1};
-  const int nbq[NQ] = {gR, gM, gM, gM, gM, gM, gN, gN, gN, gN, gN, gN, gN, gN, gN, gN, gM, gN, gN};
-  __shared__ double red[32][NQ];
-  __shared__ double res[NQ];
-  const int K = kMaxRedBlocks;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  double acc[NQ];
+// All its quotients are formed by one division, a lane each.
+// MODE RSM_START: also the complementarity mean (the start points' mu); RSM_CONTROL: also the
+// iteration's control step.  (24.6 us with every thread over all 19 quantities in turn and one
+// thread's chain of nine divisions, plus 4.4 us and a launch for the control; 5 us now.)
+constexpr int kFinalThreads = 640;
+template <int MODE>
+__global__ void __launch_bounds__(kFinalThreads) k_resid_final(Dev d, int gR, int gM, int gN, const double* part,
+                                                              cudaGraphConditionalHandle h, int set_cond) {
+  constexpr int NM = 11, NS = 5;
+  __shared__ double mx[NM], sum[NS + 1], comp[2][16];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int mslot[NM] = {RS_RP, RS_VIOL, RS_RS, RS_YMAX, RS_RD, RS_HX, RS_ATY, RS_RC, RS_BVIOL, RS_CERT, RS_ZMAX};
+  const int sslot[NS] = {RS_XFX, RS_BY, RS_XHX, RS_CX, RS_LU};
+  if (w < NS) {                                   // sums: warps 0..4
+    const int nb = w == 0 ? gR : (w == 1 ? gM : gN);
+    const double* p = part + sslot[w] * kMaxRedBlocks;
+    double acc = 0.0;
+    for (int b = lane; b < nb; b += 128) {
+      double v[4];
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    acc[q] = opq[q] == 0 ? 0.0 : -INFINITY;
-    for (int b = threadIdx.x; b < nbq[q]; b += blockDim.x) {
-      const double v = part[slot[q] * K + b];
-      acc[q] = opq[q] == 0 ? acc[q] + v : fmax(acc[q], v);
-    }
+      for (int k = 0; k < 4; ++k) v[k] = b + 32 * k < nb ? p[b + 32 * k] : 0.0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double w = __shfl_xor_sync(0xffffffffu, acc[q], o);
-      acc[q] = opq[q] == 0 ? acc[q] + w : fmax(acc[q], w);
+      for (int k = 0; k < 4; ++k)
+        if (b - lane + 32 * k < nb) acc += v[k];
     }
-    if (lane == 0) red[warp][q] = acc[q];
+    acc = warp_sum(acc);
+    if (lane == 0) sum[w] = acc;
+  } else if (w < NS + NM) {                       // maxima: warps 5..15
+    const int q = w - NS, nb = q < 4 ? gM : gN;
+    const double* p = part + mslot[q] * kMaxRedBlocks;
+    long long m = 0;
+    for (int b = lane; b < nb; b += 32) keep_max(m, p[b]);
+    m = warp_imax(m);
+    if (lane == 0) mx[q] = __longlong_as_double(m);
+  } else if (w == NS + NM && d.ucols) {           // x^T U W U^T x
+    double q = 0.0;
+    for (int64_t r = lane; r < d.ucols; r += 32) q += d.lrq[r];
+    q = warp_sum(q);
+    if (lane == 0) sum[NS] = q;
+  }
+  if (MODE == RSM_START) {
+    // the complementarity sums, added as 512 threads over the blocks, by warps, then warp by warp
+    __syncthreads();
+    if (w < 16) {
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int nb = q == 0 ? gM : gN;
+        const double* p = part + (q == 0 ? RS_SY : RS_TZ) * kMaxRedBlocks;
+        double v = 0.0;
+        for (int b = threadIdx.x; b < nb; b += 512) v += p[b];
+        v = warp_sum(v);
+        if (lane == 0) comp[q][w] = v;
+      }
+    }
   }
   __syncthreads();
-  if (threadIdx.x < NQ) {
-    const int q = threadIdx.x;
-    double t = opq[q] == 0 ? 0.0 : -INFINITY;
-    for (int w = 0; w < nw; ++w) t = opq[q] == 0 ? t + red[w][q] : fmax(t, red[w][q]);
-    res[q] = t;
+  if (w > 0) return;
+  Scal* sc = d.sc;
+  const double xHx = sum[0] + sum[2] + (d.ucols ? sum[NS] : 0.0);
+  const double pobj = 0.5 * xHx + sum[3];
+  const double by = sum[1], dobj = -0.5 * xHx - by + sum[4];
+  const double bn = sc->bnorm, cn = sc->cnorm;
+  const double nc = sc->ncomp > 0 ? (double)sc->ncomp : 1.0;
+  const double mi = fmax(d.m ? mx[3] : 0.0, mx[10]);
+  double num = 0.0, den = 1.0;
+  switch (lane) {
+    case 0: num = fmax(mx[1], mx[8]); den = 1.0 + bn; break;                       // primal
+    case 1: num = mx[4]; den = 1.0 + fmax(cn, fmax(mx[5], mx[6])); break;          // dual
+    case 2: num = fabs(pobj - dobj); den = 1.0 + fabs(pobj) + fabs(dobj); break;   // gap
+    case 3: num = mx[0]; den = 1.0 + bn; break;
+    case 4: num = mx[4]; den = 1.0 + cn; break;
+    case 5: num = mx[9]; den = mi > 0.0 ? mi : 1.0; break;
+    case 6: num = by - sum[4]; den = mi > 0.0 ? mi : 1.0; break;
+    case 7: num = 1.0 + fabs(pobj); den = nc; break;
+    case 8:
+      if (MODE == RSM_CONTROL) {
+        num = sc->rr;
+        den = sc->rhs2 > 0.0 ? sc->rhs2 : 1.0;
+      }
+      break;
+    case 9:
+      if (MODE == RSM_START) {
+        double sy = 0.0, tz = 0.0;
+        for (int i = 0; i < 16; ++i) {
+          sy += comp[0][i];
+          tz += comp[1][i];
+        }
+        num = sy + tz;
+        den = nc;
+      }
+      break;
+    default: break;
   }
-  __syncthreads();
-  const double xFx = res[0];
-  const double rp_inf = fmax(0.0, res[1]);
-  const double viol_a = fmax(0.0, res[2]);
-  const double rs_inf = fmax(0.0, res[3]);
-  const double by = res[4];
-  const double sy = res[5];
-  const double rd_inf = fmax(0.0, res[6]);
-  const double hx_inf = fmax(0.0, res[7]);
-  const double aty_inf = fmax(0.0, res[8]);
-  const double rc_inf = fmax(0.0, res[9]);
-  const double xHsx = res[10];
-  const double cx = res[11];
-  const double lzl = res[12];
-  const double uzu = res[13];
-  const double tz = res[14];
-  const double viol_b = fmax(0.0, res[15]);
-  const double ymax = d.m ? fmax(0.0, res[16]) : 0.0;
-  const double cert = fmax(0.0, res[17]);
-  const double zmax = fmax(0.0, res[18]);
-  if (threadIdx.x == 0) {
-    Scal* sc = d.sc;
-    const double xHx = xFx + xHsx + (d.ucols ? sc->lr_quad : 0.0);
-    const double pobj = 0.5 * xHx + cx;
-    const double dobj = -0.5 * xHx - by + lzl - uzu;
-    const double bn = sc->bnorm, cn = sc->cnorm;
-    const double primal = fmax(viol_a, viol_b) / (1.0 + bn);
-    const double dual = rd_inf / (1.0 + fmax(cn, fmax(hx_inf, aty_inf)));
-    const double gap = fabs(pobj - dobj) / (1.0 + fabs(pobj) + fabs(dobj));
+  const double quot = num / den;
+  double cg_rel = 0.0;
+  if (MODE == RSM_CONTROL) cg_rel = sqrt(__shfl_sync(0xffffffffu, quot, 8));
+  const double primal = __shfl_sync(0xffffffffu, quot, 0), dual = __shfl_sync(0xffffffffu, quot, 1),
+               gap = __shfl_sync(0xffffffffu, quot, 2), ep = __shfl_sync(0xffffffffu, quot, 3),
+               ed = __shfl_sync(0xffffffffu, quot, 4), cres = __shfl_sync(0xffffffffu, quot, 5),
+               cgap = __shfl_sync(0xffffffffu, quot, 6), sf = __shfl_sync(0xffffffffu, quot, 7),
+               cmean = __shfl_sync(0xffffffffu, quot, 9);
+  if (lane == 0) {
     sc->res_primal = primal;
     sc->res_dual = dual;
     sc->res_gap = gap;
@@ -404,30 +529,29 @@ __global__ void k_resid_final(Dev d, int gR, int gM, int gN, const double* part)
     sc->rel_kkt = rk;
     sc->pobj = pobj;
     sc->dobj = dobj;
-    sc->rp_inf = rp_inf;
-    sc->rd_inf = rd_inf;
-    sc->rc_inf = fmax(rs_inf, rc_inf);
-    const int nc = sc->ncomp > 0 ? sc->ncomp : 1;
-    const double ep = rp_inf / (1.0 + bn), ed = rd_inf / (1.0 + cn);
-    sc->rnorm_mu = fmax(fmax(rs_inf, rc_inf), (1.0 + fabs(pobj)) / nc * fmax(ep, ed));
-    sc->comp_mean = (sy + tz) / nc;
-    const double mi = fmax(ymax, zmax);
+    sc->rp_inf = mx[0];
+    sc->rd_inf = mx[4];
+    const double rc = fmax(mx[2], mx[7]);
+    sc->rc_inf = rc;
+    sc->rnorm_mu = fmax(rc, sf * fmax(ep, ed));
+    if (MODE == RSM_START) sc->comp_mean = cmean;
     sc->mult_inf = mi;
-    sc->cert_res = mi > 0.0 ? cert / mi : INFINITY;
-    sc->cert_gap = mi > 0.0 ? (by - lzl + uzu) / mi : 0.0;
+    sc->cert_res = mi > 0.0 ? cres : INFINITY;
+    sc->cert_gap = mi > 0.0 ? cgap : 0.0;
+    if (MODE == RSM_CONTROL) control_step(d, sc->rhs2 > 0.0 ? cg_rel : 0.0, h, set_cond);
   }
 }
 
-cudaError_t launch_residual_summary(const Dev& d, const Geo& g, cudaStream_t st) {
+cudaError_t launch_residual_summary(const Dev& d, const Geo& g, cudaStream_t st, int mode, cudaGraphConditionalHandle h) {
   double* part = d.partials;
-  if (d.nR) {
-    cudaMemsetAsync(d.vR2, 0, sizeof(double) * d.nR, st);
-    DISPATCH_G(d.g_rows, k_rows_resid<G><<<g.gR, kBlock, 0, st>>>(d, part));
-  }
-  if (d.m) k_cons_resid<<<g.eM, kBlock, 0, st>>>(d, part);
+  if (d.nR) DISPATCH_G(d.g_rows, k_rows_resid<G><<<g.gR, kBlock, 0, st>>>(d, part));
   launch_lr(d, d.x, 1, st);
-  DISPATCH_G(d.g_cols, k_cols_resid<G><<<g.gNr, kBlock, 0, st>>>(d, part));
-  k_resid_final<<<1, 512, 0, st>>>(d, g.gR, g.eM, g.gNr, part);
+  const int gM = d.m ? g.eM : 0;
+  DISPATCH_G(d.g_cols, k_cols_resid<G><<<g.gNr + gM, kBlock, 0, st>>>(d, part, g.gNr));
+  const int gR = d.nR ? g.gR : 0, sc = h != 0 ? 1 : 0;
+  if (mode == RSM_START) k_resid_final<RSM_START><<<1, kFinalThreads, 0, st>>>(d, gR, gM, g.gNr, part, h, sc);
+  else if (mode == RSM_CONTROL) k_resid_final<RSM_CONTROL><<<1, kFinalThreads, 0, st>>>(d, gR, gM, g.gNr, part, h, sc);
+  else k_resid_final<RSM_PLAIN><<<1, kFinalThreads, 0, st>>>(d, gR, gM, g.gNr, part, h, sc);
   return cudaGetLastError();
 }
 
@@ -449,8 +573,6 @@ cudaError_t launch_comp_resid(const Dev& d, const Geo& g, cudaStream_t st) {
 }
 
 // ------------------------------------------------------------------------------ start point
-
-static __device__ void set_eta(Scal* sc);
 
 // x0 = 0 projected into the box shrunk by delta_j = 0.1 min(1, (u_j - l_j) / 2) (0.1 for a
 // one-sided bound; 0 for a free variable).
@@ -518,7 +640,7 @@ cudaError_t launch_start_point(const Dev& d, const Geo& g, cudaStream_t st) {
   launch_lr(d, d.x, 0, st);
   DISPATCH_G(d.g_cols, k_start_z<G><<<g.gN, kBlock, 0, st>>>(d));
   if (d.m) k_start_y<<<g.eM, kBlock, 0, st>>>(d);
-  cudaError_t e = launch_residual_summary(d, g, st);
+  cudaError_t e = launch_residual_summary(d, g, st, RSM_START);
   if (e != cudaSuccess) return e;
   k_start_mu<<<1, 32, 0, st>>>(d);
   return cudaGetLastError();
@@ -537,9 +659,9 @@ static __device__ void set_eta(Scal* sc) {
 }
 
 // Algorithm 1's tail on the device: stop when rel KKT <= tol (reading of "mu <= mu_tol"),
-// else mu <- mu / 10 when ||r|| < mu; then the PCG tolerance eta for the next Newton step.
-__global__ void k_control(Dev d, cudaGraphConditionalHandle h, int set_cond) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// else mu <- mu / 10 when ||r|| < mu; then the PCG tolerance eta for the next Newton step.  One
+// thread, at the end of the residual summary; cg_rel: ||r|| / ||rhs|| of the step's PCG.
+static __device__ void control_step(const Dev& d, double cg_rel, cudaGraphConditionalHandle h, int set_cond) {
   Scal* sc = d.sc;
   sc->ipm_iter += 1;
   const double rk = sc->rel_kkt;
@@ -552,7 +674,6 @@ __global__ void k_control(Dev d, cudaGraphConditionalHandle h, int set_cond) {
   // residual above 1e-2 of its right-hand side (worse than the loosest tolerance the method
   // asks for).  A direction that misses a tight tolerance but is otherwise accurate is kept
   // (inexact Newton): the paper's doubly augmented system under Jacobi PCG lives there.
-  const double cg_rel = sc->rhs2 > 0.0 ? sqrt(sc->rr / sc->rhs2) : 0.0;
   sc->cg_fail_run = (sc->cg_conv || cg_rel <= 1e-2) ? 0 : sc->cg_fail_run + 1;
   if (sc->status == DS_RUNNING && sc->cg_fail_run >= 2) sc->status = DS_CG_STALL;
   if (sc->status == DS_NUMERICAL || sc->status == DS_CG_STALL || sc->status == DS_TIMEOUT) {
@@ -580,15 +701,10 @@ __global__ void k_control(Dev d, cudaGraphConditionalHandle h, int set_cond) {
     double* t = d.trace + (int64_t)sc->trace_rows * kTraceCols;
     t[0] = sc->ipm_iter; t[1] = mu_step; t[2] = rk; t[3] = sc->res_primal; t[4] = sc->res_dual;
     t[5] = sc->res_gap; t[6] = sc->alpha_p; t[7] = sc->alpha_d; t[8] = sc->cg_iter; t[9] = sc->cg_conv;
-    t[10] = sc->n_stiff; t[11] = sc->rhs2 > 0 ? sqrt(sc->rr / sc->rhs2) : 0.0; t[12] = sc->eta_used; t[13] = refine;
+    t[10] = sc->n_stiff; t[11] = cg_rel; t[12] = sc->eta_used; t[13] = refine;
     sc->trace_rows += 1;
   }
   if (set_cond) cudaGraphSetConditional(h, sc->stop ? 0u : 1u);
-}
-
-cudaError_t launch_control(const Dev& d, cudaStream_t st, cudaGraphConditionalHandle h) {
-  k_control<<<1, 32, 0, st>>>(d, h, h != 0 ? 1 : 0);
-  return cudaGetLastError();
 }
 
 // Start of a solve on the device: per-solve totals and the trace cleared.
@@ -644,7 +760,7 @@ __global__ void k_warm_shift(Dev d) {
 
 cudaError_t launch_warm_start(const Dev& d, const Geo& g, cudaStream_t st) {
   k_warm_shift<<<std::max(g.eN, g.eM), kBlock, 0, st>>>(d);
-  cudaError_t e = launch_residual_summary(d, g, st);
+  cudaError_t e = launch_residual_summary(d, g, st, RSM_START);
   if (e != cudaSuccess) return e;
   k_warm_mu<<<1, 32, 0, st>>>(d);
   return cudaGetLastError();

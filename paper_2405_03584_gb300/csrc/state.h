@@ -229,7 +229,7 @@ inline int gram_splits(int64_t n) {
   return tiles < 152 ? 4 : (tiles < 304 ? 2 : 1);
 }
 
-// ---- low-rank Hessian term: lrs = uw o (U^T v); quad: also v^T U W U^T v into the scalars ----
+// ---- low-rank Hessian term: lrs = uw o (U^T v); quad: also the terms of v^T U W U^T v (lrq) ----
 cudaError_t launch_lr(const Dev& d, const double* v, int quad, cudaStream_t st);
 // ---- setup and start point ----
 cudaError_t launch_diagH(const Dev& d, cudaStream_t st);
@@ -237,11 +237,13 @@ cudaError_t launch_fill_rowk(const Dev& d, cudaStream_t st);
 cudaError_t launch_densify_R(const Dev& d, cudaStream_t st);   // dense.cu: Rd from R (once per QP)
 cudaError_t launch_start_point(const Dev& d, const Geo& g, cudaStream_t st);
 // ---- residual summary at the current iterate and mu ----
-cudaError_t launch_residual_summary(const Dev& d, const Geo& g, cudaStream_t st);
+// RSM_START: with the complementarity mean; RSM_CONTROL: followed by the IPM control (mu test,
+// stop rule, eta; h: the loop condition it sets, 0: none)
+enum ResidMode { RSM_PLAIN = 0, RSM_START = 1, RSM_CONTROL = 2 };
+cudaError_t launch_residual_summary(const Dev& d, const Geo& g, cudaStream_t st, int mode = RSM_PLAIN,
+                                    cudaGraphConditionalHandle h = 0);
 // ---- complementarity residual vectors r_s, r_l, r_u (into ds, dzl, dzu) ----
 cudaError_t launch_comp_resid(const Dev& d, const Geo& g, cudaStream_t st);
-// ---- IPM control (mu test, stop rule, eta) ----
-cudaError_t launch_control(const Dev& d, cudaStream_t st, cudaGraphConditionalHandle h = 0);
 // ---- device-side IPM loop: solve start (totals reset), warm start, loop re-arming ----
 cudaError_t launch_solve_begin(const Dev& d, cudaStream_t st);
 cudaError_t launch_warm_start(const Dev& d, const Geo& g, cudaStream_t st);
