@@ -860,7 +860,6 @@ cudaError_t emit_step(ipm_handle* h, int pc, bool full, cudaStream_t st, cudaStr
   }
   chk(launch_recover(d, g, st));
   if (full) {
-    chk(launch_ratio(d, g, st));
     chk(launch_update(d, g, st));
     chk(launch_residual_summary(d, g, st, RSM_CONTROL, ipm_loop));
   }
@@ -978,7 +977,6 @@ int run_iteration_direct(ipm_handle* h, int pc, int64_t* launches) {
     CUDA_TRY(h, launch_refine_finish(d, g, st));
   }
   CUDA_TRY(h, launch_recover(d, g, st));
-  CUDA_TRY(h, launch_ratio(d, g, st));
   CUDA_TRY(h, launch_update(d, g, st));
   CUDA_TRY(h, launch_residual_summary(d, g, st, RSM_CONTROL));
   *launches += lc.ipm;

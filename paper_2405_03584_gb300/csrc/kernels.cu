@@ -777,40 +777,62 @@ cudaError_t launch_set_cond(cudaGraphConditionalHandle h, unsigned v, cudaStream
 
 // ------------------------------------------------------------------------------ diagonal update
 
-// theta = y / s; omega = w_R + theta on the constraint rows (omega preset to w_R); twice
-// theta for the doubly augmented system.
-__global__ void k_diag_m(Dev d) {
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < d.m; k += (int64_t)gridDim.x * blockDim.x) {
-    const double th = d.y[k] / d.s[k];
+// The diagonals of the Newton step and what its right-hand side has on the rows of R, in one
+// launch (six before: two copies, a fill and three kernels, 2-4 us each at n = 7001):
+//   theta = y / s; omega = w_R + theta and thR = theta on the constraint rows (w_R and 0 on the
+//   others; twice theta for the doubly augmented system, whose (1,1) block carries
+//   2 B^T D^-1 B = 2 A^T Theta A); u = theta o r_p - r_s / s placed on the rows (vR2);
+//   sigma = z_l / t_l + z_u / t_u; M0 = diag(H) + sigma; Minv = 1 / M0 until the Jacobi diagonal
+//   of the moderate rows replaces it.
+// Constraint rows are walked by constraint, not by row of R: a quotient costs a warp the same
+// for one lane as for 32, and the constraint rows lie scattered among R's.  Also clears the
+// step lengths' minima.
+__global__ void k_diag(Dev d) {
+  const double mu = d.sc->mu;
+  const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, dt = (int64_t)gridDim.x * blockDim.x;
+  if (t0 < 2) d.sc->step_min[t0] = kInfBits;
+  for (int64_t r = t0; r < d.nR; r += dt)
+    if (d.rowk[r] < 0) {
+      d.omega[r] = d.wR[r];
+      d.thR[r] = 0.0;
+      d.vR2[r] = 0.0;
+    }
+  for (int64_t k = t0; k < d.m; k += dt) {
+    const double s = d.s[k], y = d.y[k], rp = d.rp[k];
+    const double th = y / s;
     const int32_t row = d.arow[k];
     d.theta[k] = th;
-    // doubly augmented system: its (1,1) block carries 2 B^T D^-1 B = 2 A^T Theta A
     const double thf = d.aug ? 2.0 * th : th;
     d.omega[row] = d.wR[row] + thf;
     d.thR[row] = thf;
+    const double rs = s * y - mu;
+    const double u = th * rp - rs / s;                // theta o r2, r2 = r_p - r_s / y
+    d.vR2[row] = d.aug ? 2.0 * u : u;
+    if (d.aug) {
+      // eq:2x2_augmented: top r1 + 2 B^T D^-1 r2 = r1 - 2 A^T (theta o r2); bottom r2;
+      // Jacobi on the bottom block D = s / y: 1 / D = theta
+      const double r2 = rp - rs / y;
+      d.rhs[d.n + k] = r2;
+      d.r[d.n + k] = r2;
+      d.dx[d.n + k] = 0.0;
+      d.Minv[d.n + k] = th;
+    }
   }
-}
-
-// sigma = z_l / t_l + z_u / t_u; M0 = diag(H) + sigma.
-__global__ void k_diag_n(Dev d) {
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < d.n; j += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t j = t0; j < d.n; j += dt) {
     double sg = 0.0;
     if (d.fl[j]) sg += d.zl[j] / (d.x[j] - d.l[j]);
     if (d.fu[j]) sg += d.zu[j] / (d.u[j] - d.x[j]);
     d.sigma[j] = sg;
     const double m0 = d.diagH[j] + sg;
     d.M0[j] = m0;
-    d.Minv[j] = 1.0 / m0;   // 1 / M0 until the Jacobi diagonal of the moderate rows replaces it
+    d.Minv[j] = 1.0 / m0;
   }
 }
 
 cudaError_t launch_diag_update(const Dev& d, const Geo& g, cudaStream_t st) {
-  if (d.nR) {
-    cudaMemcpyAsync(d.omega, d.wR, sizeof(double) * d.nR, cudaMemcpyDeviceToDevice, st);
-    cudaMemsetAsync(d.thR, 0, sizeof(double) * d.nR, st);
-  }
-  if (d.m) k_diag_m<<<g.eM, kBlock, 0, st>>>(d);
-  k_diag_n<<<g.eN, kBlock, 0, st>>>(d);
+  const int64_t most = std::max(d.n, std::max(d.nR / 4, d.m));   // the rows' part is a fill
+  const int cap = 8 * (d.sm_count > 0 ? d.sm_count : 148);
+  k_diag<<<(int)std::max<int64_t>(1, std::min<int64_t>((most + kBlock - 1) / kBlock, cap)), kBlock, 0, st>>>(d);
   return cudaGetLastError();
 }
 
@@ -1024,29 +1046,6 @@ __global__ void k_gram_G(Dev d) {
 
 // ------------------------------------------------------------------------------ rhs
 
-// u = theta o r_p - r_s / s placed on R rows (vR2, pre-zeroed); the doubly augmented system
-// takes 2u there and its bottom block's right-hand side, start and Jacobi diagonal.
-__global__ void k_rhs_m(Dev d) {
-  const double mu = d.sc->mu;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < d.m; k += (int64_t)gridDim.x * blockDim.x) {
-    const double s = d.s[k];
-    const double rs = s * d.y[k] - mu;
-    const double u = d.theta[k] * d.rp[k] - rs / s;   // theta o r2, r2 = r_p - r_s / y
-    if (d.aug) {
-      // eq:2x2_augmented: top r1 + 2 B^T D^-1 r2 = r1 - 2 A^T (theta o r2); bottom r2;
-      // Jacobi on the bottom block D = s / y: 1 / D = theta
-      const double r2 = d.rp[k] - rs / d.y[k];
-      d.vR2[d.arow[k]] = 2.0 * u;
-      d.rhs[d.n + k] = r2;
-      d.r[d.n + k] = r2;
-      d.dx[d.n + k] = 0.0;
-      d.Minv[d.n + k] = d.theta[k];
-    } else {
-      d.vR2[d.arow[k]] = u;
-    }
-  }
-}
-
 // PCG start from ||rhs||^2: tolerance eta^2 ||rhs||^2, counters reset.
 static __device__ void finish_rhs(Scal* sc, double rhs2) {
   sc->rhs2 = rhs2;
@@ -1059,109 +1058,116 @@ static __device__ void finish_rhs(Scal* sc, double rhs2) {
   else if (rhs2 == 0.0) sc->cg_conv = 1;
 }
 
-// rhs = -r_d - r_l / t_l + r_u / t_u - A^T u (u = vR2 on the constraint rows); PCG start
-// r = rhs, dx = 0; ||rhs||^2.
-template <int G>
-__global__ void k_rhs_n(Dev d) {
-  __shared__ double sh[32];
-  const double mu = d.sc->mu;
-  double r2 = 0.0;
-  FOR_GROUP_ROWS(G, j, ok, d.n) {
-    const int64_t beg = ok ? d.AT_ptr[j] : 0, end = ok ? d.AT_ptr[j + 1] : 0;
-    const double atu = group_row_dot<G, false>(beg, end, glane<G>(), d.AT_idx, d.AT_val, d.vR2);
-    if (ok && glane<G>() == 0) {
-      double g = -d.rd[j] - atu;
-      const double xj = d.x[j];
-      if (d.fl[j]) { const double tl = xj - d.l[j]; g -= (tl * d.zl[j] - mu) / tl; }
-      if (d.fu[j]) { const double tu = d.u[j] - xj; g += (tu * d.zu[j] - mu) / tu; }
-      d.rhs[j] = g;
-      d.r[j] = g;
-      d.dx[j] = 0.0;
-      r2 = fma(g, g, r2);
-    }
-  }
-  double v[1] = {r2};
-  const int ops[1] = {0};
-  double out[1];
-  if (grid_reduce<1>(v, ops, d.partials + 20 * kMaxRedBlocks, &d.sc->ticket[T_INIT], out, sh)) {
-    if (threadIdx.x == 0) finish_rhs(d.sc, out[0]);
-  }
-}
-
-// The right-hand side and the Jacobi diagonal in one pass over A^T (u and theta live on the
-// constraint rows only): for each variable j the same entries give sum_k A_kj u_k (plain) and
-// sum_k A_kj^2 thR_k (squared).
-template <int G>
-__device__ __forceinline__ void group_row_dot_plain_sq(const int64_t beg, const int64_t end, const int gl,
-                                                       const int32_t* __restrict__ idx, const double* __restrict__ val,
-                                                       const double* __restrict__ xp, const double* __restrict__ xs,
-                                                       double& op, double& os) {
+// A lane's parts of sum_k A_kj u_k (plain) and sum_k A_kj^2 thR_k (squared): the right-hand side
+// and the Jacobi diagonal read the same entries of A^T.
+template <int G, bool SQ>
+__device__ __forceinline__ void group_plain_sq_part(const int64_t beg, const int64_t end, const int gl,
+                                                    const int32_t* __restrict__ idx, const double* __restrict__ val,
+                                                    const double* __restrict__ xp, const double* __restrict__ xs,
+                                                    double& op, double& os) {
   double a = 0.0, b = 0.0, a1 = 0.0, b1 = 0.0;
   int64_t e = beg + gl;
   for (; e + G < end; e += 2 * G) {
     const double v0 = __ldg(val + e), v1 = __ldg(val + e + G);
     const int i0 = __ldg(idx + e), i1 = __ldg(idx + e + G);
     a = fma(v0, __ldg(xp + i0), a);
-    b = fma(v0 * v0, __ldg(xs + i0), b);
+    if (SQ) b = fma(v0 * v0, __ldg(xs + i0), b);
     a1 = fma(v1, __ldg(xp + i1), a1);
-    b1 = fma(v1 * v1, __ldg(xs + i1), b1);
+    if (SQ) b1 = fma(v1 * v1, __ldg(xs + i1), b1);
   }
   if (e < end) {
     const double v0 = __ldg(val + e);
     const int i0 = __ldg(idx + e);
     a = fma(v0, __ldg(xp + i0), a);
-    b = fma(v0 * v0, __ldg(xs + i0), b);
+    if (SQ) b = fma(v0 * v0, __ldg(xs + i0), b);
   }
-  a += a1;
-  b += b1;
-#pragma unroll
-  for (int o = G / 2; o > 0; o >>= 1) {
-    a += __shfl_xor_sync(0xffffffffu, a, o);
-    b += __shfl_xor_sync(0xffffffffu, b, o);
-  }
-  op = a;
-  os = b;
+  op = a + a1;
+  os = b + b1;
 }
 
-template <int G>
-__global__ void __launch_bounds__(256, 4) k_rhs_jacobi(Dev d) {
+// rhs = -r_d - r_l / t_l + r_u / t_u - A^T u (u = vR2 on the constraint rows) and, with JAC, the
+// Jacobi diagonal's inverse; PCG start r = rhs, dx = 0; ||rhs||^2.  As in k_cols_resid the groups
+// leave their sums in shared memory and the block's 256 / G variables are finished by as many
+// neighbouring threads (four quotients each: one lane in G doing them cost 12 of 63 us at n =
+// 50000), and the two sums share one tree.
+template <int G, bool JAC>
+__global__ void __launch_bounds__(256, 4) k_rhs(Dev d) {
+  constexpr int C = kBlock / G;
+  constexpr int NW = (C + 31) / 32;
+  __shared__ double st[2][2][C];
   __shared__ double sh[32];
+  __shared__ bool s_last;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, gl = glane<G>(), c = tid / G;
   const double mu = d.sc->mu;
   double r2 = 0.0;
-  FOR_GROUP_ROWS(G, j, ok, d.n) {
-    const int64_t beg = ok ? d.AT_ptr[j] : 0, end = ok ? d.AT_ptr[j + 1] : 0;
-    double atu, dth;
-    group_row_dot_plain_sq<G>(beg, end, glane<G>(), d.AT_idx, d.AT_val, d.vR2, d.thR, atu, dth);
-    if (ok && glane<G>() == 0) {
-      d.Minv[j] = 1.0 / (d.M0[j] + dth);
-      double gj = -d.rd[j] - atu;
-      const double xj = d.x[j];
-      if (d.fl[j]) { const double tl = xj - d.l[j]; gj -= (tl * d.zl[j] - mu) / tl; }
-      if (d.fu[j]) { const double tu = d.u[j] - xj; gj += (tu * d.zu[j] - mu) / tu; }
-      d.rhs[j] = gj;
-      d.r[j] = gj;
-      d.dx[j] = 0.0;
-      r2 = fma(gj, gj, r2);
+  int buf = 0;
+  for (int64_t j0 = (int64_t)blockIdx.x * C; j0 < d.n; j0 += (int64_t)gridDim.x * C, buf ^= 1) {
+    const int64_t j = j0 + c;
+    const bool ok = j < d.n;
+    double a, b;
+    group_plain_sq_part<G, JAC>(ok ? d.AT_ptr[j] : 0, ok ? d.AT_ptr[j + 1] : 0, gl, d.AT_idx, d.AT_val, d.vR2, d.thR, a, b);
+    if (JAC) {
+      const bool up = gl & (G / 2);
+      const double keep = up ? b : a, give = up ? a : b;
+      a = keep + __shfl_xor_sync(0xffffffffu, give, G / 2);
+    } else {
+      a += __shfl_xor_sync(0xffffffffu, a, G / 2);
+    }
+#pragma unroll
+    for (int o = G / 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if (gl == 0) st[buf][0][c] = a;
+    if (JAC && gl == G / 2) st[buf][1][c] = a;
+    __syncthreads();
+    const int64_t jj = j0 + tid;
+    if (tid < C && jj < d.n) {
+      if (JAC) d.Minv[jj] = 1.0 / (d.M0[jj] + st[buf][1][tid]);
+      double g = -d.rd[jj] - st[buf][0][tid];
+      const double xj = d.x[jj];
+      if (d.fl[jj]) { const double tl = xj - d.l[jj]; g -= (tl * d.zl[jj] - mu) / tl; }
+      if (d.fu[jj]) { const double tu = d.u[jj] - xj; g += (tu * d.zu[jj] - mu) / tu; }
+      d.rhs[jj] = g;
+      d.r[jj] = g;
+      d.dx[jj] = 0.0;
+      r2 = fma(g, g, r2);
     }
   }
-  if (d.aug)   // the bottom block's right-hand side (written by k_rhs_m)
+  if (JAC && d.aug)   // the bottom block's right-hand side (written by k_diag)
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < d.m; k += (int64_t)gridDim.x * blockDim.x)
       r2 = fma(d.rhs[d.n + k], d.rhs[d.n + k], r2);
-  double v[1] = {r2};
-  const int ops[1] = {0};
-  double out[1];
-  if (grid_reduce<1>(v, ops, d.partials + 20 * kMaxRedBlocks, &d.sc->ticket[T_INIT], out, sh)) {
-    if (threadIdx.x == 0) finish_rhs(d.sc, out[0]);
+  // ||rhs||^2: block parts, added by the last block
+  if ((JAC && d.aug) || w < NW) r2 = warp_sum(r2);
+  if (lane == 0) sh[w] = r2;
+  __syncthreads();
+  double* part = d.partials + 20 * kMaxRedBlocks;
+  if (tid == 0) {
+    const int nw = JAC && d.aug ? kBlock / 32 : NW;
+    double t = sh[0];
+    for (int i = 1; i < nw; ++i) t += sh[i];
+    part[blockIdx.x] = t;
+    __threadfence();
+    s_last = atomicAdd(&d.sc->ticket[T_INIT], 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last || w > 0) return;
+  __threadfence();
+  double t = 0.0;
+  for (int b = lane; b < (int)gridDim.x; b += 32) t += __ldcg(part + b);
+  t = warp_sum(t);
+  if (lane == 0) {
+    d.sc->ticket[T_INIT] = 0u;
+    finish_rhs(d.sc, t);
   }
 }
 
 cudaError_t launch_rhs(const Dev& d, const Geo& g, int precond, cudaStream_t st) {
-  if (d.nR) cudaMemsetAsync(d.vR2, 0, sizeof(double) * d.nR, st);
-  if (d.m) k_rhs_m<<<g.eM, kBlock, 0, st>>>(d);
+  // one block per 256 / g_at variables, at most the four per SM the kernel is compiled for
+  const int gat = d.g_at > 0 ? d.g_at : 32;
+  const int64_t want = (d.n * gat + kBlock - 1) / kBlock;
+  const int nb = (int)std::min<int64_t>(want, 4 * (int64_t)(d.sm_count > 0 ? d.sm_count : 148));
   if (precond == PC_DENSE) {
-    DISPATCH_G(d.g_at, k_rhs_n<G><<<g.gN, kBlock, 0, st>>>(d));
+    DISPATCH_G(d.g_at, k_rhs<G, false><<<nb, kBlock, 0, st>>>(d));
   } else {
-    DISPATCH_G(d.g_at, k_rhs_jacobi<G><<<g.gNr, kBlock, 0, st>>>(d));
+    DISPATCH_G(d.g_at, k_rhs<G, true><<<nb, kBlock, 0, st>>>(d));
   }
   return cudaGetLastError();
 }
@@ -1643,114 +1649,159 @@ cudaError_t launch_apply_ru(const Dev& d, const Geo& g, cudaStream_t st) {
 
 // ------------------------------------------------------------------------------ recovery
 
-// A dx on the constraint rows; ds = -r_p - A dx; dy = theta (A dx + r_p) - r_s / s.
-template <int G>
-__global__ void k_recover_m(Dev d) {
-  const double mu = d.sc->mu;
-  FOR_GROUP_ROWS(G, k, ok, d.m) {
-    const int32_t row = ok ? d.arow[k] : 0;
-    const int64_t beg = ok ? d.R_ptr[row] : 0, end = ok ? d.R_ptr[row + 1] : 0;
-    const double adx = group_row_dot<G, false>(beg, end, glane<G>(), d.R_idx, d.R_val, d.dx);
-    if (ok && glane<G>() == 0) {
-      const double s = d.s[k];
-      const double rs = s * d.y[k] - mu;
-      d.ds[k] = -d.rp[k] - adx;
-      // doubly augmented: dy is the solved bottom block
-      d.dy[k] = d.aug ? d.dx[d.n + k] : d.theta[k] * (adx + d.rp[k]) - rs / s;
-    }
+// The ratio test's quotient -v / dv of a positive v that falls (INFINITY otherwise) as the bits
+// of the float64: for the quotients met here (>= 0) their order as integers is the numbers', so
+// block and grid minima run on the integer pipe and one atomic a block; NaN never wins.
+__device__ __forceinline__ void keep_ratio(long long& m, double v, double dv) {
+  if (dv < 0.0) {
+    const long long b = __double_as_longlong(-v / dv);
+    m = b < m ? b : m;
   }
 }
 
-// dz_l = (-r_l - z_l dx) / t_l, dz_u = (-r_u + z_u dx) / t_u.
-__global__ void k_recover_n(Dev d) {
-  const double mu = d.sc->mu;
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < d.n; j += (int64_t)gridDim.x * blockDim.x) {
-    const double xj = d.x[j], dxj = d.dx[j];
-    double dzl = 0.0, dzu = 0.0;
-    if (d.fl[j]) { const double tl = xj - d.l[j]; const double rl = tl * d.zl[j] - mu; dzl = (-rl - d.zl[j] * dxj) / tl; }
-    if (d.fu[j]) { const double tu = d.u[j] - xj; const double ru = tu * d.zu[j] - mu; dzu = (-ru + d.zu[j] * dxj) / tu; }
-    d.dzl[j] = dzl;
-    d.dzu[j] = dzu;
+// Minima of a block into the step's (primal, dual).
+__device__ __forceinline__ void block_ratio(const Dev& d, long long ap, long long ad) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long a = __shfl_xor_sync(0xffffffffu, ap, o), b = __shfl_xor_sync(0xffffffffu, ad, o);
+    ap = a < ap ? a : ap;
+    ad = b < ad ? b : ad;
   }
+  if ((threadIdx.x & 31) == 0) {
+    if (ap < kInfBits) atomicMin(&d.sc->step_min[0], ap);
+    if (ad < kInfBits) atomicMin(&d.sc->step_min[1], ad);
+  }
+}
+
+// alpha = min(1, tau times the minimum ratio), separate for (x, s) and (y, z) or their minimum.
+__device__ __forceinline__ void step_lengths(const Scal* sc, double& a_p, double& a_d) {
+  a_p = fmin(1.0, sc->tau * __longlong_as_double(sc->step_min[0]));
+  a_d = fmin(1.0, sc->tau * __longlong_as_double(sc->step_min[1]));
+  if (sc->equal_steps) a_p = a_d = fmin(a_p, a_d);
+}
+
+// The full direction and its ratio test in one launch.  Blocks [0, gm): constraint rows, A dx by
+// groups of G lanes, then ds = -r_p - A dx and dy = theta (A dx + r_p) - r_s / s by the block's
+// first 256 / G threads (as in k_cols_resid); the other blocks: dz_l = (-r_l - z_l dx) / t_l,
+// dz_u = (-r_u + z_u dx) / t_u.  (Five launches before, 29 us at n = 7001.)
+template <int G>
+__global__ void k_recover(Dev d, int gm) {
+  constexpr int C = kBlock / G;
+  __shared__ double st[2][C];
+  const double mu = d.sc->mu;
+  long long ap = kInfBits, ad = kInfBits;
+  const int tid = threadIdx.x;
+  if ((int)blockIdx.x < gm) {
+    int buf = 0;
+    for (int64_t k0 = (int64_t)blockIdx.x * C; k0 < d.m; k0 += (int64_t)gm * C, buf ^= 1) {
+      const int64_t kg = k0 + tid / G;
+      const bool ok = kg < d.m;
+      const int32_t row = ok ? d.arow[kg] : 0;
+      const int64_t beg = ok ? d.R_ptr[row] : 0, end = ok ? d.R_ptr[row + 1] : 0;
+      const double t = group_row_dot<G, false>(beg, end, glane<G>(), d.R_idx, d.R_val, d.dx);
+      if (glane<G>() == 0) st[buf][tid / G] = t;
+      __syncthreads();
+      const int64_t k = k0 + tid;
+      if (tid < C && k < d.m) {
+        const double adx = st[buf][tid], s = d.s[k], y = d.y[k], rp = d.rp[k];
+        const double ds = -rp - adx;
+        // doubly augmented: dy is the solved bottom block
+        // each operation rounded by itself: the value does not hang on how the compiler would fuse
+        const double dy = d.aug ? d.dx[d.n + k]
+                                : __dsub_rn(__dmul_rn(d.theta[k], adx + rp), __dsub_rn(__dmul_rn(s, y), mu) / s);
+        d.ds[k] = ds;
+        d.dy[k] = dy;
+        keep_ratio(ap, s, ds);
+        keep_ratio(ad, y, dy);
+      }
+    }
+  } else {
+    const int64_t nb = (int64_t)gridDim.x - gm;
+    for (int64_t j = ((int64_t)blockIdx.x - gm) * blockDim.x + tid; j < d.n; j += nb * blockDim.x) {
+      const double xj = d.x[j], dxj = d.dx[j];
+      double dzl = 0.0, dzu = 0.0;
+      if (d.fl[j]) {
+        const double tl = xj - d.l[j], z = d.zl[j];
+        const double rl = tl * z - mu;
+        dzl = (-rl - z * dxj) / tl;
+        keep_ratio(ap, tl, dxj);
+        keep_ratio(ad, z, dzl);
+      }
+      if (d.fu[j]) {
+        const double tu = d.u[j] - xj, z = d.zu[j];
+        const double ru = tu * z - mu;
+        dzu = (-ru + z * dxj) / tu;
+        keep_ratio(ap, tu, -dxj);
+        keep_ratio(ad, z, dzu);
+      }
+      d.dzl[j] = dzl;
+      d.dzu[j] = dzu;
+    }
+  }
+  block_ratio(d, ap, ad);
 }
 
 cudaError_t launch_recover(const Dev& d, const Geo& g, cudaStream_t st) {
-  if (d.m) DISPATCH_G(d.g_rows, k_recover_m<G><<<g.gM, kBlock, 0, st>>>(d));
-  k_recover_n<<<g.eN, kBlock, 0, st>>>(d);
+  DISPATCH_G(d.g_rows, k_recover<G><<<g.gM + g.eN, kBlock, 0, st>>>(d, g.gM));
   return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------------------ ratio test
 
-static __device__ __forceinline__ double ratio_of(double v, double dv) { return dv < 0.0 ? -v / dv : INFINITY; }
-
-__global__ void k_ratio_m(Dev d, double* part) {
-  __shared__ double sh[32];
-  double ap = INFINITY, ad = INFINITY;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < d.m; k += (int64_t)gridDim.x * blockDim.x) {
-    ap = fmin(ap, ratio_of(d.s[k], d.ds[k]));
-    ad = fmin(ad, ratio_of(d.y[k], d.dy[k]));
-  }
-  double v = block_reduce<2>(ap, sh);
-  if (threadIdx.x == 0) part[0 * kMaxRedBlocks + blockIdx.x] = v;
-  v = block_reduce<2>(ad, sh);
-  if (threadIdx.x == 0) part[1 * kMaxRedBlocks + blockIdx.x] = v;
+// The ratio test alone, on given directions (the step-level call).
+__global__ void k_ratio_begin(Dev d) {
+  if (threadIdx.x < 2) d.sc->step_min[threadIdx.x] = kInfBits;
 }
 
-__global__ void k_ratio_n(Dev d, double* part) {
-  __shared__ double sh[32];
-  double ap = INFINITY, ad = INFINITY;
+__global__ void k_ratio(Dev d) {
+  long long ap = kInfBits, ad = kInfBits;
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < d.m; k += (int64_t)gridDim.x * blockDim.x) {
+    keep_ratio(ap, d.s[k], d.ds[k]);
+    keep_ratio(ad, d.y[k], d.dy[k]);
+  }
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < d.n; j += (int64_t)gridDim.x * blockDim.x) {
     const double xj = d.x[j], dxj = d.dx[j];
-    if (d.fl[j]) { ap = fmin(ap, ratio_of(xj - d.l[j], dxj)); ad = fmin(ad, ratio_of(d.zl[j], d.dzl[j])); }
-    if (d.fu[j]) { ap = fmin(ap, ratio_of(d.u[j] - xj, -dxj)); ad = fmin(ad, ratio_of(d.zu[j], d.dzu[j])); }
+    if (d.fl[j]) { keep_ratio(ap, xj - d.l[j], dxj); keep_ratio(ad, d.zl[j], d.dzl[j]); }
+    if (d.fu[j]) { keep_ratio(ap, d.u[j] - xj, -dxj); keep_ratio(ad, d.zu[j], d.dzu[j]); }
   }
-  double v = block_reduce<2>(ap, sh);
-  if (threadIdx.x == 0) part[2 * kMaxRedBlocks + blockIdx.x] = v;
-  v = block_reduce<2>(ad, sh);
-  if (threadIdx.x == 0) part[3 * kMaxRedBlocks + blockIdx.x] = v;
+  block_ratio(d, ap, ad);
 }
 
-__global__ void k_ratio_final(Dev d, int gM, int gN, const double* part) {
-  __shared__ double sh[32];
-  auto mn = [&](int q, int nb) -> double {
-    double acc = INFINITY;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) acc = fmin(acc, part[q * kMaxRedBlocks + b]);
-    return block_reduce<2>(acc, sh);
-  };
-  const double ap = fmin(mn(0, gM), mn(2, gN));
-  const double ad = fmin(mn(1, gM), mn(3, gN));
+__global__ void k_ratio_end(Dev d) {
   if (threadIdx.x == 0) {
-    Scal* sc = d.sc;
-    double a_p = fmin(1.0, sc->tau * ap);
-    double a_d = fmin(1.0, sc->tau * ad);
-    if (sc->equal_steps) a_p = a_d = fmin(a_p, a_d);
-    sc->alpha_p = a_p;
-    sc->alpha_d = a_d;
+    double a_p, a_d;
+    step_lengths(d.sc, a_p, a_d);
+    d.sc->alpha_p = a_p;
+    d.sc->alpha_d = a_d;
   }
 }
 
 cudaError_t launch_ratio(const Dev& d, const Geo& g, cudaStream_t st) {
-  double* part = d.partials + 22 * kMaxRedBlocks;
-  if (d.m) k_ratio_m<<<g.eM, kBlock, 0, st>>>(d, part);
-  k_ratio_n<<<g.eN, kBlock, 0, st>>>(d, part);
-  k_ratio_final<<<1, 256, 0, st>>>(d, d.m ? g.eM : 0, g.eN, part);
+  k_ratio_begin<<<1, 32, 0, st>>>(d);
+  k_ratio<<<std::max(g.eN, g.eM), kBlock, 0, st>>>(d);
+  k_ratio_end<<<1, 32, 0, st>>>(d);
   return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------------------ update
 
-__global__ void k_update_n(Dev d) {
-  const double ap = d.sc->alpha_p, ad = d.sc->alpha_d;
+// x, s by alpha_p, y, z by alpha_d; one thread a block forms the step lengths.
+__global__ void k_update(Dev d) {
+  __shared__ double al[2];
+  if (threadIdx.x == 0) {
+    step_lengths(d.sc, al[0], al[1]);
+    if (blockIdx.x == 0) {
+      d.sc->alpha_p = al[0];
+      d.sc->alpha_d = al[1];
+    }
+  }
+  __syncthreads();
+  const double ap = al[0], ad = al[1];
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < d.n; j += (int64_t)gridDim.x * blockDim.x) {
     d.x[j] = fma(ap, d.dx[j], d.x[j]);
     if (d.fl[j]) d.zl[j] = fma(ad, d.dzl[j], d.zl[j]);
     if (d.fu[j]) d.zu[j] = fma(ad, d.dzu[j], d.zu[j]);
   }
-}
-
-__global__ void k_update_m(Dev d) {
-  const double ap = d.sc->alpha_p, ad = d.sc->alpha_d;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < d.m; k += (int64_t)gridDim.x * blockDim.x) {
     d.s[k] = fma(ap, d.ds[k], d.s[k]);
     d.y[k] = fma(ad, d.dy[k], d.y[k]);
@@ -1758,8 +1809,7 @@ __global__ void k_update_m(Dev d) {
 }
 
 cudaError_t launch_update(const Dev& d, const Geo& g, cudaStream_t st) {
-  k_update_n<<<g.eN, kBlock, 0, st>>>(d);
-  if (d.m) k_update_m<<<g.eM, kBlock, 0, st>>>(d);
+  k_update<<<std::max(g.eN, g.eM), kBlock, 0, st>>>(d);
   return cudaGetLastError();
 }
 

@@ -302,7 +302,7 @@ cudaError_t launch_refine_inner(const Dev& d, const Geo& g, cudaGraphConditional
 cudaError_t launch_refine_tail(const Dev& d, const Geo& g, cudaGraphConditionalHandle h, cudaStream_t st);
 cudaError_t launch_refine_fallback(const Dev& d, const Geo& g, cudaStream_t st);
 cudaError_t launch_refine_finish(const Dev& d, const Geo& g, cudaStream_t st);
-// ---- direction recovery, ratio test, update ----
+// ---- direction recovery with its ratio test; the ratio test alone; update ----
 cudaError_t launch_recover(const Dev& d, const Geo& g, cudaStream_t st);
 cudaError_t launch_ratio(const Dev& d, const Geo& g, cudaStream_t st);
 cudaError_t launch_update(const Dev& d, const Geo& g, cudaStream_t st);
