@@ -261,16 +261,22 @@ void carve_state(Carver& cv, Dev& d, int64_t n, int64_t m, int64_t nR, int stiff
   d.zl = cv.take<double>(n); d.zu = cv.take<double>(n);
   d.theta = cv.take<double>(m); d.sigma = cv.take<double>(n); d.omega = cv.take<double>(nR);
   d.M0 = cv.take<double>(n); d.Minv = cv.take<double>(n + m); d.thR = cv.take<double>(nR);
-  d.rd = cv.take<double>(n); d.rp = cv.take<double>(m); d.Hx = cv.take<double>(n); d.Aty = cv.take<double>(n);
+  d.rd = cv.take<double>(n); d.rp = cv.take<double>(m);
   d.tR = cv.take<double>(nR); d.vR = cv.take<double>(nR); d.vR2 = cv.take<double>(nR);
   // PCG vectors hold n + m entries: the doubly augmented system appends the multipliers
-  d.dx = cv.take<double>(n + m); d.r = cv.take<double>(n + m); d.z = cv.take<double>(n + m);
-  d.p = cv.take<double>(n + m); d.q = cv.take<double>(n + m); d.rhs = cv.take<double>(n + m);
-  d.ds = cv.take<double>(m); d.dy = cv.take<double>(m); d.dzl = cv.take<double>(n); d.dzu = cv.take<double>(n);
-  d.ratio = cv.take<double>(m); d.slotR = cv.take<int32_t>(nR); d.stiff_k = cv.take<int32_t>(stiff_cap);
+  d.dx = cv.take<double>(n + m); d.r = cv.take<double>(n + m); d.rhs = cv.take<double>(n + m);
+  d.ds = cv.take<double>(m); d.dy = cv.take<double>(m);
+  // one stretch of 40 n bytes and more that is idle while the preconditioner is built
+  d.dzl = cv.take<double>(n); d.dzu = cv.take<double>(n); d.z = cv.take<double>(n + m);
+  d.p = cv.take<double>(n + m); d.q = cv.take<double>(n + m);
+  d.sc_words = m ? (stiff_cap + 31) / 32 : 0;
+  d.sc_mask = d.sc_words <= 10 ? reinterpret_cast<unsigned*>(d.dzl) : cv.take<unsigned>(n * d.sc_words);
+  d.ratio = d.ds;
+  d.cand = reinterpret_cast<int32_t*>(d.dy);
+  d.stiff_k = cv.take<int32_t>(stiff_cap);
   d.st_beg = cv.take<int64_t>(stiff_cap); d.st_end = cv.take<int64_t>(stiff_cap);
   d.rowk = cv.take<int32_t>(nR);
-  d.sc_cnt = cv.take<int32_t>(n); d.sc_ptr = cv.take<int64_t>(n + 1);
+  d.sc_run = cv.take<int2>(n);
   d.sc_slot = cv.take<int32_t>(sc_cap); d.sc_val = cv.take<double>(sc_cap); d.sc_cap = sc_cap;
   d.G = cv.take<double>((int64_t)stiff_cap * stiff_cap); d.Ginv = cv.take<double>((int64_t)stiff_cap * stiff_cap);
   d.us = cv.take<double>(stiff_cap); d.ts = cv.take<double>(stiff_cap); d.stiff_cap = stiff_cap;
@@ -1123,7 +1129,7 @@ int ipm_create(const ipm_options* opt, ipm_handle** out) {
     delete h;
     return IPM_ERR_CUDA;
   }
-  if (prepare_tail() != cudaSuccess) {   // a per-device attribute: cheap to set again
+  if (prepare_tail() != cudaSuccess || prepare_steps() != cudaSuccess) {   // per device: cheap to set again
     cudaGetLastError();
     ipm_destroy(h);
     return IPM_ERR_CUDA;
@@ -1505,7 +1511,6 @@ static int load_qp(ipm_handle* h, const ipm_qp* qp, int64_t m_ar, void* stream) 
   if ((rc = up(d.fl, q.fl.data(), n))) return rc;
   if ((rc = up(d.fu, q.fu.data(), n))) return rc;
   CUDA_TRY(h, cudaMemsetAsync(d.hist, 0, sizeof(unsigned int) * kHistBins, h->st));
-  CUDA_TRY(h, cudaMemsetAsync(d.slotR, 0xff, sizeof(int32_t) * std::max<int64_t>(q.nR, 1), h->st));
   CUDA_TRY(h, launch_fill_rowk(d, h->st));
   CUDA_TRY(h, launch_densify_R(d, h->st));
   if (d.ucap) CUDA_TRY(h, cudaMemsetAsync(d.lrs, 0, sizeof(double) * d.ucap, h->st));
@@ -1750,7 +1755,6 @@ int ipm_share_qp(ipm_handle* h, ipm_handle* src, void* stream) {
   if (d.ucols && (rc = cp(d.uw, sd.uw, 8 * d.ucols))) return rc;
   if (d.ucols && (rc = cp(d.U, sd.U, 8 * n * d.ucols))) return rc;
   CUDA_TRY(h, cudaMemsetAsync(d.hist, 0, sizeof(unsigned int) * kHistBins, h->st));
-  CUDA_TRY(h, cudaMemsetAsync(d.slotR, 0xff, sizeof(int32_t) * std::max<int64_t>(nR, 1), h->st));
   CUDA_TRY(h, launch_fill_rowk(d, h->st));
   CUDA_TRY(h, launch_densify_R(d, h->st));
   if (d.ucap) CUDA_TRY(h, cudaMemsetAsync(d.lrs, 0, sizeof(double) * d.ucap, h->st));

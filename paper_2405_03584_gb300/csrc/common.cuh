@@ -45,6 +45,7 @@ struct Scal {
   // preconditioner
   double stiff_gamma, stiff_thresh;
   int n_stiff, stiff_max, max_stiff_seen, chol_fail;
+  int n_cand, sc_used;               // rows above gamma so far, stiff entries placed
   // FP64 refinement of a reduced-precision Newton step
   double tol2_outer, rr_outer, refine_eta;
   // primal infeasibility certificate (Farkas): with (y, z) scaled by its largest entry,

@@ -351,8 +351,6 @@ __global__ void __launch_bounds__(256, 4) k_cols_resid(Dev d, double* part, int 
       const double hx = st[buf][0][tid] + hsx + (d.ucols ? st[buf][3][tid] : 0.0);
       const double aty = st[buf][1][tid];
       const double rd = hx + cj + aty - zl + zu;
-      d.Hx[jj] = hx;
-      d.Aty[jj] = aty;
       d.rd[jj] = rd;
       keep_abs_max(cert, aty - zl + zu);
       keep_abs_max(zmax, zl);
@@ -786,11 +784,12 @@ cudaError_t launch_set_cond(cudaGraphConditionalHandle h, unsigned v, cudaStream
 //   of the moderate rows replaces it.
 // Constraint rows are walked by constraint, not by row of R: a quotient costs a warp the same
 // for one lane as for 32, and the constraint rows lie scattered among R's.  Also clears the
-// step lengths' minima.
+// step lengths' minima and the variables' stiff-row masks.
 __global__ void k_diag(Dev d) {
   const double mu = d.sc->mu;
   const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, dt = (int64_t)gridDim.x * blockDim.x;
   if (t0 < 2) d.sc->step_min[t0] = kInfBits;
+  for (int64_t i = t0; i < d.n * d.sc_words; i += dt) d.sc_mask[i] = 0u;
   for (int64_t r = t0; r < d.nR; r += dt)
     if (d.rowk[r] < 0) {
       d.omega[r] = d.wR[r];
@@ -860,16 +859,32 @@ cudaError_t launch_jacobi_full(const Dev& d, const Geo& g, double* out, cudaStre
 
 // ------------------------------------------------------------------------------ stiff rows
 
-// ratio_k = theta_k sum_j A_kj^2 / M0_j; histogram of log2(ratio / gamma) in half-octave bins;
-// the last block picks the smallest threshold bin whose cumulative count from the top stays
-// <= stiff_max.  Rows with ratio >= stiff_thresh form the low-rank correction.
+// Half-octave bin of y = ratio / gamma > 1, floor(2 log2 y), from the float64's exponent and
+// whether its mantissa reaches sqrt 2 (float64 log2 takes some forty instructions a warp).
+__device__ __forceinline__ int half_octave(double y) {
+  const long long b = __double_as_longlong(y);
+  const int e = (int)(b >> 52) - 1023;
+  const int bin = 2 * e + ((b & 0xfffffffffffffll) >= 0x6a09e667f3bcdll ? 1 : 0);
+  return bin < 0 ? 0 : (bin >= kHistBins ? kHistBins - 1 : bin);
+}
+
+// The stiff rows, in one launch: ratio_k = theta_k sum_j A_kj^2 / M0_j of every constraint row,
+// a histogram of the ratios above gamma in half-octave bins and the list of those rows; the last
+// block picks the smallest threshold bin whose count from the top stays <= stiff_max, takes the
+// listed rows at or above it, orders them by constraint and gives each its slot (thR = 0: its
+// theta leaves the Jacobi part).  Only listed rows are looked at again: a pass of one block
+// over all m took 8 us at m = 3500 and 133 us at m = 68618.
 template <int G>
-__global__ void k_stiff_ratio(Dev d) {
+__global__ void k_stiff_select(Dev d) {
   __shared__ unsigned int h[kHistBins];
+  __shared__ int list[2048];
+  __shared__ int s_cnt;
+  __shared__ double s_thr;
   __shared__ bool s_last;
+  Scal* sc = d.sc;
   for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) h[i] = 0u;
   __syncthreads();
-  const double gamma = d.sc->stiff_gamma;
+  const double gamma = sc->stiff_gamma;
   FOR_GROUP_ROWS(G, k, ok, d.m) {
     const int32_t row = ok ? d.arow[k] : 0;
     const int64_t beg = ok ? d.R_ptr[row] : 0, end = ok ? d.R_ptr[row + 1] : 0;
@@ -877,11 +892,10 @@ __global__ void k_stiff_ratio(Dev d) {
     const double acc = group_row_dot<G, true>(beg, end, glane<G>(), d.R_idx, d.R_val, d.Minv);
     if (ok && glane<G>() == 0) {
       const double ratio = d.theta[k] * acc;
-      d.ratio[k] = ratio;
       if (ratio > gamma) {
-        int bin = (int)floor(2.0 * log2(ratio / gamma));
-        bin = bin < 0 ? 0 : (bin >= kHistBins ? kHistBins - 1 : bin);
-        atomicAdd(&h[bin], 1u);
+        d.ratio[k] = ratio;
+        d.cand[atomicAdd(&sc->n_cand, 1)] = (int32_t)k;
+        atomicAdd(&h[half_octave(ratio / gamma)], 1u);
       }
     }
   }
@@ -890,157 +904,194 @@ __global__ void k_stiff_ratio(Dev d) {
     if (h[i]) atomicAdd(&d.hist[i], h[i]);
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned int t = atomicAdd(&d.sc->ticket[T_HIST], 1u);
-    s_last = (t == gridDim.x - 1);
-  }
+  if (threadIdx.x == 0) s_last = atomicAdd(&sc->ticket[T_HIST], 1u) == gridDim.x - 1;
   __syncthreads();
-  if (s_last && threadIdx.x == 0) {
-    __threadfence();
-    const int cap = d.sc->stiff_max;
-    unsigned int cum = 0;
-    int cut = kHistBins;  // no stiff rows
-    for (int b = kHistBins - 1; b >= 0; --b) {
-      unsigned int c = __ldcg(&d.hist[b]);
-      if (cum + c > (unsigned)cap) break;
-      cum += c;
-      cut = b;
+  if (!s_last) return;
+  __threadfence();
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid < 32) {
+    // lane l: bins 63 - 2l and 62 - 2l; counts from the top by a scan over the lanes
+    const unsigned c1 = __ldcg(&d.hist[63 - 2 * lane]), c0 = __ldcg(&d.hist[62 - 2 * lane]);
+    unsigned cum = c1 + c0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned t = __shfl_up_sync(0xffffffffu, cum, o);
+      if (lane >= o) cum += t;
     }
-    // rows in bins >= cut are stiff: threshold = gamma * 2^(cut/2) (bins are half octaves)
-    d.sc->stiff_thresh = cut >= kHistBins ? INFINITY : (cut == 0 ? gamma : gamma * exp2(0.5 * cut));
-    for (int b = 0; b < kHistBins; ++b) d.hist[b] = 0u;
-    d.sc->ticket[T_HIST] = 0u;
-  }
-}
-
-// Exclusive scan of per-item 0/1 (or counts) by one block in two levels: every thread scans
-// a contiguous run serially, then the block scans the run totals.  Returns the total; calls
-// emit(i, offset) for every item i in order-preserving positions.
-template <typename Val, typename Emit>
-__device__ long long block_scan_runs(int64_t count, Val val, Emit emit) {
-  __shared__ long long tsum[1024];
-  const int t = threadIdx.x, nt = blockDim.x;
-  const int64_t run = (count + nt - 1) / nt;
-  const int64_t b0 = t * run, b1 = b0 + run < count ? b0 + run : count;
-  long long acc = 0;
-  for (int64_t i = b0; i < b1; ++i) acc += val(i);
-  tsum[t] = acc;
-  __syncthreads();
-  // Hillis-Steele inclusive scan of the nt run totals
-  for (int off = 1; off < nt; off <<= 1) {
-    long long v = t >= off ? tsum[t - off] : 0;
-    __syncthreads();
-    tsum[t] += v;
-    __syncthreads();
-  }
-  long long base = t ? tsum[t - 1] : 0;
-  const long long total = tsum[nt - 1];
-  for (int64_t i = b0; i < b1; ++i) {
-    const long long v = val(i);
-    emit(i, base, v);
-    base += v;
+    const unsigned cap = (unsigned)sc->stiff_max;
+    int cut = kHistBins;                           // no stiff rows
+    if (cum - c0 <= cap) cut = 63 - 2 * lane;
+    if (cum <= cap) cut = 62 - 2 * lane;
+    cut = __reduce_min_sync(0xffffffffu, cut);
+    if (lane == 0) {
+      // rows in bins >= cut are stiff: threshold = gamma * 2^(cut/2)
+      s_thr = cut >= kHistBins ? INFINITY : (cut == 0 ? gamma : gamma * exp2(0.5 * cut));
+      s_cnt = 0;
+    }
   }
   __syncthreads();
-  return total;
-}
-
-// Ordered compaction (one block): slot of every stiff row, thR = 0 on stiff rows.
-__global__ void k_stiff_compact(Dev d) {
-  const double thr = d.sc->stiff_thresh;
-  const double gamma = d.sc->stiff_gamma;
-  const int cap = d.stiff_cap;
-  auto flag = [&](int64_t k) -> long long {
-    const double rt = d.ratio[k];
-    return (rt > gamma && rt >= thr) ? 1 : 0;
-  };
-  const long long total = block_scan_runs(d.m, flag, [&](int64_t k, long long off, long long v) {
-    const int32_t row = d.arow[k];
-    if (v && off < cap) {
-      d.stiff_k[off] = (int32_t)k;
-      d.st_beg[off] = d.R_ptr[row];
-      d.st_end[off] = d.R_ptr[row + 1];
-      d.slotR[row] = (int32_t)off;
+  const double thr = s_thr;
+  const int nc = *(volatile int*)&sc->n_cand;
+  for (int i = tid; i < nc; i += blockDim.x) {
+    const int32_t k = __ldcg(&d.cand[i]);
+    if (__ldcg(&d.ratio[k]) >= thr) {
+      const int at = atomicAdd(&s_cnt, 1);
+      if (at < 2048) list[at] = k;
+    }
+  }
+  __syncthreads();
+  const int total = min(s_cnt, 2048), ns = min(total, d.stiff_cap);
+  for (int i = tid; i < total; i += blockDim.x) {
+    const int k = list[i];
+    int rank = 0;
+    for (int q = 0; q < total; ++q) rank += list[q] < k ? 1 : 0;
+    if (rank < ns) {
+      const int32_t row = d.arow[k];
+      d.stiff_k[rank] = k;
+      d.st_beg[rank] = d.R_ptr[row];
+      d.st_end[rank] = d.R_ptr[row + 1];
       d.thR[row] = 0.0;
-    } else {
-      d.slotR[row] = -1;
     }
-  });
-  if (threadIdx.x == 0) {
-    const int ns = total < cap ? (int)total : cap;
-    d.sc->n_stiff = ns;
-    if (ns > d.sc->max_stiff_seen) d.sc->max_stiff_seen = ns;
+  }
+  for (int i = tid; i < kHistBins; i += blockDim.x) d.hist[i] = 0u;
+  if (tid == 0) {
+    sc->stiff_thresh = thr;
+    sc->n_stiff = ns;
+    sc->sc_used = 0;
+    if (ns > sc->max_stiff_seen) sc->max_stiff_seen = ns;
+    sc->n_cand = 0;
+    sc->ticket[T_HIST] = 0u;
   }
 }
 
-// Stiff entries per variable (count, then ordered fill) from the stored transpose.
-__global__ void k_sc_count(Dev d) {
+// Stiff entries per variable, built from the stiff rows alone (a pass over A^T for the counts, a
+// one-block scan and a second pass took 21 us at n = 7001 and 53 us at n = 50000): each entry
+// (slot a, variable j) sets bit a of j's mask; the masks' counts give every variable a run of
+// the list; an entry's place in its run is the number of lower bits, so a run holds its slots in
+// increasing order.  (Runs are handed out in any order; nothing depends on where a run lies.)
+__global__ void k_sc_mask(Dev d) {
+  const int ns = d.sc->n_stiff, lane = threadIdx.x & 31;
+  for (int a = gwarp(); a < ns; a += nwarps())
+    for (int64_t e = d.st_beg[a] + lane; e < d.st_end[a]; e += 32)
+      atomicOr(&d.sc_mask[(int64_t)d.R_idx[e] * d.sc_words + (a >> 5)], 1u << (a & 31));
+}
+
+__global__ void k_sc_runs(Dev d) {
   if (d.sc->n_stiff == 0) return;
-  for (int64_t j = gwarp(); j < d.n; j += nwarps()) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t j0 = (int64_t)blockIdx.x * blockDim.x; j0 < d.n; j0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t j = j0 + threadIdx.x;
     int cnt = 0;
-    for (int64_t e = d.AT_ptr[j] + (threadIdx.x & 31); e < d.AT_ptr[j + 1]; e += 32)
-      cnt += d.slotR[d.AT_idx[e]] >= 0 ? 1 : 0;
-    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    if ((threadIdx.x & 31) == 0) d.sc_cnt[j] = cnt;
-  }
-}
-
-// Exclusive scan of sc_cnt into sc_ptr (one block, two levels).
-__global__ void k_sc_scan(Dev d) {
-  if (d.sc->n_stiff == 0) return;
-  const long long total = block_scan_runs(d.n, [&](int64_t j) -> long long { return d.sc_cnt[j]; },
-                                          [&](int64_t j, long long off, long long) { d.sc_ptr[j] = off; });
-  if (threadIdx.x == 0) {
-    d.sc_ptr[d.n] = total;
-    if (total > d.sc_cap) d.sc->n_stiff = 0;   // does not fit: fall back to plain Jacobi
+    if (j < d.n)
+      for (int w = 0; w < d.sc_words; ++w) cnt += __popc(d.sc_mask[j * d.sc_words + w]);
+    int cum = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, cum, o);
+      if (lane >= o) cum += t;
+    }
+    int base = 0;
+    if (lane == 31 && cum) base = atomicAdd(&d.sc->sc_used, cum);
+    base = __shfl_sync(0xffffffffu, base, 31) + cum - cnt;
+    if (j < d.n) d.sc_run[j] = make_int2(base, base + cnt <= d.sc_cap ? cnt : 0);
   }
 }
 
 __global__ void k_sc_fill(Dev d) {
-  if (d.sc->n_stiff == 0) return;
-  const int lane = threadIdx.x & 31;
-  for (int64_t j = gwarp(); j < d.n; j += nwarps()) {
-    int64_t out = d.sc_ptr[j];
-    for (int64_t e0 = d.AT_ptr[j]; e0 < d.AT_ptr[j + 1]; e0 += 32) {
-      const int64_t e = e0 + lane;
-      int slot = -1;
-      if (e < d.AT_ptr[j + 1]) slot = d.slotR[d.AT_idx[e]];
-      const unsigned bal = __ballot_sync(0xffffffffu, slot >= 0);
-      if (slot >= 0) {
-        const int64_t pos = out + __popc(bal & ((1u << lane) - 1u));
-        d.sc_slot[pos] = slot;
-        d.sc_val[pos] = d.AT_val[e];
+  const int ns = d.sc->n_stiff, lane = threadIdx.x & 31;
+  for (int a = gwarp(); a < ns; a += nwarps())
+    for (int64_t e = d.st_beg[a] + lane; e < d.st_end[a]; e += 32) {
+      const int64_t j = d.R_idx[e];
+      const unsigned* m = d.sc_mask + j * d.sc_words;
+      const int2 run = d.sc_run[j];
+      int at = __popc(m[a >> 5] & ((1u << (a & 31)) - 1u));
+      for (int w = 0; w < (a >> 5); ++w) at += __popc(m[w]);
+      if (at < run.y) {
+        d.sc_slot[run.x + at] = a;
+        d.sc_val[run.x + at] = d.R_val[e];
       }
-      out += __popc(bal);
     }
-  }
 }
 
 // G = Theta_s^{-1} + A_s M^{-1} A_s^T (dense, n_stiff x n_stiff, leading dimension stiff_cap).
-// One block per stiff row a accumulates row a in shared memory: for every entry (j, R_aj) of
-// the row, add R_aj / M_j * (column j's stiff entries).  Entries of a column list are distinct
-// slots, so lanes never collide; the j order is fixed, hence deterministic.
-__global__ void k_gram_G(Dev d) {
-  extern __shared__ double grow[];
-  const int ns = d.sc->n_stiff;
-  const int cap = d.stiff_cap;
-  for (int a = blockIdx.x; a < ns; a += gridDim.x) {
-    for (int i = threadIdx.x; i < ns; i += blockDim.x) grow[i] = 0.0;
-    __syncthreads();
-    const int32_t k = d.stiff_k[a];
-    const int32_t row = d.arow[k];
-    for (int64_t e = d.R_ptr[row]; e < d.R_ptr[row + 1]; ++e) {
-      const int32_t j = d.R_idx[e];
-      const double f = d.R_val[e] * d.Minv[j];
-      const int64_t b0 = d.sc_ptr[j], b1 = d.sc_ptr[j + 1];
-      for (int64_t t = b0 + threadIdx.x; t < b1; t += blockDim.x) grow[d.sc_slot[t]] += f * d.sc_val[t];
-      __syncthreads();
+// One block per stiff row a, one thread per slot b: for every entry (j, R_aj) of the row in
+// order, thread b adds (R_aj / M_j) A_bj if bit b of j's mask is set.  The row's entries, masks
+// and the variables' runs are staged in shared memory 256 entries at a time, so what remains is
+// each slot's chain of additions.  (With a barrier per entry: 27 us at n = 7001, 42 entries a
+// row; 87 us at n = 50000, 250 a row.)
+constexpr int kGramEntries = 256, kGramItems = 2048, kGramSlots = 4;   // 4 * 256 slots = stiff_max's limit
+__global__ void __launch_bounds__(256) k_gram_G(Dev d) {
+  extern __shared__ unsigned gm[];               // masks [word][entry], then ranks before a word [word][entry]
+  __shared__ double f[kGramEntries], lv[kGramItems];
+  __shared__ int base[kGramEntries], off[kGramEntries + 1], wsum[8];
+  const int ns = d.sc->n_stiff, a = blockIdx.x;
+  if (a >= ns) return;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int words = (ns + 31) >> 5;
+  unsigned short* pre = reinterpret_cast<unsigned short*>(gm + (size_t)words * kGramEntries);
+  double acc[kGramSlots] = {0.0, 0.0, 0.0, 0.0};
+  const int64_t beg = d.st_beg[a], end = d.st_end[a];
+  for (int64_t e0 = beg; e0 < end; e0 += kGramEntries) {
+    const int ne = (int)(end - e0 < kGramEntries ? end - e0 : kGramEntries);
+    int cnt = 0;
+    if (tid < ne) {
+      const int64_t j = d.R_idx[e0 + tid];
+      f[tid] = d.R_val[e0 + tid] * d.Minv[j];
+      const int2 run = d.sc_run[j];
+      base[tid] = run.x;
+      cnt = run.y;
+      int p = 0;
+      for (int q = 0; q < words; ++q) {
+        const unsigned m = cnt ? d.sc_mask[j * d.sc_words + q] : 0u;
+        gm[q * kGramEntries + tid] = m;
+        pre[q * kGramEntries + tid] = (unsigned short)p;
+        p += __popc(m);
+      }
     }
-    for (int i = threadIdx.x; i < ns; i += blockDim.x) {
-      double v = grow[i];
-      if (i == a) v += 1.0 / d.theta[k];
-      d.G[(int64_t)a * cap + i] = v;
+    int cum = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, cum, o);
+      if (lane >= o) cum += t;
+    }
+    if (lane == 31) wsum[w] = cum;
+    __syncthreads();
+    int before = 0;
+    for (int q = 0; q < w; ++q) before += wsum[q];
+    off[tid] = before + cum - cnt;
+    if (tid == 255) off[256] = before + cum;
+    __syncthreads();
+    const int items = off[kGramEntries];
+    const bool staged = items <= kGramItems;
+    if (staged)
+      for (int i = tid; i < items; i += 256) {
+        int lo = 0, hi = kGramEntries;             // the last entry whose run starts at or before i
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          if (off[mid] <= i) lo = mid;
+          else hi = mid;
+        }
+        lv[i] = d.sc_val[base[lo] + i - off[lo]];
+      }
+    __syncthreads();
+#pragma unroll
+    for (int g = 0; g < kGramSlots; ++g) {
+      const int q = w + 8 * g;                     // the mask word of this warp's slots
+      if (q < words)
+        for (int e = 0; e < ne; ++e) {
+          const unsigned m = gm[q * kGramEntries + e];
+          if (m >> lane & 1u) {
+            const int at = pre[q * kGramEntries + e] + __popc(m & ((1u << lane) - 1u));
+            acc[g] = fma(f[e], staged ? lv[off[e] + at] : d.sc_val[base[e] + at], acc[g]);
+          }
+        }
     }
     __syncthreads();
+  }
+#pragma unroll
+  for (int g = 0; g < kGramSlots; ++g) {
+    const int b = tid + 256 * g;
+    if (b < ns) d.G[(int64_t)a * d.stiff_cap + b] = b == a ? acc[g] + 1.0 / d.theta[d.stiff_k[a]] : acc[g];
   }
 }
 
@@ -1362,7 +1413,8 @@ __global__ void k_stiff_corr(Dev d, int init) {
     double zj = d.z[j];
     if (ns > 0) {
       double acc = 0.0;
-      for (int64_t t = d.sc_ptr[j]; t < d.sc_ptr[j + 1]; ++t) acc = fma(d.sc_val[t], d.ts[d.sc_slot[t]], acc);
+      const int2 run = d.sc_run[j];
+      for (int t = run.x; t < run.x + run.y; ++t) acc = fma(d.sc_val[t], d.ts[d.sc_slot[t]], acc);
       zj -= d.Minv[j] * acc;
       d.z[j] = zj;
     }
@@ -1818,12 +1870,14 @@ cudaError_t launch_update(const Dev& d, const Geo& g, cudaStream_t st) {
 cudaError_t launch_dense_build(const Dev& d, cudaStream_t st);       // dense.cu
 cudaError_t launch_stiff_factor(const Dev& d, cudaStream_t st);      // dense.cu
 
+cudaError_t prepare_steps() {
+  return cudaFuncSetAttribute(k_gram_G, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              kGramSlots * 8 * kGramEntries * 6);
+}
+
 // Before the right-hand side: stiff-row selection (JACOBI_LR).
 cudaError_t launch_precond_build(const Dev& d, const Geo& g, int precond, cudaStream_t st) {
-  if (precond == PC_JACOBI_LR && d.m) {
-    DISPATCH_G(d.g_rows, k_stiff_ratio<G><<<g.gM, kBlock, 0, st>>>(d));
-    k_stiff_compact<<<1, 1024, 0, st>>>(d);
-  }
+  if (precond == PC_JACOBI_LR && d.m) DISPATCH_G(d.g_rows, k_stiff_select<G><<<g.gM, kBlock, 0, st>>>(d));
   return cudaGetLastError();
 }
 
@@ -1833,11 +1887,11 @@ cudaError_t launch_precond_finish(const Dev& d, const Geo& g, int precond, cudaS
   if (precond == PC_DENSE) return launch_dense_build(d, st);
   if (precond == PC_BLOCK32) return launch_block_factor(d, st);
   if (precond == PC_JACOBI_LR && d.m) {
-    k_sc_count<<<g.gN, kBlock, 0, st>>>(d);
-    k_sc_scan<<<1, 1024, 0, st>>>(d);
-    k_sc_fill<<<g.gN, kBlock, 0, st>>>(d);
-    const size_t smem = sizeof(double) * (size_t)d.stiff_cap;
-    k_gram_G<<<d.stiff_cap, 256, smem, st>>>(d);
+    const int nb = (d.stiff_cap + 7) / 8;
+    k_sc_mask<<<nb, kBlock, 0, st>>>(d);
+    k_sc_runs<<<g.eN, kBlock, 0, st>>>(d);
+    k_sc_fill<<<nb, kBlock, 0, st>>>(d);
+    k_gram_G<<<d.stiff_cap, 256, (size_t)d.sc_words * kGramEntries * 6, st>>>(d);
     cudaError_t e = launch_stiff_factor(d, st);
     if (e != cudaSuccess) return e;
   }

@@ -369,8 +369,10 @@ __global__ void __launch_bounds__(256, 6) k_op_cols_lp(Dev d, int standalone) {
     if (ok && gl == 0) {
       const double pj = d.p[j];
       double st = 0.0;
-      if (stiff)
-        for (int64_t t = d.sc_ptr[j]; t < d.sc_ptr[j + 1]; ++t) st = fma(d.sc_val[t], d.us2[d.sc_slot[t]], st);
+      if (stiff) {
+        const int2 run = d.sc_run[j];
+        for (int t = run.x; t < run.x + run.y; ++t) st = fma(d.sc_val[t], d.us2[d.sc_slot[t]], st);
+      }
       const double qj = (double)acc + hs + st + (d.h0[j] + d.sigma[j]) * pj;
       d.q[j] = qj;
       pq = fma(pj, qj, pq);

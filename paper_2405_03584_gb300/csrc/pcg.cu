@@ -230,8 +230,9 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_pcg_tail(Dev d, int npart, 
     for (int e = 0; e < E; ++e) {
       const int j = j0 + tid + e * kTailThreads;
       const bool in = act && j < j1;
-      cb[e] = in ? (int)d.sc_ptr[j] : 0;
-      cn[e] = in ? (int)d.sc_ptr[j + 1] - cb[e] : 0;
+      const int2 run = in ? d.sc_run[j] : make_int2(0, 0);
+      cb[e] = run.x;
+      cn[e] = run.y;
     }
   };
   auto fetch_first = [&]() {

@@ -44,19 +44,21 @@ struct Dev {
   double *x, *s, *y, *zl, *zu;
   // per IPM iteration
   double *theta, *sigma, *omega, *M0, *Minv, *thR;  // thR: theta placed on R rows (Jacobi part)
-  double *rd, *rp, *Hx, *Aty;
+  double *rd, *rp;
   double *tR, *vR, *vR2;       // nR work vectors
   // PCG and direction
   double *dx, *r, *z, *p, *q, *rhs;
   double *ds, *dy, *dzl, *dzu;
   // stiff-row low-rank correction
-  double* ratio;               // m
-  int32_t* slotR;              // nR: slot of a stiff row, -1 otherwise
+  double* ratio;               // m (shares ds)
   int32_t* rowk;               // nR: constraint index of a row of R, -1 for the factor's rows
   int32_t* stiff_k;            // stiff_cap: constraint index of each slot
   int64_t *st_beg, *st_end;    // stiff_cap: entries of each slot's row of R
-  int32_t* sc_cnt;             // n
-  int64_t* sc_ptr;             // n+1: stiff entries per variable (CSC of the stiff rows)
+  int32_t* cand;               // m (shares dy): constraint rows above gamma
+  unsigned* sc_mask;           // n x sc_words: the stiff rows of each variable, one bit a slot (shares
+                               // dzl, dzu, z, p, q where these are large enough: it is dead by then)
+  int sc_words;
+  int2* sc_run;                // n: first of a variable's stiff entries in sc_slot, sc_val, and their number
   int32_t* sc_slot; double* sc_val;  // sc_cap
   int64_t sc_cap;
   double *G, *Ginv, *us, *ts;  // stiff_cap^2, stiff_cap^2, stiff_cap, stiff_cap
@@ -260,7 +262,8 @@ cudaError_t launch_cg_body(const Dev& d, const Geo& g, int precond, cudaGraphCon
                            bool in_graph = true, bool lowp = false);
 // ---- the vector half of a PCG iteration as one cluster kernel (pcg.cu) ----
 bool tail_runs(const Dev& d, int precond);   // the cluster kernel covers this system
-cudaError_t prepare_tail();                  // once per process and device
+cudaError_t prepare_tail();                  // kernel attributes, per device
+cudaError_t prepare_steps();                 // the same for kernels.cu
 cudaError_t launch_tail_init(const Dev& d, int precond, cudaGraphConditionalHandle h, cudaStream_t st);
 cudaError_t launch_tail_iter(const Dev& d, int precond, int npart, cudaGraphConditionalHandle h, bool in_graph,
                              cudaStream_t st);
