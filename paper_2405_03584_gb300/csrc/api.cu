@@ -35,7 +35,7 @@ namespace {
 struct LoopCounts {
   int top = 0;       // outside every loop
   int ipm = 0;       // IPM-loop body, outside nested loops
-  int pcg = 0;       // one PCG trip
+  int pcg = 0;       // one PCG trip (pcg_per_trip iterations)
   int refine = 0;    // refinement body, outside its PCG loop
   int fallback = 0;  // one trip of the FP64 fallback loop
   int ru = 0;        // reduced precision with residual replacement: one PCG loop per step
@@ -790,6 +790,23 @@ double refine_factor(const ipm_handle* h) {
   return refine_replaces(h) ? 0.01 : 0.1;
 }
 
+// PCG iterations captured in one trip of the while node.  A trip of the node itself costs 3.5 us
+// on GB300 and a launch that finds the PCG done about 1, so two iterations a trip pay where a step
+// takes several: float64 storage with a Jacobi preconditioner (solves at n = 1500 / 7001: 6.39 /
+// 10.79 ms at one, 6.19 / 10.51 at two, 6.12 / 10.48 at three).  The dense preconditioner's PCG
+// ends after one (one step at n = 24: 216 us at one, 223 at two), and the reduced storages'
+// iteration has twice the launches (FP32 batch of eight: 31.4 ms at one, 32.2 at two).
+int pcg_per_trip(const Dev& d, int pc) {
+  return d.storage == ST_F64 && (pc == PC_JACOBI || pc == PC_JACOBI_LR) ? 2 : 1;
+}
+
+template <typename Body>
+cudaError_t pcg_trip(int count, Body body) {
+  cudaError_t e = cudaSuccess;
+  for (int k = 0; k < count && e == cudaSuccess; ++k) e = body();
+  return e;
+}
+
 // Emits (into the capture running on `st`) one Newton step -- diagonal update, preconditioner,
 // right-hand side, PCG (nested while loops; with a reduced-precision store the PCG loop sits in
 // an FP64 refinement loop followed by an FP64 fallback loop) and direction recovery -- and,
@@ -814,7 +831,7 @@ cudaError_t emit_step(ipm_handle* h, int pc, bool full, cudaStream_t st, cudaStr
     chk(launch_cg_init(d, g, pc, st, hp));
     if (e == cudaSuccess)
       chk(add_while(st, s2, [&](cudaGraphConditionalHandle ch, cudaStream_t bs) {
-            return launch_cg_body(d, g, pc, ch, bs, true, false);
+            return pcg_trip(pcg_per_trip(d, pc), [&] { return launch_cg_body(d, g, pc, ch, bs, true, false); });
           }, &c->pcg, &hp));
   } else if (refine_replaces(h)) {
     // one reduced-precision PCG with residual replacement, then the FP64 fallback
@@ -937,7 +954,7 @@ int run_iteration_direct(ipm_handle* h, int pc, int64_t* launches) {
       CUDA_TRY(h, cudaMemcpyAsync(&h->hs->cg_done, &d.sc->cg_done, sizeof(int), cudaMemcpyDeviceToHost, st));
       CUDA_TRY(h, cudaStreamSynchronize(st));
       done = h->hs->cg_done;
-      *launches += lowp ? lc.pcg : lc.pcg;
+      *launches += lc.pcg / pcg_per_trip(d, pc);
     }
     return IPM_OK;
   };
@@ -958,7 +975,7 @@ int run_iteration_direct(ipm_handle* h, int pc, int64_t* launches) {
       CUDA_TRY(h, cudaMemcpyAsync(&h->hs->cg_done, &d.sc->cg_done, sizeof(int), cudaMemcpyDeviceToHost, st));
       CUDA_TRY(h, cudaStreamSynchronize(st));
       done = h->hs->cg_done;
-      *launches += lc.pcg;
+      *launches += lc.pcg / pcg_per_trip(d, pc);
     }
     CUDA_TRY(h, launch_ru_end(d, g, st));
     CUDA_TRY(h, launch_refine_fallback(d, g, st));
@@ -1859,13 +1876,15 @@ static int fill_info(ipm_handle* h, int64_t direct_launches) {
     for (int r = 0; r < rows; ++r) {
       const double* t = h->htrace + (size_t)r * kTraceCols;
       const int64_t cg = (int64_t)t[8], ref = (int64_t)t[13];
-      launches += lc.ipm + 1;  // + the loop re-arm kernel counted in ipm
+      const int per = pcg_per_trip(h->d, pc);
+      const int64_t trips = std::max<int64_t>(1, (cg + per - 1) / per);
+      launches += lc.ipm;
       if (!lowp) {
-        launches += std::max<int64_t>(1, cg) * lc.pcg;
+        launches += trips * lc.pcg;
       } else if (lc.ru) {
-        launches += std::max<int64_t>(1, cg) * lc.pcg + lc.fallback;
+        launches += trips * lc.pcg + lc.fallback;
       } else {
-        launches += (cg + ref) * lc.pcg + ref * lc.refine + lc.fallback;
+        launches += (trips + ref) * lc.pcg + ref * lc.refine + lc.fallback;
       }
     }
   }
