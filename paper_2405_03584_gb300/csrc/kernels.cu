@@ -75,52 +75,79 @@ Geo make_geo(const Dev& d) {
 // reduction over the n rows of U split into row chunks, one partial vector per block, summed
 // in block order), then (U (W t))_j inside the column kernels (lr_row).  Row-major U makes
 // both passes read rows of U contiguously.
+//
+// A thread owns 8 neighbouring columns (64 bytes of a row, in 16-byte loads where rows start on
+// 16 bytes) and walks every rg-th row of its block's chunk, rg = 256 / ceil(ucols / 8) rows of
+// threads side by side: of 256 threads 250 carry columns at 200 columns, where 32 lanes over
+// 128-column slices carried 200 of 256 values, and every float64 instruction of a warp costs the
+// same.  (n = 77373, 200 columns: 41 us before.)
+constexpr int kLrCols = 8;
+constexpr int kLrSlice = 256 * kLrCols;          // columns a block covers at a time
+template <bool VEC>
 __global__ void __launch_bounds__(256) k_lr_part(Dev d, const double* __restrict__ v) {
-  // 8 warps per block; warp w takes rows j0 + w, j0 + w + 8, ... of the block's chunk; lane l
-  // accumulates columns r0 + l + 32 c (c < 4) of a 128-column slice; the warps' sums are
-  // added in warp order through shared memory.
-  constexpr int RC = 4;
-  __shared__ double sh[8][32 * RC];
+  __shared__ double sh[256][kLrCols + 1];
   const int64_t uc = d.ucols, n = d.n;
   const int64_t per = (n + gridDim.x - 1) / gridDim.x;
   const int64_t j0 = (int64_t)blockIdx.x * per, j1 = j0 + per < n ? j0 + per : n;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int64_t r0 = 0; r0 < uc; r0 += 32 * RC) {
-    double acc[RC];
+  const int tid = threadIdx.x;
+  for (int64_t r0 = 0; r0 < uc; r0 += kLrSlice) {
+    const int w = (int)(uc - r0 < kLrSlice ? uc - r0 : kLrSlice);
+    const int nch = (w + kLrCols - 1) / kLrCols, rg = 256 / nch;
+    const int c = tid % nch, g = tid / nch;
+    const int cols = w - c * kLrCols < kLrCols ? w - c * kLrCols : kLrCols;
+    double acc[kLrCols];
 #pragma unroll
-    for (int c = 0; c < RC; ++c) acc[c] = 0.0;
-    int64_t j = j0 + w;
-    for (; j + 8 < j1; j += 16) {
-      const double* u0 = d.U + j * uc + r0 + lane;
-      const double* u1 = u0 + 8 * uc;
-      const double x0 = __ldg(v + j), x1 = __ldg(v + j + 8);
-      double t0[RC], t1[RC];
+    for (int k = 0; k < kLrCols; ++k) acc[k] = 0.0;
+    if (g < rg) {
+      const double* u = d.U + r0 + c * kLrCols;
+      if (VEC && cols == kLrCols) {
+        int64_t j = j0 + g;
+        for (; j + rg < j1; j += 2 * rg) {
+          const double2* p0 = reinterpret_cast<const double2*>(u + j * uc);
+          const double2* p1 = reinterpret_cast<const double2*>(u + (j + rg) * uc);
+          double2 a[kLrCols / 2], b[kLrCols / 2];
+          const double x0 = __ldg(v + j), x1 = __ldg(v + j + rg);
 #pragma unroll
-      for (int c = 0; c < RC; ++c) {
-        const bool in = r0 + lane + 32 * c < uc;
-        t0[c] = in ? __ldg(u0 + 32 * c) : 0.0;
-        t1[c] = in ? __ldg(u1 + 32 * c) : 0.0;
+          for (int k = 0; k < kLrCols / 2; ++k) a[k] = __ldg(p0 + k);
+#pragma unroll
+          for (int k = 0; k < kLrCols / 2; ++k) b[k] = __ldg(p1 + k);
+#pragma unroll
+          for (int k = 0; k < kLrCols / 2; ++k) {
+            acc[2 * k] = fma(a[k].x, x0, acc[2 * k]);
+            acc[2 * k + 1] = fma(a[k].y, x0, acc[2 * k + 1]);
+          }
+#pragma unroll
+          for (int k = 0; k < kLrCols / 2; ++k) {
+            acc[2 * k] = fma(b[k].x, x1, acc[2 * k]);
+            acc[2 * k + 1] = fma(b[k].y, x1, acc[2 * k + 1]);
+          }
+        }
+        if (j < j1) {
+          const double2* p0 = reinterpret_cast<const double2*>(u + j * uc);
+          const double x0 = __ldg(v + j);
+#pragma unroll
+          for (int k = 0; k < kLrCols / 2; ++k) {
+            const double2 a = __ldg(p0 + k);
+            acc[2 * k] = fma(a.x, x0, acc[2 * k]);
+            acc[2 * k + 1] = fma(a.y, x0, acc[2 * k + 1]);
+          }
+        }
+      } else {
+        for (int64_t j = j0 + g; j < j1; j += rg) {
+          const double x0 = __ldg(v + j);
+#pragma unroll
+          for (int k = 0; k < kLrCols; ++k)
+            if (k < cols) acc[k] = fma(__ldg(u + j * uc + k), x0, acc[k]);
+        }
       }
-#pragma unroll
-      for (int c = 0; c < RC; ++c) acc[c] = fma(t1[c], x1, fma(t0[c], x0, acc[c]));
-    }
-    if (j < j1) {
-      const double* u0 = d.U + j * uc + r0 + lane;
-      const double x0 = __ldg(v + j);
-#pragma unroll
-      for (int c = 0; c < RC; ++c)
-        if (r0 + lane + 32 * c < uc) acc[c] = fma(__ldg(u0 + 32 * c), x0, acc[c]);
     }
 #pragma unroll
-    for (int c = 0; c < RC; ++c) sh[w][lane + 32 * c] = acc[c];
+    for (int k = 0; k < kLrCols; ++k) sh[tid][k] = acc[k];
     __syncthreads();
-    for (int t = threadIdx.x; t < 32 * RC; t += blockDim.x) {
-      if (r0 + t < uc) {
-        double s = 0.0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) s += sh[q][t];
-        d.upart[(r0 + t) * (int64_t)d.ublocks + blockIdx.x] = s;   // column-major: the final sum reads runs
-      }
+    for (int t = tid; t < w; t += 256) {
+      double s = 0.0;
+      for (int q = 0; q < rg; ++q) s += sh[q * nch + t / kLrCols][t % kLrCols];
+      d.upart[(r0 + t) * (int64_t)d.ublocks + blockIdx.x] = s;   // column-major: the final sum reads runs
     }
     __syncthreads();
   }
@@ -146,7 +173,8 @@ __global__ void k_lr_final(Dev d, int quad) {
 
 cudaError_t launch_lr(const Dev& d, const double* v, int quad, cudaStream_t st) {
   if (!d.ucols) return cudaSuccess;
-  k_lr_part<<<d.ublocks, 256, 0, st>>>(d, v);
+  if (d.ucols & 1) k_lr_part<false><<<d.ublocks, 256, 0, st>>>(d, v);
+  else k_lr_part<true><<<d.ublocks, 256, 0, st>>>(d, v);
   k_lr_final<<<(int)std::min<int64_t>((d.ucols + 7) / 8, 4096), 256, 0, st>>>(d, quad);
   return cudaGetLastError();
 }

@@ -128,20 +128,43 @@ struct Dev {
 };
 
 // (U lrs)_j by a group of G lanes over the contiguous row j of U (all lanes of the group get it).
+// An even column count makes every row start on 16 bytes: two columns a load then, of U and of
+// the weights alike (the loads' issue slots, not their bytes, held this pass at twice the
+// float64 pipe's time).
 template <int G>
 __device__ __forceinline__ double lr_row(const Dev& d, const int64_t j, const bool ok, const int gl) {
   double a = 0.0;
   if (ok) {
     const double* row = d.U + j * d.ucols;
     double a1 = 0.0, a2 = 0.0, a3 = 0.0;
-    int64_t r = gl;
-    for (; r + 3 * G < d.ucols; r += 4 * G) {
-      a = fma(__ldg(row + r), __ldg(d.lrs + r), a);
-      a1 = fma(__ldg(row + r + G), __ldg(d.lrs + r + G), a1);
-      a2 = fma(__ldg(row + r + 2 * G), __ldg(d.lrs + r + 2 * G), a2);
-      a3 = fma(__ldg(row + r + 3 * G), __ldg(d.lrs + r + 3 * G), a3);
+    if ((d.ucols & 1) == 0) {
+      const double2* r2 = reinterpret_cast<const double2*>(row);
+      const double2* s2 = reinterpret_cast<const double2*>(d.lrs);
+      const int nv = (int)(d.ucols >> 1);
+      int v = gl;
+      for (; v + G < nv; v += 2 * G) {
+        const double2 u0 = __ldg(r2 + v), u1 = __ldg(r2 + v + G);
+        const double2 s0 = __ldg(s2 + v), s1 = __ldg(s2 + v + G);
+        a = fma(u0.x, s0.x, a);
+        a1 = fma(u0.y, s0.y, a1);
+        a2 = fma(u1.x, s1.x, a2);
+        a3 = fma(u1.y, s1.y, a3);
+      }
+      if (v < nv) {
+        const double2 u0 = __ldg(r2 + v), s0 = __ldg(s2 + v);
+        a = fma(u0.x, s0.x, a);
+        a1 = fma(u0.y, s0.y, a1);
+      }
+    } else {
+      int64_t r = gl;
+      for (; r + 3 * G < d.ucols; r += 4 * G) {
+        a = fma(__ldg(row + r), __ldg(d.lrs + r), a);
+        a1 = fma(__ldg(row + r + G), __ldg(d.lrs + r + G), a1);
+        a2 = fma(__ldg(row + r + 2 * G), __ldg(d.lrs + r + 2 * G), a2);
+        a3 = fma(__ldg(row + r + 3 * G), __ldg(d.lrs + r + 3 * G), a3);
+      }
+      for (; r < d.ucols; r += G) a = fma(__ldg(row + r), __ldg(d.lrs + r), a);
     }
-    for (; r < d.ucols; r += G) a = fma(__ldg(row + r), __ldg(d.lrs + r), a);
     a = (a + a1) + (a2 + a3);
   }
 #pragma unroll
