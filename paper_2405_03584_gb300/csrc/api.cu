@@ -117,6 +117,7 @@ struct ipm_handle {
   std::vector<int32_t> row_of;
   std::vector<double> trace;        // IPM_TRACE_COLS doubles per IPM iteration of the last solve
   double* htrace = nullptr;         // pinned: trace rows copied back after a solve
+  char* stage = nullptr;            // pinned (htrace's allocation): vectors on their way to or from host memory
   int trace_cap = 0;
   int pending = 0;                  // an asynchronous solve was launched and not yet waited for
   // Bumped whenever the buffers or kernel parameters that a captured solve graph holds change
@@ -186,6 +187,7 @@ void free_arena(ipm_handle* h) {
   destroy_graphs(h);
   if (h->htrace) cudaFreeHost(h->htrace);
   h->htrace = nullptr;
+  h->stage = nullptr;
   h->trace_cap = 0;
   if (h->arena) cudaFree(h->arena);
   h->arena = nullptr;
@@ -261,11 +263,13 @@ void carve_state(Carver& cv, Dev& d, int64_t n, int64_t m, int64_t nR, int stiff
   d.zl = cv.take<double>(n); d.zu = cv.take<double>(n);
   d.theta = cv.take<double>(m); d.sigma = cv.take<double>(n); d.omega = cv.take<double>(nR);
   d.M0 = cv.take<double>(n); d.Minv = cv.take<double>(n + m); d.thR = cv.take<double>(nR);
-  d.rd = cv.take<double>(n); d.rp = cv.take<double>(m);
   d.tR = cv.take<double>(nR); d.vR = cv.take<double>(nR); d.vR2 = cv.take<double>(nR);
   // PCG vectors hold n + m entries: the doubly augmented system appends the multipliers
-  d.dx = cv.take<double>(n + m); d.r = cv.take<double>(n + m); d.rhs = cv.take<double>(n + m);
-  d.ds = cv.take<double>(m); d.dy = cv.take<double>(m);
+  d.r = cv.take<double>(n + m); d.rhs = cv.take<double>(n + m);
+  // what the step-level calls return, side by side: one copy brings back a call's results
+  // (x .. zu above likewise)
+  d.rd = cv.take<double>(n); d.rp = cv.take<double>(m); d.sc = cv.take<Scal>(1);
+  d.dx = cv.take<double>(n + m); d.ds = cv.take<double>(m); d.dy = cv.take<double>(m);
   // one stretch of 40 n bytes and more that is idle while the preconditioner is built
   d.dzl = cv.take<double>(n); d.dzu = cv.take<double>(n); d.z = cv.take<double>(n + m);
   d.p = cv.take<double>(n + m); d.q = cv.take<double>(n + m);
@@ -331,7 +335,6 @@ void carve_state(Carver& cv, Dev& d, int64_t n, int64_t m, int64_t nR, int stiff
   }
   d.trace = cv.take<double>((int64_t)trace_cap * kTraceCols);
   d.partials = cv.take<double>(32 * (int64_t)kMaxRedBlocks);
-  d.sc = cv.take<Scal>(1);
 }
 
 // Stiff-row capacity of a handle and the matching capacity of the stiff CSC lists.
@@ -352,14 +355,20 @@ int dev_alloc(ipm_handle* h, void** p, size_t bytes, const char* what) {
   return IPM_OK;
 }
 
-// Pinned trace buffer for the rows copied back after each solve.
+// Pinned buffers: the trace rows copied back after each solve, and a stage that holds the largest
+// stretch of results a call copies out at once (rd .. dzu).
 int alloc_trace(ipm_handle* h) {
   h->trace_cap = h->opt.max_ipm;
-  if (cudaMallocHost(&h->htrace, sizeof(double) * kTraceCols * (size_t)h->trace_cap) != cudaSuccess) {
+  const size_t tb = sizeof(double) * kTraceCols * (size_t)h->trace_cap;
+  const Dev& d = h->d;
+  const size_t step = (size_t)((const char*)(d.dzu + d.n) - (const char*)d.rd);
+  const size_t iter = (size_t)((const char*)(d.zu + d.n) - (const char*)d.x);
+  if (cudaMallocHost(&h->htrace, tb + std::max(step, iter)) != cudaSuccess) {
     cudaGetLastError();
     h->htrace = nullptr;
     return fail(h, IPM_ERR_OOM, "pinned trace buffer");
   }
+  h->stage = (char*)h->htrace + tb;
   return IPM_OK;
 }
 
@@ -935,7 +944,8 @@ int ensure_dir_graph(ipm_handle* h, int pc) {
   if (gr.dir) return IPM_OK;
   gr.dir_c = LoopCounts{};
   CUDA_TRY(h, cudaStreamBeginCapture(h->st, cudaStreamCaptureModeThreadLocal));
-  cudaError_t e = emit_step(h, pc, false, h->st, h->st2, h->st3, 0, &gr.dir_c);
+  cudaError_t e = launch_residual_summary(h->d, h->g, h->st, RSM_STEP);
+  if (e == cudaSuccess) e = emit_step(h, pc, false, h->st, h->st2, h->st3, 0, &gr.dir_c);
   return finish_capture(h, e, h->st, &gr.dir, nullptr, &gr.dir_c.top);
 }
 
@@ -1035,6 +1045,7 @@ int push_options(ipm_handle* h) {
   s.cnorm = h->cnorm;
   s.bnorm = h->bnorm;
   s.ncomp = h->ncomp;
+  s.trace_cap = h->trace_cap;
   return IPM_OK;
 }
 
@@ -1050,6 +1061,35 @@ int copy_in(ipm_handle* h, double* dst, const double* src, int64_t n, int mem) {
   if (!src) return fail(h, IPM_ERR_ARG, "missing vector");
   CUDA_TRY(h, cudaMemcpyAsync(dst, src, sizeof(double) * (size_t)n,
                               mem == IPM_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->st));
+  return IPM_OK;
+}
+
+// Results for host memory go through the pinned stage: one copy of a stretch of the arena, one
+// synchronisation, then plain copies to the caller's arrays.  (A copy into pageable memory is
+// staged by the runtime, one at a time and synchronously: five of them and two of the scalars were
+// 100 us of a Newton step at n = 24.)
+struct Staged {
+  const char* begin;
+  char* at;
+};
+int stage_out(ipm_handle* h, const void* begin, const void* end, size_t offset, Staged* s) {
+  s->begin = (const char*)begin;
+  s->at = h->stage + offset;
+  CUDA_TRY(h, cudaMemcpyAsync(s->at, begin, (size_t)((const char*)end - (const char*)begin), cudaMemcpyDeviceToHost, h->st));
+  return IPM_OK;
+}
+void unstage(const Staged& s, double* dst, const double* src, int64_t n) {
+  if (dst && n > 0) std::memcpy(dst, s.at + ((const char*)src - s.begin), sizeof(double) * (size_t)n);
+}
+
+// One vector to the caller; host memory: done on return.
+int copy_vector_out(ipm_handle* h, double* dst, const double* src, int64_t n, int mem) {
+  if (mem != IPM_MEM_HOST) return copy_out(h, dst, src, n, mem);
+  Staged t;
+  int rc;
+  if ((rc = stage_out(h, src, src + n, 0, &t))) return rc;
+  CUDA_TRY(h, cudaStreamSynchronize(h->st));
+  unstage(t, dst, src, n);
   return IPM_OK;
 }
 
@@ -1175,6 +1215,7 @@ int ipm_update_costs(ipm_handle* h, const double* f_w, const double* c, int mem,
   if ((rc = enter(h, stream))) return rc;
   if (f_w && fr) CUDA_TRY(h, cudaMemcpyAsync((void*)d.wR, hw.data(), 8 * fr, cudaMemcpyHostToDevice, h->st));
   if (c) CUDA_TRY(h, cudaMemcpyAsync((void*)d.c, hc.data(), 8 * d.n, cudaMemcpyHostToDevice, h->st));
+  if (c) CUDA_TRY(h, cudaMemcpyAsync(&d.sc->cnorm, &cn, sizeof(double), cudaMemcpyHostToDevice, h->st));
   if (f_w) CUDA_TRY(h, launch_diagH(d, h->st));
   if (f_w && d.nblk) CUDA_TRY(h, launch_block_const(d, h->st));   // the blocks' fixed part has w in it
   CUDA_TRY(h, cudaStreamSynchronize(h->st));   // host staging buffers go out of scope
@@ -1803,11 +1844,7 @@ int ipm_device_bytes(const ipm_handle* h, int64_t* matrix_bytes, int64_t* state_
 // of the device scalars and trace back to pinned host memory; does not wait.
 static int solve_launch(ipm_handle* h, int flags, int64_t* direct_launches) {
   int rc;
-  if ((rc = pull_scal(h))) return rc;
-  push_options(h);
-  h->hs->eta_override = 0;
-  h->hs->trace_cap = h->trace_cap;
-  CUDA_TRY(h, cudaMemcpyAsync(h->d.sc, h->hs, sizeof(Scal), cudaMemcpyHostToDevice, h->st));
+  // (the options and norms have been in the device scalars since the QP was loaded)
   const bool warm = (flags & IPM_WARM) && h->have_iterate;
   const int pc = h->precond;
   h->have_iterate = true;
@@ -1987,10 +2024,25 @@ int ipm_get_xyz(ipm_handle* h, double* x, double* y, double* zl, double* zu, dou
   int rc;
   if ((rc = enter(h, stream))) return rc;
   const Dev& d = h->d;
-  if ((rc = copy_out(h, x, d.x, d.n, mem))) return rc;
-  if ((rc = copy_out(h, zl, d.zl, d.n, mem))) return rc;
-  if ((rc = copy_out(h, zu, d.zu, d.n, mem))) return rc;
-  if (!h->stacked) {
+  if (mem == IPM_MEM_HOST) {
+    Staged t;
+    if ((rc = stage_out(h, d.x, d.zu + d.n, 0, &t))) return rc;
+    CUDA_TRY(h, cudaStreamSynchronize(h->st));
+    unstage(t, x, d.x, d.n);
+    unstage(t, zl, d.zl, d.n);
+    unstage(t, zu, d.zu, d.n);
+    if (!h->stacked) {
+      unstage(t, y, d.y, d.m);
+      unstage(t, s, d.s, d.m);
+    }
+  } else {
+    if ((rc = copy_out(h, x, d.x, d.n, mem))) return rc;
+    if ((rc = copy_out(h, zl, d.zl, d.n, mem))) return rc;
+    if ((rc = copy_out(h, zu, d.zu, d.n, mem))) return rc;
+  }
+  if (!h->stacked && mem == IPM_MEM_HOST) {
+    // unstaged above
+  } else if (!h->stacked) {
     if ((rc = copy_out(h, y, d.y, d.m, mem))) return rc;
     if ((rc = copy_out(h, s, d.s, d.m, mem))) return rc;
   } else if (y || s) {
@@ -2016,7 +2068,6 @@ int ipm_get_xyz(ipm_handle* h, double* x, double* y, double* zl, double* zu, dou
     if (s && mu) CUDA_TRY(h, cudaMemcpyAsync(s, so.data(), 8 * (size_t)mu, cudaMemcpyDefault, h->st));
     CUDA_TRY(h, cudaStreamSynchronize(h->st));   // yo, so go out of scope
   }
-  if (mem == IPM_MEM_HOST) CUDA_TRY(h, cudaStreamSynchronize(h->st));
   if (info) ipm_get_info(h, info);
   return leave(h, stream);
 }
@@ -2074,12 +2125,24 @@ int ipm_residuals(ipm_handle* h, double* rd, double* rp, double* rs, double* rl,
   CUDA_TRY(h, launch_residual_summary(d, h->g, h->st));
   // complementarity residuals into scratch vectors (ds: r_s, dzl: r_l, dzu: r_u)
   CUDA_TRY(h, launch_comp_resid(d, h->g, h->st));
-  if ((rc = copy_out(h, rd, d.rd, d.n, mem))) return rc;
-  if ((rc = copy_out(h, rp, d.rp, d.m, mem))) return rc;
-  if ((rc = copy_out(h, rs, d.ds, d.m, mem))) return rc;
-  if ((rc = copy_out(h, rl, d.dzl, d.n, mem))) return rc;
-  if ((rc = copy_out(h, ru, d.dzu, d.n, mem))) return rc;
-  if ((rc = pull_scal(h))) return rc;
+  if (mem == IPM_MEM_HOST) {
+    Staged t;
+    if ((rc = stage_out(h, d.rd, d.dzu + d.n, 0, &t))) return rc;
+    CUDA_TRY(h, cudaStreamSynchronize(h->st));
+    unstage(t, rd, d.rd, d.n);
+    unstage(t, rp, d.rp, d.m);
+    unstage(t, rs, d.ds, d.m);
+    unstage(t, rl, d.dzl, d.n);
+    unstage(t, ru, d.dzu, d.n);
+    std::memcpy(h->hs, t.at + ((const char*)d.sc - t.begin), sizeof(Scal));
+  } else {
+    if ((rc = copy_out(h, rd, d.rd, d.n, mem))) return rc;
+    if ((rc = copy_out(h, rp, d.rp, d.m, mem))) return rc;
+    if ((rc = copy_out(h, rs, d.ds, d.m, mem))) return rc;
+    if ((rc = copy_out(h, rl, d.dzl, d.n, mem))) return rc;
+    if ((rc = copy_out(h, ru, d.dzu, d.n, mem))) return rc;
+    if ((rc = pull_scal(h))) return rc;
+  }
   if (kkt) {
     kkt[0] = h->hs->rel_kkt;
     kkt[1] = h->hs->res_primal;
@@ -2097,10 +2160,14 @@ int ipm_apply_kkt(ipm_handle* h, const double* p, double* q, int mem, void* stre
   if ((rc = enter(h, stream))) return rc;
   const Dev& d = h->d;
   CUDA_TRY(h, launch_diag_update(d, h->g, h->st));
-  if ((rc = copy_in(h, d.p, p, d.n, mem))) return rc;
+  if (mem == IPM_MEM_HOST) {
+    std::memcpy(h->stage, p, sizeof(double) * (size_t)d.n);
+    CUDA_TRY(h, cudaMemcpyAsync(d.p, h->stage, sizeof(double) * (size_t)d.n, cudaMemcpyHostToDevice, h->st));
+  } else if ((rc = copy_in(h, d.p, p, d.n, mem))) {
+    return rc;
+  }
   CUDA_TRY(h, launch_apply(d, h->g, h->st));
-  if ((rc = copy_out(h, q, d.q, d.n, mem))) return rc;
-  if (mem == IPM_MEM_HOST) CUDA_TRY(h, cudaStreamSynchronize(h->st));
+  if ((rc = copy_vector_out(h, q, d.q, d.n, mem))) return rc;
   return leave(h, stream);
 }
 
@@ -2113,8 +2180,7 @@ int ipm_precond_diag(ipm_handle* h, double* diag, int mem, void* stream) {
   const Dev& d = h->d;
   CUDA_TRY(h, launch_diag_update(d, h->g, h->st));
   CUDA_TRY(h, launch_jacobi_full(d, h->g, d.q, h->st));
-  if ((rc = copy_out(h, diag, d.q, d.n, mem))) return rc;
-  if (mem == IPM_MEM_HOST) CUDA_TRY(h, cudaStreamSynchronize(h->st));
+  if ((rc = copy_vector_out(h, diag, d.q, d.n, mem))) return rc;
   return leave(h, stream);
 }
 
@@ -2126,26 +2192,29 @@ int ipm_newton_direction(ipm_handle* h, double eta, double* dx, double* ds, doub
   int rc;
   if ((rc = enter(h, stream))) return rc;
   const Dev& d = h->d;
-  // residual summary at the current iterate, then eta
-  CUDA_TRY(h, launch_residual_summary(d, h->g, h->st));
-  if ((rc = pull_scal(h))) return rc;
-  push_options(h);
-  Scal& s = *h->hs;
-  if (eta > 0) {
-    s.eta = eta;
-  } else {
-    double e = s.eta_factor * s.rel_kkt;
-    s.eta = std::min(s.eta_max, std::max(s.eta_min, std::isfinite(e) ? e : s.eta_max));
-  }
-  CUDA_TRY(h, cudaMemcpyAsync(d.sc, h->hs, sizeof(Scal), cudaMemcpyHostToDevice, h->st));
+  // one graph: residual summary at the current iterate, eta, the step
   if ((rc = ensure_dir_graph(h, h->precond))) return rc;
+  CUDA_TRY(h, launch_ask_eta(d, eta > 0 ? eta : 0.0, h->st));
   CUDA_TRY(h, cudaGraphLaunch(h->graphs[h->precond].dir, h->st));
-  if ((rc = copy_out(h, dx, d.dx, d.n, mem))) return rc;
-  if ((rc = copy_out(h, ds, d.ds, d.m, mem))) return rc;
-  if ((rc = copy_out(h, dy, d.dy, d.m, mem))) return rc;
-  if ((rc = copy_out(h, dzl, d.dzl, d.n, mem))) return rc;
-  if ((rc = copy_out(h, dzu, d.dzu, d.n, mem))) return rc;
-  if ((rc = pull_scal(h))) return rc;
+  if (mem == IPM_MEM_HOST) {
+    Staged t;
+    if ((rc = stage_out(h, d.sc, d.dzu + d.n, 0, &t))) return rc;
+    CUDA_TRY(h, cudaStreamSynchronize(h->st));
+    unstage(t, dx, d.dx, d.n);
+    unstage(t, ds, d.ds, d.m);
+    unstage(t, dy, d.dy, d.m);
+    unstage(t, dzl, d.dzl, d.n);
+    unstage(t, dzu, d.dzu, d.n);
+    std::memcpy(h->hs, t.at, sizeof(Scal));
+  } else {
+    if ((rc = copy_out(h, dx, d.dx, d.n, mem))) return rc;
+    if ((rc = copy_out(h, ds, d.ds, d.m, mem))) return rc;
+    if ((rc = copy_out(h, dy, d.dy, d.m, mem))) return rc;
+    if ((rc = copy_out(h, dzl, d.dzl, d.n, mem))) return rc;
+    if ((rc = copy_out(h, dzu, d.dzu, d.n, mem))) return rc;
+    if ((rc = pull_scal(h))) return rc;
+  }
+  const Scal& s = *h->hs;
   if (rep) {
     rep->iters = s.cg_iter;
     rep->converged = s.cg_conv;
@@ -2276,7 +2345,6 @@ int ipm_batch_solve(ipm_batch* b, void* stream, int* statuses) {
   }
   for (ipm_handle* h : b->hs) {
     push_options(h);
-    h->hs->eta_override = 0;
     h->hs->trace_cap = h->trace_cap;
   }
   if (cudaEventRecord(b->ev, (cudaStream_t)stream) != cudaSuccess || cudaStreamWaitEvent(b->st, b->ev, 0) != cudaSuccess ||

@@ -37,8 +37,9 @@ struct Scal {
   double mu, mu0, eta, tol_kkt, tau;
   double cnorm, bnorm;               // ||c||_inf, ||b||_inf (set once)
   int ipm_iter, max_ipm, status, stop;
-  int equal_steps, eta_override;     // eta_override: eta was set by the caller
+  int equal_steps;
   double eta_factor, eta_min, eta_max, eta_used;
+  double eta_asked;                  // tolerance asked for a single step, 0: the rule's
   // PCG
   double rz, pq, alpha, beta, rr, rhs2, tol2;
   int cg_iter, cg_done, cg_max, cg_conv;

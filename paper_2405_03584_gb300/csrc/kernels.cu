@@ -565,6 +565,10 @@ __global__ void __launch_bounds__(kFinalThreads) k_resid_final(Dev d, int gR, in
     sc->cert_res = mi > 0.0 ? cres : INFINITY;
     sc->cert_gap = mi > 0.0 ? cgap : 0.0;
     if (MODE == RSM_CONTROL) control_step(d, sc->rhs2 > 0.0 ? cg_rel : 0.0, h, set_cond);
+    if (MODE == RSM_STEP) {
+      set_eta(sc);
+      if (sc->eta_asked > 0.0) sc->eta = sc->eta_asked;
+    }
   }
 }
 
@@ -577,6 +581,7 @@ cudaError_t launch_residual_summary(const Dev& d, const Geo& g, cudaStream_t st,
   const int gR = d.nR ? g.gR : 0, sc = h != 0 ? 1 : 0;
   if (mode == RSM_START) k_resid_final<RSM_START><<<1, kFinalThreads, 0, st>>>(d, gR, gM, g.gNr, part, h, sc);
   else if (mode == RSM_CONTROL) k_resid_final<RSM_CONTROL><<<1, kFinalThreads, 0, st>>>(d, gR, gM, g.gNr, part, h, sc);
+  else if (mode == RSM_STEP) k_resid_final<RSM_STEP><<<1, kFinalThreads, 0, st>>>(d, gR, gM, g.gNr, part, h, sc);
   else k_resid_final<RSM_PLAIN><<<1, kFinalThreads, 0, st>>>(d, gR, gM, g.gNr, part, h, sc);
   return cudaGetLastError();
 }
@@ -677,7 +682,6 @@ cudaError_t launch_start_point(const Dev& d, const Geo& g, cudaStream_t st) {
 // Inexact-Newton forcing term of the PCG solve: ||r|| <= eta ||rhs|| with
 // eta = clamp(eta_factor * relKKT, eta_min, eta_max) (reading; the paper states no tolerance).
 static __device__ void set_eta(Scal* sc) {
-  if (sc->eta_override) return;
   double e = sc->eta_factor * sc->rel_kkt;
   if (!(e <= sc->eta_max)) e = sc->eta_max;
   if (e < sc->eta_min) e = sc->eta_min;
@@ -731,6 +735,15 @@ static __device__ void control_step(const Dev& d, double cg_rel, cudaGraphCondit
     sc->trace_rows += 1;
   }
   if (set_cond) cudaGraphSetConditional(h, sc->stop ? 0u : 1u);
+}
+
+__global__ void k_ask_eta(Dev d, double eta) {
+  if (threadIdx.x == 0) d.sc->eta_asked = eta;
+}
+
+cudaError_t launch_ask_eta(const Dev& d, double eta, cudaStream_t st) {
+  k_ask_eta<<<1, 32, 0, st>>>(d, eta);
+  return cudaGetLastError();
 }
 
 // Start of a solve on the device: per-solve totals and the trace cleared.

@@ -263,8 +263,10 @@ cudaError_t launch_densify_R(const Dev& d, cudaStream_t st);   // dense.cu: Rd f
 cudaError_t launch_start_point(const Dev& d, const Geo& g, cudaStream_t st);
 // ---- residual summary at the current iterate and mu ----
 // RSM_START: with the complementarity mean; RSM_CONTROL: followed by the IPM control (mu test,
-// stop rule, eta; h: the loop condition it sets, 0: none)
-enum ResidMode { RSM_PLAIN = 0, RSM_START = 1, RSM_CONTROL = 2 };
+// stop rule, eta; h: the loop condition it sets, 0: none); RSM_STEP: followed by the eta of a
+// single step (the one asked for by launch_ask_eta, or the rule's)
+enum ResidMode { RSM_PLAIN = 0, RSM_START = 1, RSM_CONTROL = 2, RSM_STEP = 3 };
+cudaError_t launch_ask_eta(const Dev& d, double eta, cudaStream_t st);   // 0: by the rule
 cudaError_t launch_residual_summary(const Dev& d, const Geo& g, cudaStream_t st, int mode = RSM_PLAIN,
                                     cudaGraphConditionalHandle h = 0);
 // ---- complementarity residual vectors r_s, r_l, r_u (into ds, dzl, dzu) ----
