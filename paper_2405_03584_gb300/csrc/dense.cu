@@ -23,6 +23,7 @@
 // The factorisation runs once per IPM iteration.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "state.h"
 
@@ -179,6 +180,109 @@ __device__ void tile_potrf(R (*t)[kT + 1], R* rs, const R* A, int64_t ld, int nn
   }
 }
 
+// The diagonal tile in pairs: L D L^T by groups of four pivots, scaled to the Cholesky factor at
+// the end.  What bounds a tile is the chain from pivot to pivot; a reciprocal (the float32
+// estimate and two terms of its error series, in pairs) is shorter than a reciprocal square root
+// followed by a scaling, and four pivots share one barrier: in period p warp 0 (lane i: row i)
+// takes columns 4p .. 4p + 3 into registers, applies group p - 1 to them and factors them, while
+// the other warps apply group p - 1 to the columns beyond.  All square roots are taken at once
+// afterwards.  (One pivot and one square root a barrier: 9.7 us a tile.)
+__device__ __forceinline__ float2 r_rcp(float2 d) {
+  const float r0 = __fdividef(1.f, d.x);
+  float e = __fmaf_rn(-d.x, r0, 1.f);
+  e = __fmaf_rn(-d.y, r0, e);
+  return df_fast_sum(r0, __fmul_rn(r0, __fmaf_rn(e, e, e)));
+}
+
+__device__ void tile_potrf_pairs(float2 (*t)[kT + 1], float2* rs, const float2* A, int64_t ld, int nn, int base,
+                                 const double* diag0, int* nfloor) {
+  __shared__ unsigned short pairs[kTriPairs];
+  __shared__ float2 a4[2][4][kT];      // a group's columns before scaling (L D), by parity
+  __shared__ float2 dg[kT], sq[kT];    // pivots, their square roots
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (int r = ty; r < kT; r += blockDim.x >> 5) {
+    const int gi = base + r, gj = base + tx;
+    t[r][tx] = (gi < nn && gj < nn) ? A[(int64_t)gi * ld + gj] : make_float2(r == tx ? 1.f : 0.f, 0.f);
+  }
+  const float2 fl = r_floor(r_const<float2>(ty == 0 && base + tx < nn ? kFloorRel * fabs(diag0[base + tx]) : 0.0));
+  // pairs (i, j), 1 <= j <= i < 32, by j descending: those with j >= q are the first (32 - q)(33 - q) / 2
+  for (int e = threadIdx.x; e < kTriPairs; e += blockDim.x) {
+    int j = kT - 1, rem = e;
+    while (rem >= kT - j) {
+      rem -= kT - j;
+      --j;
+    }
+    pairs[e] = (unsigned short)((j + rem) * kT + j);
+  }
+  __syncthreads();
+  float2 l[4], x[4];                   // warp 0: the last group's columns, scaled and not
+#pragma unroll
+  for (int s = 0; s < 4; ++s) l[s] = x[s] = make_float2(0.f, 0.f);
+  for (int p = 0; p < kT / 4; ++p) {
+    const int c0 = 4 * p;
+    if (ty == 0) {
+      float2 y[4];
+#pragma unroll
+      for (int s = 0; s < 4; ++s) y[s] = t[tx][c0 + s];
+      if (p > 0) {
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) y[s] = r_fms(y[s], l[q], r_shfl(x[q], c0 + s));
+      }
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        float2 piv = r_shfl(y[s], c0 + s);
+        const float2 flc = r_shfl(fl, c0 + s);
+        if (base + c0 + s < nn && !r_above(piv, flc)) {
+          piv = flc;
+          if (nfloor && tx == 0) atomicAdd(nfloor, 1);
+        }
+        const float2 r = r_rcp(piv);
+        if (tx == 0) dg[c0 + s] = piv;
+        x[s] = y[s];
+        l[s] = tx > c0 + s ? r_mul(y[s], r) : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int q = s + 1; q < 4; ++q) y[q] = r_fms(y[q], l[s], r_shfl(x[s], c0 + q));
+      }
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        a4[p & 1][s][tx] = x[s];
+        if (tx > c0 + s) t[tx][c0 + s] = l[s];
+      }
+    } else if (p > 0) {
+      const int b0 = c0 - 4, cnt = (kT - c0 - 4) * (kT - c0 - 3) / 2;   // columns >= c0 + 4
+      for (int e = threadIdx.x - 32; e < cnt; e += blockDim.x - 32) {
+        const int i = pairs[e] / kT, j = pairs[e] % kT;
+        float2 v = t[i][j];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) v = r_fms(v, t[i][b0 + s], a4[(p - 1) & 1][s][j]);
+        t[i][j] = v;
+      }
+    }
+    __syncthreads();
+  }
+  if (ty == 0) {
+    const float2 piv = dg[tx], r = r_rsqrt(piv), q = r_mul(piv, r);
+    rs[tx] = r;
+    sq[tx] = q;
+    t[tx][tx] = q;
+  }
+  __syncthreads();
+  for (int r = ty; r < kT; r += blockDim.x >> 5)
+    if (tx < r) t[r][tx] = r_mul(t[r][tx], sq[tx]);
+  __syncthreads();
+}
+
+template <class R>
+__device__ __forceinline__ void tile_factor(R (*t)[kT + 1], R* rs, const R* A, int64_t ld, int nn, int base,
+                                            const double* diag0, int* nfloor) {
+  if constexpr (sizeof(R) == sizeof(double) && !std::is_same<R, double>::value)
+    tile_potrf_pairs(t, rs, A, ld, nn, base, diag0, nfloor);
+  else
+    tile_potrf<R>(t, rs, A, ld, nn, base, diag0, nfloor);
+}
+
 // Panel of tile column kb: block 0 the diagonal tile, block b >= 1 rows
 // [base + 32 + kPanelRows (b - 1), + kPanelRows) below it, one warp per row.  Every block loads
 // the diagonal tile from A, and a block may start after block 0 has finished (when other
@@ -195,7 +299,7 @@ __global__ void __launch_bounds__(kPanelThreads) k_chol_panel(R* A, int64_t ld, 
   if (blockIdx.x > 0 && row0 >= nn) return;   // whole block: before any barrier
   __shared__ R t[kT][kT + 1];
   __shared__ R rs[kT];
-  tile_potrf<R>(t, rs, A, ld, nn, base, diag0, blockIdx.x == 0 ? nfloor : nullptr);
+  tile_factor<R>(t, rs, A, ld, nn, base, diag0, blockIdx.x == 0 ? nfloor : nullptr);
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   if (blockIdx.x == 0) {
     for (int r = ty; r < kT; r += kPanelThreads / 32)
@@ -395,20 +499,34 @@ __global__ void k_dense_maxima(Dev d) {
 // One block: B = nR max_i omega_i max R^2 + max_j |h0_j + sigma_j| + max |Hs| + (a bound on
 // the low-rank term) bounds every |K_ij|; s = 2^-2e with 2^2e > B puts K's entries below 1 in
 // magnitude.  Then the scaled row weights as pairs, wdf_i = s omega_i.
+// (The maxima are of numbers >= 0 and are taken on their bits: a float64 tree over 32 warps holds
+// the SM for 2500 cycles a quantity.)
 __global__ void __launch_bounds__(1024) k_dense_prep(Dev d) {
-  __shared__ double sh[32];
+  __shared__ unsigned long long sm[3];
   __shared__ double s_scale;
-  double mw = 0.0, md = 0.0, ml = 0.0;
-  for (int64_t i = threadIdx.x; i < d.nR; i += blockDim.x) mw = fmax(mw, fabs(d.omega[i]));
-  for (int64_t j = threadIdx.x; j < d.n; j += blockDim.x) md = fmax(md, fabs(d.h0[j] + d.sigma[j]));
+  if (threadIdx.x < 3) sm[threadIdx.x] = 0ull;
+  __syncthreads();
+  unsigned long long m[3] = {0ull, 0ull, 0ull};
+  auto keep = [](unsigned long long& a, double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(fabs(v));
+    if (b > a && b <= 0x7ff0000000000000ull) a = b;
+  };
+  for (int i = threadIdx.x; i < d.nR; i += blockDim.x) keep(m[0], d.omega[i]);
+  for (int j = threadIdx.x; j < d.n; j += blockDim.x) keep(m[1], d.h0[j] + d.sigma[j]);
   if (d.ucols)
     for (int64_t e = threadIdx.x; e < d.n * d.ucols; e += blockDim.x) {
       const double u = d.U[e];
-      ml = fmax(ml, u * u * fabs(d.uw[e % d.ucols]) * (double)d.ucols);
+      keep(m[2], u * u * fabs(d.uw[e % d.ucols]) * (double)d.ucols);
     }
-  mw = block_reduce<1>(mw, sh);
-  md = block_reduce<1>(md, sh);
-  ml = block_reduce<1>(ml, sh);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m[q] = max(m[q], __shfl_xor_sync(0xffffffffu, m[q], o));
+    if ((threadIdx.x & 31) == 0 && m[q]) atomicMax(&sm[q], m[q]);
+  }
+  __syncthreads();
+  const double mw = __longlong_as_double((long long)sm[0]), md = __longlong_as_double((long long)sm[1]),
+               ml = __longlong_as_double((long long)sm[2]);
   if (threadIdx.x == 0) {
     const unsigned long long* aux = reinterpret_cast<const unsigned long long*>(d.dense_aux);
     const double rmax2 = __longlong_as_double((long long)aux[0]);
@@ -429,7 +547,7 @@ __global__ void __launch_bounds__(1024) k_dense_prep(Dev d) {
 
 // K = R^T diag(omega) R + U W U^T (scaled, as pairs) by 32 x 32 tiles: one block per tile of
 // the lower triangle, 2 x 2 outputs per thread, each a sum in row order, so K is
-// deterministic; off-diagonal tiles are written to both triangles.
+// deterministic.
 constexpr int kGT = 32;
 
 __device__ __forceinline__ void tile_of_block(int64_t b, int64_t& tj, int64_t& tl) {
@@ -460,9 +578,9 @@ __device__ __forceinline__ void gram_lowrank_acc(const Dev& d, int64_t J0, int64
   }
 }
 
-// the tile's stores (both triangles off the diagonal)
-__device__ __forceinline__ void gram_store(const Dev& d, int64_t J0, int64_t L0, int64_t tj, int64_t tl,
-                                           const float (&h)[2][2], const float (&l)[2][2]) {
+// the tile's stores (the factorisation reads the lower triangle and its last pass fills the upper)
+__device__ __forceinline__ void gram_store(const Dev& d, int64_t J0, int64_t L0, const float (&h)[2][2],
+                                           const float (&l)[2][2]) {
   const int64_t n = d.n;
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
 #pragma unroll
@@ -473,7 +591,6 @@ __device__ __forceinline__ void gram_store(const Dev& d, int64_t J0, int64_t L0,
       if (j < n && lc < n) {
         const float2 v = df_fast_sum(h[a][c], l[a][c]);
         d.Kd[j * n + lc] = v;
-        if (tj != tl) d.Kd[lc * n + j] = v;
       }
     }
 }
@@ -520,7 +637,7 @@ __global__ void __launch_bounds__(256) k_gram_tiles(Dev d) {
     __syncthreads();
   }
   gram_lowrank_acc(d, J0, L0, sJ, sL, h, l);
-  gram_store(d, J0, L0, tj, tl, h, l);
+  gram_store(d, J0, L0, h, l);
 }
 
 // From the dense copy of R (pairs): chunks of 32 rows of Rd staged in shared memory (one side
@@ -574,7 +691,7 @@ __global__ void __launch_bounds__(256) k_gram_gemm(Dev d) {
   }
   if (blockIdx.y == 0) gram_lowrank_acc(d, J0, L0, &sA[0][0], &sB[0][0], h, l);
   if (gridDim.y == 1) {
-    gram_store(d, J0, L0, tj, tl, h, l);
+    gram_store(d, J0, L0, h, l);
     return;
   }
   float2* part = d.gram_part + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * kGT * kGT;
@@ -606,7 +723,6 @@ __global__ void k_gram_sum(Dev d, int splits, int64_t tiles) {
     }
     const float2 v = df_fast_sum(h, l);
     d.Kd[j * n + lc] = v;
-    if (tj != tl) d.Kd[lc * n + j] = v;
   }
 }
 
@@ -631,7 +747,8 @@ cudaError_t launch_densify_R(const Dev& d, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// Adds s (diag(h0 + sigma) + Hs) (each entry once: no conflicts), in float64 on the pair.
+// Adds s (diag(h0 + sigma) + Hs) to the lower triangle (each entry once: no conflicts), in float64
+// on the pair.
 __global__ void k_gram_diag_hs(Dev d) {
   const int64_t n = d.n;
   const double s = d.dense_aux[2];
@@ -643,6 +760,7 @@ __global__ void k_gram_diag_hs(Dev d) {
     if (d.Hs_ptr) {
       __syncthreads();
       for (int64_t e = d.Hs_ptr[j] + threadIdx.x; e < d.Hs_ptr[j + 1]; e += blockDim.x) {
+        if (d.Hs_idx[e] > j) continue;
         float2* kp = d.Kd + j * n + d.Hs_idx[e];
         *kp = df_split(df_value(kp->x, kp->y) + s * d.Hs_val[e]);
       }

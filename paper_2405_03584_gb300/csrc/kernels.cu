@@ -1488,21 +1488,91 @@ __global__ void k_stiff_corr(Dev d, int init) {
 // r' = 2^-e r (2^e >= max |r|, exact) and z = s 2^e z'.  In blocks of 32 rows: the block's
 // 32 values come from the inverse of its diagonal tile (one warp per row, a shuffle-tree sum
 // of pairs: no row-by-row chain), then all threads update the remaining rows with the block's
-// 32 columns while the next tile's inverse is staged in shared memory.  Thread r reads its
-// row's 32 factor entries (256 contiguous bytes: after the first miss the rest hit L1).  One block of 1024
-// threads; y in shared memory (n <= 2048).  r^T z -> rz / beta; init: p = z.  (PCG with the
-// factor converges in one or two iterations, so this replaces forming K^{-1} once per IPM
-// iteration.)
+// 32 columns.  One block of 1024 threads; y in shared memory (n <= 2048).  r^T z -> rz / beta;
+// init: p = z.  (PCG with the factor converges in one or two iterations, so this replaces
+// forming K^{-1} once per IPM iteration.)
+//
+// The chain of 2 n / 32 steps is what bounds it, so nothing in a step waits for memory that
+// could have been asked for before: each thread pair's 32 factor entries of the next block (16
+// entries a thread, in 16-byte loads where rows start on 16 bytes) and the next tile's inverse
+// are fetched into registers before the barriers of the current step, and a row's 32 terms are
+// split over two threads with two accumulators each.  (n = 500: 128 us for the two sweeps with one
+// thread a row loading as it went.)
+struct TrsvRow {
+  float2 v[16];
+};
+// 16 entries of a row from column c0; VEC: 16-byte loads (row and column even)
+template <bool VEC>
+__device__ __forceinline__ void trsv_fetch(const float2* row, int c0, int left, TrsvRow& t) {
+  if (VEC && left >= 16) {
+    const float4* p = reinterpret_cast<const float4*>(row + c0);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const float4 u = p[k];
+      t.v[2 * k] = make_float2(u.x, u.y);
+      t.v[2 * k + 1] = make_float2(u.z, u.w);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) t.v[k] = k < left ? row[c0 + k] : make_float2(0.f, 0.f);
+  }
+}
+__device__ __forceinline__ void trsv_dot(const TrsvRow& t, const float2* yk, float& h, float& l) {
+  float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f;
+#pragma unroll
+  for (int k = 0; k < 16; k += 2) {
+    df_mac(t.v[k], yk[k], h0, l0);
+    df_mac(t.v[k + 1], yk[k + 1], h1, l1);
+  }
+  float e;
+  two_sum(h0, h1, h, e);
+  l = __fadd_rn(__fadd_rn(l0, l1), e);
+}
+
+// y[r] -= row r's 32 terms for rows r0 <= r < r1 (rows beyond the first 512 of the range load as
+// they go), two neighbouring threads a row; `row`: the thread's fetched part of row r0 + tid / 2.
+template <bool VEC>
+__device__ __forceinline__ void trsv_rows(const float2* K, int64_t ld, int kb, int bs, int r0, int r1, float2* y,
+                                          const float2* yk, TrsvRow& row) {
+  const int tid = threadIdx.x, half = tid & 1, c0 = 16 * half;
+  for (int rr = r0; rr < r1; rr += 512) {
+    const int r = rr + (tid >> 1);
+    if (rr != r0 && r < r1) trsv_fetch<VEC>(K + (int64_t)r * ld, kb + c0, bs - c0, row);
+    float h = 0.f, l = 0.f;
+    if (r < r1) trsv_dot(row, yk + c0, h, l);
+    const float oh = __shfl_xor_sync(0xffffffffu, h, 1), ol = __shfl_xor_sync(0xffffffffu, l, 1);
+    if (r < r1 && half == 0) {
+      float sm, e;
+      two_sum(h, oh, sm, e);
+      y[r] = df_sub_sum(y[r], sm, __fadd_rn(__fadd_rn(l, ol), e));
+    }
+  }
+}
+
+template <bool VEC>
 __global__ void __launch_bounds__(1024) k_dense_trsv(Dev d, int init) {
   extern __shared__ float2 y[];
   __shared__ double sh[32];
-  __shared__ float2 Li[2][32][33];
+  __shared__ float2 Li[32][33];
   __shared__ float2 yk[32];
   if (!init && d.sc->cg_done) return;
   const int n = (int)d.n;
   const int nt = (n + 31) / 32;
   const float2* K = d.Kd;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, c0 = 16 * (tid & 1);
+  // tile t's inverse entry and the thread's part of its row below (forward) or above (backward)
+  // the tile, for the step to come
+  float2 li = d.chol_tinv[warp * 32 + lane];
+  TrsvRow row;
+  auto fetch_fwd = [&](int t) {
+    const int kb = t * 32, bs = min(32, n - kb), r = kb + bs + (tid >> 1);
+    if (r < n) trsv_fetch<VEC>(K + (int64_t)r * n, kb + c0, bs - c0, row);
+  };
+  auto fetch_bwd = [&](int t) {
+    const int kb = t * 32, bs = min(32, n - kb), r = tid >> 1;
+    if (r < kb) trsv_fetch<VEC>(K + (int64_t)r * n, kb + c0, bs - c0, row);
+  };
+  fetch_fwd(0);
   double rmax = 0.0;
   for (int i = tid; i < n; i += blockDim.x) rmax = fmax(rmax, fabs(d.r[i]));
   rmax = block_reduce<1>(rmax, sh);
@@ -1510,42 +1580,42 @@ __global__ void __launch_bounds__(1024) k_dense_trsv(Dev d, int init) {
   if (rmax > 0.0 && isfinite(rmax)) frexp(rmax, &er);
   const double rs = ldexp(1.0, -er);
   for (int i = tid; i < n; i += blockDim.x) y[i] = df_split(d.r[i] * rs);
-  if (nt > 0) Li[0][warp][lane] = d.chol_tinv[warp * 32 + lane];
+  Li[warp][lane] = li;
   __syncthreads();
   // forward: L y = r'
   for (int t = 0; t < nt; ++t) {
-    const int kb = t * 32, bs = min(32, n - kb), cur = t & 1;
+    const int kb = t * 32, bs = min(32, n - kb);
+    if (t + 1 < nt) li = d.chol_tinv[(int64_t)(t + 1) * 1024 + warp * 32 + lane];
     float h = 0.f, l = 0.f;
-    if (lane < bs) df_mac(Li[cur][warp][lane], y[kb + lane], h, l);
+    if (lane < bs) df_mac(Li[warp][lane], y[kb + lane], h, l);
     df_group_pair<32>(h, l);
     if (lane == 0) yk[warp] = df_fast_sum(h, l);
     __syncthreads();
-    if (t + 1 < nt) Li[cur ^ 1][warp][lane] = d.chol_tinv[(int64_t)(t + 1) * 1024 + warp * 32 + lane];
     if (tid < bs) y[kb + tid] = yk[tid];
-    for (int r = kb + bs + tid; r < n; r += blockDim.x) {
-      const float2* Lr = K + (int64_t)r * n + kb;
-      float ah = 0.f, al = 0.f;
-      for (int c = 0; c < bs; ++c) df_mac(Lr[c], yk[c], ah, al);
-      y[r] = df_sub_sum(y[r], ah, al);
+    trsv_rows<VEC>(K, n, kb, bs, kb + bs, n, y, yk, row);
+    if (t + 1 < nt) {
+      Li[warp][lane] = li;
+      fetch_fwd(t + 1);
+    } else {
+      fetch_bwd(t);
     }
     __syncthreads();
   }
   // backward: L^T z' = y, with L^T row i in the upper triangle of row i; tile nt - 1's
   // inverse is still staged
   for (int t = nt - 1; t >= 0; --t) {
-    const int kb = t * 32, bs = min(32, n - kb), cur = t & 1;
+    const int kb = t * 32, bs = min(32, n - kb);
+    if (t > 0) li = d.chol_tinv[(int64_t)(t - 1) * 1024 + warp * 32 + lane];
     float h = 0.f, l = 0.f;
-    if (lane < bs) df_mac(Li[cur][lane][warp], y[kb + lane], h, l);
+    if (lane < bs) df_mac(Li[lane][warp], y[kb + lane], h, l);
     df_group_pair<32>(h, l);
     if (lane == 0) yk[warp] = df_fast_sum(h, l);
     __syncthreads();
-    if (t > 0) Li[cur ^ 1][warp][lane] = d.chol_tinv[(int64_t)(t - 1) * 1024 + warp * 32 + lane];
     if (tid < bs) y[kb + tid] = yk[tid];
-    for (int r = tid; r < kb; r += blockDim.x) {
-      const float2* Ur = K + (int64_t)r * n + kb;
-      float ah = 0.f, al = 0.f;
-      for (int c = 0; c < bs; ++c) df_mac(Ur[c], yk[c], ah, al);
-      y[r] = df_sub_sum(y[r], ah, al);
+    trsv_rows<VEC>(K, n, kb, bs, 0, kb, y, yk, row);
+    if (t > 0) {
+      Li[warp][lane] = li;
+      fetch_bwd(t - 1);
     }
     __syncthreads();
   }
@@ -1571,6 +1641,11 @@ __global__ void __launch_bounds__(1024) k_dense_trsv(Dev d, int init) {
       sc->rz = rz;
     }
   }
+}
+
+static void launch_trsv(const Dev& d, int init, cudaStream_t st) {
+  if (d.n & 1) k_dense_trsv<false><<<1, 1024, sizeof(float2) * d.n, st>>>(d, init);
+  else k_dense_trsv<true><<<1, 1024, sizeof(float2) * d.n, st>>>(d, init);
 }
 
 // Jacobi start: z = r / M, p = z, rz = r^T z.
@@ -1616,7 +1691,7 @@ cudaError_t launch_cg_init(const Dev& d, const Geo& g, int precond, cudaStream_t
   }
   if (precond == PC_BLOCK32) return launch_block_apply(d, 1, st);
   if (precond == PC_DENSE) {
-    k_dense_trsv<<<1, 1024, sizeof(float2) * d.n, st>>>(d, 1);
+    launch_trsv(d, 1, st);
   } else {
     k_cg_init_diag<<<g.eN, kBlock, 0, st>>>(d);
     if (precond == PC_JACOBI_LR && d.m) {
@@ -1657,7 +1732,7 @@ cudaError_t launch_cg_body(const Dev& d, const Geo& g, int precond, cudaGraphCon
     launch_block_apply(d, 0, st);
   } else if (precond == PC_DENSE) {
     k_cg_update<2><<<g.eN, kBlock, 0, st>>>(d, npart);
-    k_dense_trsv<<<1, 1024, sizeof(float2) * d.n, st>>>(d, 0);
+    launch_trsv(d, 0, st);
   } else if (precond == PC_JACOBI_LR && d.m) {
     k_cg_update<1><<<g.eN, kBlock, 0, st>>>(d, npart);
     const int gs = (d.stiff_cap + 7) / 8;
