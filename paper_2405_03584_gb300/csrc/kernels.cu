@@ -76,12 +76,13 @@ Geo make_geo(const Dev& d) {
 // in block order), then (U (W t))_j inside the column kernels (lr_row).  Row-major U makes
 // both passes read rows of U contiguously.
 //
-// A thread owns 8 neighbouring columns (64 bytes of a row, in 16-byte loads where rows start on
-// 16 bytes) and walks every rg-th row of its block's chunk, rg = 256 / ceil(ucols / 8) rows of
+// A thread owns 8 columns (in 16-byte loads of two where rows start on 16 bytes; neighbouring
+// threads load neighbouring ones) and walks every rg-th row of its block's chunk, rg = 256 / ceil(ucols / 8) rows of
 // threads side by side: of 256 threads 250 carry columns at 200 columns, where 32 lanes over
 // 128-column slices carried 200 of 256 values, and every float64 instruction of a warp costs the
 // same.  (n = 77373, 200 columns: 41 us before.)
 constexpr int kLrCols = 8;
+constexpr int kLrTile = kBlock / 4;              // rows of U a block of the column pass takes at a time
 constexpr int kLrSlice = 256 * kLrCols;          // columns a block covers at a time
 template <bool VEC>
 __global__ void __launch_bounds__(256) k_lr_part(Dev d, const double* __restrict__ v) {
@@ -94,50 +95,53 @@ __global__ void __launch_bounds__(256) k_lr_part(Dev d, const double* __restrict
     const int w = (int)(uc - r0 < kLrSlice ? uc - r0 : kLrSlice);
     const int nch = (w + kLrCols - 1) / kLrCols, rg = 256 / nch;
     const int c = tid % nch, g = tid / nch;
-    const int cols = w - c * kLrCols < kLrCols ? w - c * kLrCols : kLrCols;
+    const int nv = w / 2;                  // VEC: pairs of columns
     double acc[kLrCols];
 #pragma unroll
     for (int k = 0; k < kLrCols; ++k) acc[k] = 0.0;
     if (g < rg) {
-      const double* u = d.U + r0 + c * kLrCols;
-      if (VEC && cols == kLrCols) {
+      if (VEC) {
+        const double2* u = reinterpret_cast<const double2*>(d.U + r0) + c;
+        const int64_t uv = uc / 2;
         int64_t j = j0 + g;
-        for (; j + rg < j1; j += 2 * rg) {
-          const double2* p0 = reinterpret_cast<const double2*>(u + j * uc);
-          const double2* p1 = reinterpret_cast<const double2*>(u + (j + rg) * uc);
-          double2 a[kLrCols / 2], b[kLrCols / 2];
-          const double x0 = __ldg(v + j), x1 = __ldg(v + j + rg);
+        if (c + (kLrCols / 2 - 1) * nch < nv) {
+          for (; j + rg < j1; j += 2 * rg) {
+            const double2 *p0 = u + j * uv, *p1 = u + (j + rg) * uv;
+            double2 a[kLrCols / 2], b[kLrCols / 2];
+            const double x0 = __ldg(v + j), x1 = __ldg(v + j + rg);
 #pragma unroll
-          for (int k = 0; k < kLrCols / 2; ++k) a[k] = __ldg(p0 + k);
+            for (int k = 0; k < kLrCols / 2; ++k) a[k] = __ldg(p0 + k * nch);
 #pragma unroll
-          for (int k = 0; k < kLrCols / 2; ++k) b[k] = __ldg(p1 + k);
+            for (int k = 0; k < kLrCols / 2; ++k) b[k] = __ldg(p1 + k * nch);
 #pragma unroll
-          for (int k = 0; k < kLrCols / 2; ++k) {
-            acc[2 * k] = fma(a[k].x, x0, acc[2 * k]);
-            acc[2 * k + 1] = fma(a[k].y, x0, acc[2 * k + 1]);
-          }
+            for (int k = 0; k < kLrCols / 2; ++k) {
+              acc[2 * k] = fma(a[k].x, x0, acc[2 * k]);
+              acc[2 * k + 1] = fma(a[k].y, x0, acc[2 * k + 1]);
+            }
 #pragma unroll
-          for (int k = 0; k < kLrCols / 2; ++k) {
-            acc[2 * k] = fma(b[k].x, x1, acc[2 * k]);
-            acc[2 * k + 1] = fma(b[k].y, x1, acc[2 * k + 1]);
+            for (int k = 0; k < kLrCols / 2; ++k) {
+              acc[2 * k] = fma(b[k].x, x1, acc[2 * k]);
+              acc[2 * k + 1] = fma(b[k].y, x1, acc[2 * k + 1]);
+            }
           }
         }
-        if (j < j1) {
-          const double2* p0 = reinterpret_cast<const double2*>(u + j * uc);
+        for (; j < j1; j += rg) {
           const double x0 = __ldg(v + j);
 #pragma unroll
-          for (int k = 0; k < kLrCols / 2; ++k) {
-            const double2 a = __ldg(p0 + k);
-            acc[2 * k] = fma(a.x, x0, acc[2 * k]);
-            acc[2 * k + 1] = fma(a.y, x0, acc[2 * k + 1]);
-          }
+          for (int k = 0; k < kLrCols / 2; ++k)
+            if (c + k * nch < nv) {
+              const double2 a = __ldg(u + j * uv + k * nch);
+              acc[2 * k] = fma(a.x, x0, acc[2 * k]);
+              acc[2 * k + 1] = fma(a.y, x0, acc[2 * k + 1]);
+            }
         }
       } else {
+        const double* u = d.U + r0 + c;
         for (int64_t j = j0 + g; j < j1; j += rg) {
           const double x0 = __ldg(v + j);
 #pragma unroll
           for (int k = 0; k < kLrCols; ++k)
-            if (k < cols) acc[k] = fma(__ldg(u + j * uc + k), x0, acc[k]);
+            if (c + k * nch < w) acc[k] = fma(__ldg(u + j * uc + k * nch), x0, acc[k]);
         }
       }
     }
@@ -145,8 +149,10 @@ __global__ void __launch_bounds__(256) k_lr_part(Dev d, const double* __restrict
     for (int k = 0; k < kLrCols; ++k) sh[tid][k] = acc[k];
     __syncthreads();
     for (int t = tid; t < w; t += 256) {
+      // the thread and accumulator of column t
+      const int i = VEC ? t / 2 : t, th = i % nch, k = VEC ? 2 * (i / nch) + (t & 1) : i / nch;
       double s = 0.0;
-      for (int q = 0; q < rg; ++q) s += sh[q * nch + t / kLrCols][t % kLrCols];
+      for (int q = 0; q < rg; ++q) s += sh[q * nch + th][k];
       d.upart[(r0 + t) * (int64_t)d.ublocks + blockIdx.x] = s;   // column-major: the final sum reads runs
     }
     __syncthreads();
@@ -1330,32 +1336,125 @@ cudaError_t launch_op_rows_runs(const Dev& d, const Geo& g, int mode, cudaStream
 // q = R^T v + Hs p + (h0 + sigma) o p; p^T q by blocks.
 // MODE 0: inside PCG; MODE 1: a single operator apply (no scalars touched); MODE 2: as 1,
 // when the reduced-precision PCG asks for a residual replacement.
-template <int MODE, int G>
+// EXT: with any of a sparse block of H, the low-rank term and the augmented system; without, the
+// pass keeps its registers for the loads (six blocks an SM allow 40; with them 24 bytes spill).
+// The block's 256 / G variables are finished by that many neighbouring threads: the last
+// float64 instructions of a variable cost a warp the same for one lane as for 32 (n = 50000,
+// 49.9 million entries: 132 -> 119 us with both; the entries' multiply-adds alone take 84 us of
+// the float64 pipe).
+template <int MODE, int G, bool EXT>
 __global__ void __launch_bounds__(256, kOpColsMinBlocks) k_op_cols(Dev d) {
+  constexpr int C = kBlock / G;
   __shared__ double sh[32];
+  __shared__ double st[2][C];
   if (MODE == 0 && d.sc->cg_done) return;
   if (MODE == 2 && !d.sc->ru_do) return;
+  const int tid = threadIdx.x, gl = glane<G>();
   double pq = 0.0;
-  FOR_GROUP_ROWS(G, j, ok, d.n) {
+  int buf = 0;
+  for (int64_t j0 = (int64_t)blockIdx.x * C; j0 < d.n; j0 += (int64_t)gridDim.x * C, buf ^= 1) {
+    const int64_t j = j0 + tid / G;
+    const bool ok = j < d.n;
     const int64_t beg = ok ? d.RT_ptr[j] : 0, end = ok ? d.RT_ptr[j + 1] : 0;
-    double acc = group_row_dot<G, false>(beg, end, glane<G>(), d.RT_idx, d.RT_val, d.vR);
-    if (d.Hs_ptr) {
+    double acc = group_row_dot<G, false>(beg, end, gl, d.RT_idx, d.RT_val, d.vR);
+    if (EXT && d.Hs_ptr) {
       const int64_t hb = ok ? d.Hs_ptr[j] : 0, he = ok ? d.Hs_ptr[j + 1] : 0;
-      acc += group_row_dot<G, false>(hb, he, glane<G>(), d.Hs_idx, d.Hs_val, d.p);
+      acc += group_row_dot<G, false>(hb, he, gl, d.Hs_idx, d.Hs_val, d.p);
     }
-    if (d.ucols) acc += lr_row<G>(d, j, ok, glane<G>());
-    if (ok && glane<G>() == 0) {
-      const double pj = d.p[j];
-      const double qj = acc + (d.h0[j] + d.sigma[j]) * pj;
-      d.q[j] = qj;
+    if (EXT && d.ucols) acc += lr_row<G>(d, j, ok, gl);
+    if (gl == 0) st[buf][tid / G] = acc;
+    __syncthreads();
+    const int64_t jj = j0 + tid;
+    if (tid < C && jj < d.n) {
+      const double pj = d.p[jj];
+      const double qj = st[buf][tid] + (d.h0[jj] + d.sigma[jj]) * pj;
+      d.q[jj] = qj;
       pq = fma(pj, qj, pq);
     }
   }
   if (MODE != 0) return;
-  if (d.aug)   // p^T q over the bottom block too (q's bottom written by the rows pass)
+  if (EXT && d.aug)   // p^T q over the bottom block too (q's bottom written by the rows pass)
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < d.m; k += (int64_t)gridDim.x * blockDim.x)
       pq = fma(d.p[d.n + k], d.q[d.n + k], pq);
   store_pq_part(d, pq, sh);
+}
+
+// The same where H has the low-rank term alone (no matrix rows, no sparse block; float64 storage,
+// an even number of columns): a block takes kLrTile rows of U at a time, four lanes a row, four
+// 16-byte loads of U in flight a lane, and finishes its rows by that many neighbouring threads.
+// n = 77373, 200 columns: 45.9 us in the general kernel, 38.2 here; the float64 pipe alone takes
+// 26 us, U (124 MB, the size of the L2) 18 us from memory.  Loading the next four pairs ahead of
+// the adds at 64 registers a thread was slower (42.8 us).
+template <int MODE>
+__global__ void __launch_bounds__(256, kOpColsMinBlocks) k_op_cols_lr(Dev d) {
+  constexpr int G = 4, B = 4;
+  __shared__ double sh[32];
+  __shared__ double st[2][kLrTile];
+  if (MODE == 0 && d.sc->cg_done) return;
+  const int tid = threadIdx.x, gl = tid & (G - 1), c = tid / G;
+  const int nv = (int)(d.ucols >> 1);
+  const double2* s2 = reinterpret_cast<const double2*>(d.lrs);
+  double pq = 0.0;
+  int buf = 0;
+  for (int64_t j0 = (int64_t)blockIdx.x * kLrTile; j0 < d.n; j0 += (int64_t)gridDim.x * kLrTile, buf ^= 1) {
+    const int64_t j = j0 + c < d.n ? j0 + c : d.n - 1;
+    const double2* row = reinterpret_cast<const double2*>(d.U + j * d.ucols);
+    double a0 = 0.0, a1 = 0.0;
+    for (int v = gl; v < nv; v += B * G) {
+      double2 u[B], w[B];
+#pragma unroll
+      for (int k = 0; k < B; ++k) {
+        const bool in = v + k * G < nv;
+        u[k] = in ? __ldg(row + v + k * G) : make_double2(0.0, 0.0);
+        w[k] = in ? __ldg(s2 + v + k * G) : make_double2(0.0, 0.0);
+      }
+#pragma unroll
+      for (int k = 0; k < B; ++k)
+        if (v - gl + k * G < nv) {     // the same for the whole group: no float64 work past the row's end
+          a0 = fma(u[k].x, w[k].x, a0);
+          a1 = fma(u[k].y, w[k].y, a1);
+        }
+    }
+    a0 += a1;
+    a0 += __shfl_xor_sync(0xffffffffu, a0, 2);
+    a0 += __shfl_xor_sync(0xffffffffu, a0, 1);
+    if (gl == 0) st[buf][c] = a0;
+    __syncthreads();
+    const int64_t jj = j0 + tid;
+    if (tid < kLrTile && jj < d.n) {
+      const double pj = d.p[jj];
+      const double qj = st[buf][tid] + (d.h0[jj] + d.sigma[jj]) * pj;
+      d.q[jj] = qj;
+      pq = fma(pj, qj, pq);
+    }
+  }
+  if (MODE == 0) store_pq_part(d, pq, sh);
+}
+
+static bool lr_alone(const Dev& d) {
+  return d.storage == ST_F64 && d.ucols && !(d.ucols & 1) && !d.nnzR && !d.Hs_ptr && !d.aug;
+}
+
+// Its blocks: as many tiles each as the most loaded block of a resident wave has, on fewer blocks.
+static int lr_blocks(const Dev& d, const Geo& g) {
+  const int64_t tiles = (d.n + kLrTile - 1) / kLrTile, each = (tiles + g.gN64 - 1) / g.gN64;
+  return (int)((tiles + each - 1) / each);
+}
+
+static void launch_op_cols(const Dev& d, const Geo& g, int mode, cudaStream_t st) {
+  if (lr_alone(d)) {
+    const int gl = lr_blocks(d, g);
+    if (mode == 0) k_op_cols_lr<0><<<gl, kBlock, 0, st>>>(d);
+    else k_op_cols_lr<1><<<gl, kBlock, 0, st>>>(d);
+  } else if (d.Hs_ptr || d.ucols || d.aug) {
+    if (mode == 0) DISPATCH_G(d.g_cols, k_op_cols<0, G, true><<<g.gN64, kBlock, 0, st>>>(d));
+    else if (mode == 1) DISPATCH_G(d.g_cols, k_op_cols<1, G, true><<<g.gN64, kBlock, 0, st>>>(d));
+    else DISPATCH_G(d.g_cols, k_op_cols<2, G, true><<<g.gN64, kBlock, 0, st>>>(d));
+  } else {
+    if (mode == 0) DISPATCH_G(d.g_cols, k_op_cols<0, G, false><<<g.gN64, kBlock, 0, st>>>(d));
+    else if (mode == 1) DISPATCH_G(d.g_cols, k_op_cols<1, G, false><<<g.gN64, kBlock, 0, st>>>(d));
+    else DISPATCH_G(d.g_cols, k_op_cols<2, G, false><<<g.gN64, kBlock, 0, st>>>(d));
+  }
 }
 
 // The whole-chip form of the iteration's vector half (pcg.cu's cluster kernel where that does
@@ -1366,10 +1465,13 @@ __global__ void __launch_bounds__(256, kOpColsMinBlocks) k_op_cols(Dev d) {
 template <int ZM>
 __global__ void k_cg_update(Dev d, int npart) {
   __shared__ double sh[32];
+  __shared__ double s_alpha;
   if (d.sc->cg_done) return;
   const double pq = sum_pq_parts(d, npart, sh);
   const bool good = pq > 0.0 && isfinite(pq);      // else breakdown: keep the last iterate
-  const double alpha = good ? d.sc->rz / pq : 0.0;
+  if (threadIdx.x == 0) s_alpha = good ? d.sc->rz / pq : 0.0;
+  __syncthreads();
+  const double alpha = s_alpha;
   double rr = 0.0, rz = 0.0;
   if (good)
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < d.nsys; j += (int64_t)gridDim.x * blockDim.x) {
@@ -1707,6 +1809,9 @@ cudaError_t launch_cg_init(const Dev& d, const Geo& g, int precond, cudaStream_t
 cudaError_t launch_cg_body(const Dev& d, const Geo& g, int precond, cudaGraphConditionalHandle h, cudaStream_t st,
                            bool in_graph, bool lowp) {
   const bool tail = tail_runs(d, precond);
+  // one block an SM: every block adds up the parts of p^T q and one more tree of partial sums (the
+  // reduced storages keep the blocks their results are rounded by)
+  const int gU = d.storage == ST_F64 ? std::min(g.eN, d.sm_count > 0 ? d.sm_count : 148) : g.eN;
   int npart = g.gNc;
   if (lowp) {
     cudaError_t e = launch_op_lp(d, g, !tail, st);
@@ -1723,24 +1828,24 @@ cudaError_t launch_cg_body(const Dev& d, const Geo& g, int precond, cudaGraphCon
     if (d.runs) launch_op_rows_runs(d, g, 0, st);
     else if (d.nR) DISPATCH_G(d.g_rows, k_op_rows<0, G><<<g.gR64, kBlock, 0, st>>>(d));
     launch_lr(d, d.p, 0, st);
-    DISPATCH_G(d.g_cols, k_op_cols<0, G><<<g.gN64, kBlock, 0, st>>>(d));
-    npart = g.gN64;
+    launch_op_cols(d, g, 0, st);
+    npart = lr_alone(d) ? lr_blocks(d, g) : g.gN64;
   }
   if (tail) return launch_tail_iter(d, precond, npart, h, in_graph, st);
   if (precond == PC_BLOCK32) {
-    k_cg_update<2><<<g.eN, kBlock, 0, st>>>(d, npart);
+    k_cg_update<2><<<gU, kBlock, 0, st>>>(d, npart);
     launch_block_apply(d, 0, st);
   } else if (precond == PC_DENSE) {
-    k_cg_update<2><<<g.eN, kBlock, 0, st>>>(d, npart);
+    k_cg_update<2><<<gU, kBlock, 0, st>>>(d, npart);
     launch_trsv(d, 0, st);
   } else if (precond == PC_JACOBI_LR && d.m) {
-    k_cg_update<1><<<g.eN, kBlock, 0, st>>>(d, npart);
+    k_cg_update<1><<<gU, kBlock, 0, st>>>(d, npart);
     const int gs = (d.stiff_cap + 7) / 8;
     k_stiff_u<<<gs, kBlock, 0, st>>>(d, 0);
     k_stiff_t<<<gs, kBlock, 0, st>>>(d, 0);
     k_stiff_corr<<<g.eN, kBlock, 0, st>>>(d, 0);
   } else {
-    k_cg_update<0><<<g.eN, kBlock, 0, st>>>(d, npart);
+    k_cg_update<0><<<gU, kBlock, 0, st>>>(d, npart);
   }
   k_cg_p<<<g.eN, kBlock, 0, st>>>(d, h, in_graph ? 1 : 0);
   return cudaGetLastError();
@@ -1775,7 +1880,7 @@ cudaError_t launch_op_cols_only(const Dev& d, const Geo& g, cudaStream_t st) {
   // (the low-rank term uses us from the last launch_lr; the measurement does not re-run it)
   if (d.mx) return launch_op_cols_mx(d, g, 1, st);
   if (d.df) return launch_op_cols_df(d, g, 1, st);
-  DISPATCH_G(d.g_cols, k_op_cols<1, G><<<g.gN64, kBlock, 0, st>>>(d));
+  launch_op_cols(d, g, 1, st);
   return cudaGetLastError();
 }
 
@@ -1800,7 +1905,7 @@ cudaError_t launch_apply(const Dev& d, const Geo& g, cudaStream_t st) {
   if (d.runs && d.storage == ST_F64) launch_op_rows_runs(d, g, 1, st);
   else if (d.nR) DISPATCH_G(d.g_rows, k_op_rows<1, G><<<g.gR64, kBlock, 0, st>>>(d));
   launch_lr(d, d.p, 0, st);
-  DISPATCH_G(d.g_cols, k_op_cols<1, G><<<g.gN64, kBlock, 0, st>>>(d));
+  launch_op_cols(d, g, 1, st);
   return cudaGetLastError();
 }
 
@@ -1811,7 +1916,7 @@ cudaError_t launch_apply_ru(const Dev& d, const Geo& g, cudaStream_t st) {
   d2.p = d.dx;
   if (d.nR) DISPATCH_G(d.g_rows, k_op_rows<2, G><<<g.gR64, kBlock, 0, st>>>(d2));
   if (d.ucols) launch_lr(d2, d2.p, 0, st);
-  DISPATCH_G(d.g_cols, k_op_cols<2, G><<<g.gN64, kBlock, 0, st>>>(d2));
+  launch_op_cols(d2, g, 2, st);
   return cudaGetLastError();
 }
 
