@@ -42,6 +42,7 @@ struct Scal {
   double eta_asked;                  // tolerance asked for a single step, 0: the rule's
   // PCG
   double rz, pq, alpha, beta, rr, rhs2, tol2;
+  double rz_old;               // rz before the running iteration (k_cg_update -> k_cg_dir)
   int cg_iter, cg_done, cg_max, cg_conv;
   // preconditioner
   double stiff_gamma, stiff_thresh;
@@ -168,6 +169,31 @@ __device__ bool grid_reduce(const double (&v)[NQ], const int (&ops)[NQ], double*
   }
   if (threadIdx.x == 0) *ticket = 0u;
   return true;
+}
+
+// Sums of NQ <= 8 quantities over the kBlock threads of the block, valid in every thread.  The
+// float64 pipe takes a warp's addition in 64 cycles whatever its lanes carry, so the eight
+// warps' values are added through shared memory by one warp a quantity (the warps of different
+// quantities sit on different quarters of the SM) and only the last 32 by shuffles: 12 additions
+// one after the other against 2 x 5 + 3 x 5 in every warp.  sm: NQ * kBlock doubles.
+template <int NQ>
+__device__ __forceinline__ void block_sums(const double (&v)[NQ], double* sm, double (&out)[NQ]) {
+  __shared__ double s_out[NQ];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) sm[q * kBlock + threadIdx.x] = v[q];
+  __syncthreads();
+  if (wid < NQ) {
+    const double* p = sm + wid * kBlock + lane;
+    double t = p[0];
+#pragma unroll
+    for (int w = 1; w < kBlock / 32; ++w) t += p[32 * w];
+    t = warp_sum(t);
+    if (lane == 0) s_out[wid] = t;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) out[q] = s_out[q];
 }
 
 // Dot product of one CSR row with a dense vector, computed by one warp (all lanes return the

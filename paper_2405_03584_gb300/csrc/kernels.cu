@@ -181,7 +181,7 @@ cudaError_t launch_lr(const Dev& d, const double* v, int quad, cudaStream_t st) 
   if (!d.ucols) return cudaSuccess;
   if (d.ucols & 1) k_lr_part<false><<<d.ublocks, 256, 0, st>>>(d, v);
   else k_lr_part<true><<<d.ublocks, 256, 0, st>>>(d, v);
-  k_lr_final<<<(int)std::min<int64_t>((d.ucols + 7) / 8, 4096), 256, 0, st>>>(d, quad);
+  k_lr_final<<<(int)std::min<int64_t>(d.ucols, 4096), 32, 0, st>>>(d, quad);
   return cudaGetLastError();
 }
 
@@ -1463,34 +1463,60 @@ static void launch_op_cols(const Dev& d, const Geo& g, int mode, cudaStream_t st
 // ZM 0 (Jacobi): z = r / M, r^T z, beta.  ZM 1 (Jacobi + low rank): z0 = r / M only.
 // ZM 2 (dense): z is left to the dense apply.
 template <int ZM>
-__global__ void k_cg_update(Dev d, int npart) {
+__global__ void __launch_bounds__(256) k_cg_update(Dev d, int npart) {
+  __shared__ double sm[2 * kBlock];
   __shared__ double sh[32];
   __shared__ double s_alpha;
-  if (d.sc->cg_done) return;
-  const double pq = sum_pq_parts(d, npart, sh);
+  Scal* sc = d.sc;
+  if (sc->cg_done) return;
+  double t1[1] = {0.0}, pq1[1];
+  for (int b = threadIdx.x; b < npart; b += blockDim.x) t1[0] += __ldcg(d.partials + 16 * kMaxRedBlocks + b);
+  block_sums<1>(t1, sm, pq1);
+  const double pq = pq1[0];
   const bool good = pq > 0.0 && isfinite(pq);      // else breakdown: keep the last iterate
-  if (threadIdx.x == 0) s_alpha = good ? d.sc->rz / pq : 0.0;
+  if (threadIdx.x == 0) s_alpha = good ? sc->rz / pq : 0.0;
   __syncthreads();
   const double alpha = s_alpha;
   double rr = 0.0, rz = 0.0;
   if (good)
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < d.nsys; j += (int64_t)gridDim.x * blockDim.x) {
-    d.dx[j] = fma(alpha, d.p[j], d.dx[j]);
-    const double rj = fma(-alpha, d.q[j], d.r[j]);
-    d.r[j] = rj;
-    rr = fma(rj, rj, rr);
-    if (ZM < 2) {
-      const double zj = rj * d.Minv[j];
-      d.z[j] = zj;
-      rz = fma(rj, zj, rz);
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < d.nsys; j += (int64_t)gridDim.x * blockDim.x) {
+      d.dx[j] = fma(alpha, d.p[j], d.dx[j]);
+      const double rj = fma(-alpha, d.q[j], d.r[j]);
+      d.r[j] = rj;
+      rr = fma(rj, rj, rr);
+      if (ZM < 2) {
+        const double zj = rj * d.Minv[j];
+        d.z[j] = zj;
+        if (ZM == 0) rz = fma(rj, zj, rz);
+      }
     }
-  }
-  double v[2] = {rr, rz};
-  const int ops[2] = {0, 0};
-  double out[2];
-  if (grid_reduce<2>(v, ops, d.partials + 17 * kMaxRedBlocks, &d.sc->ticket[T_UPD], out, sh)) {
+  if (ZM == 0) {
+    // the parts of both sums are added up by every block of k_cg_dir, the next kernel
+    const double v[2] = {rr, rz};
+    double out[2];
+    block_sums<2>(v, sm, out);
     if (threadIdx.x == 0) {
-      Scal* sc = d.sc;
+      d.partials[17 * kMaxRedBlocks + blockIdx.x] = out[0];
+      d.partials[18 * kMaxRedBlocks + blockIdx.x] = out[1];
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      sc->pq = pq;
+      sc->alpha = alpha;
+      if (good) {
+        sc->cg_iter += 1;
+        sc->rz_old = sc->rz;
+      } else {
+        sc->cg_done = 1;
+        if (!isfinite(pq)) sc->status = DS_NUMERICAL;
+      }
+    }
+    return;
+  }
+  const double v[1] = {rr};
+  const int ops[1] = {0};
+  double out[1];
+  if (grid_reduce<1>(v, ops, d.partials + 17 * kMaxRedBlocks, &sc->ticket[T_UPD], out, sh)) {
+    if (threadIdx.x == 0) {
       sc->pq = pq;
       sc->alpha = alpha;
       if (!good) {
@@ -1509,10 +1535,51 @@ __global__ void k_cg_update(Dev d, int npart) {
       } else if (sc->cg_iter >= sc->cg_max) {
         sc->cg_done = 1;
       }
-      if (ZM == 0 && !sc->cg_done) {
-        sc->beta = out[1] / sc->rz;
-        sc->rz = out[1];
-      }
+    }
+  }
+}
+
+// After k_cg_update<0>: ||r||^2 and r^T z from its parts, the test, beta, and the next direction.
+// Every block adds up the parts and comes to the same decision; block 0 writes the scalars that
+// no other block reads here (n = 77373: 13.0 us for the two kernels; 16.4 us with a last-block
+// reduction and three shuffle trees in all warps of k_cg_update).
+__global__ void __launch_bounds__(256) k_cg_dir(Dev d, int npart, cudaGraphConditionalHandle h, int set_cond) {
+  __shared__ double sm[2 * kBlock];
+  __shared__ double s_beta;
+  Scal* sc = d.sc;
+  const bool first = blockIdx.x == 0 && threadIdx.x == 0;
+  if (sc->cg_done) {
+    if (set_cond && first) cudaGraphSetConditional(h, 0u);
+    return;
+  }
+  double v[2] = {0.0, 0.0}, out[2];
+  for (int b = threadIdx.x; b < npart; b += blockDim.x) {
+    v[0] += __ldcg(d.partials + 17 * kMaxRedBlocks + b);
+    v[1] += __ldcg(d.partials + 18 * kMaxRedBlocks + b);
+  }
+  block_sums<2>(v, sm, out);
+  const bool bad = !isfinite(out[0]), conv = out[0] <= sc->tol2;
+  const bool done = bad || conv || sc->cg_iter >= sc->cg_max;
+  if (threadIdx.x == 0) s_beta = out[1] / sc->rz_old;
+  __syncthreads();
+  const double beta = s_beta;
+  if (!done)
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < d.nsys; j += (int64_t)gridDim.x * blockDim.x) {
+      const double pj = fma(beta, d.p[j], d.z[j]);
+      d.p[j] = pj;
+      if (d.p32) d.p32[j] = (float)pj;
+      if (d.p_df && j < d.n) d.p_df[j] = df_split(pj);
+    }
+  if (first) {
+    if (set_cond) cudaGraphSetConditional(h, done ? 0u : 1u);
+    sc->rr = out[0];
+    if (bad) sc->status = DS_NUMERICAL;
+    if (!bad && conv) sc->cg_conv = 1;
+    if (done) {
+      sc->cg_done = 1;
+    } else {
+      sc->beta = beta;
+      sc->rz = out[1];
     }
   }
 }
@@ -1846,6 +1913,8 @@ cudaError_t launch_cg_body(const Dev& d, const Geo& g, int precond, cudaGraphCon
     k_stiff_corr<<<g.eN, kBlock, 0, st>>>(d, 0);
   } else {
     k_cg_update<0><<<gU, kBlock, 0, st>>>(d, npart);
+    k_cg_dir<<<gU, kBlock, 0, st>>>(d, gU, h, in_graph ? 1 : 0);
+    return cudaGetLastError();
   }
   k_cg_p<<<g.eN, kBlock, 0, st>>>(d, h, in_graph ? 1 : 0);
   return cudaGetLastError();
