@@ -444,13 +444,102 @@ __global__ void __launch_bounds__(256) k_chol_tile_inv(const float2* A, int64_t 
   for (int r = ty; r < kT; r += 8) tinv[(int64_t)blockIdx.x * kT * kT + r * kT + tx] = X[r][tx];
 }
 
-// Column c of A^{-1} = L^{-T} L^{-1} e_c (float64): forward sweep reads row p of the upper part
-// (= column p of L), backward sweep reads row q of L; both contiguous.  One block per column at
-// a time.
+// Column c of A^{-1} = L^{-T} L^{-1} e_c (float64) by one warp, nn <= 32 E: lane i holds rows
+// i, i + 32, ...; the forward sweep reads row p of the upper part (= column p of L), the backward
+// sweep row q of L, four rows fetched ahead of the four in work.  What bounds it is the chain of
+// 2 nn steps (multiply, shuffle, multiply-add), so nothing but registers is on it.  (A block per
+// column with the vector in shared memory, two barriers and a load from L2 in every step: 48 us
+// at n = 7001's interior point iterations, 25 us here.)
+constexpr int kInvMax = 256, kInvAhead = 4;
+template <int E>
+__device__ void inv_column(const double* A, int64_t ld, int nn, const double* rinv, double* Ainv, int64_t ldi, int c) {
+  const int lane = threadIdx.x & 31;
+  double y[E], ri[E], cur[kInvAhead][E], nxt[kInvAhead][E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int i = lane + 32 * e;
+    y[e] = i == c ? 1.0 : 0.0;
+    ri[e] = i < nn ? rinv[i] : 0.0;
+  }
+  auto fetch = [&](int p0) {
+#pragma unroll
+    for (int s = 0; s < kInvAhead; ++s)
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int p = p0 + s, i = lane + 32 * e;
+        nxt[s][e] = p >= 0 && p < nn && i < nn ? A[(int64_t)p * ld + i] : 0.0;
+      }
+  };
+  auto take = [&]() {
+#pragma unroll
+    for (int s = 0; s < kInvAhead; ++s)
+#pragma unroll
+      for (int e = 0; e < E; ++e) cur[s][e] = nxt[s][e];
+  };
+  fetch(c & ~(kInvAhead - 1));
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    if (32 * e + 32 <= c) continue;
+    for (int p0 = max(32 * e, c & ~(kInvAhead - 1)); p0 < min(32 * e + 32, nn); p0 += kInvAhead) {
+      take();
+      fetch(p0 + kInvAhead);
+#pragma unroll
+      for (int s = 0; s < kInvAhead; ++s) {
+        const int p = p0 + s;
+        if (p < c || p >= nn) continue;
+        const double m = y[e] * ri[e], yp = __shfl_sync(0xffffffffu, m, p & 31);
+        if (lane > (p & 31)) y[e] = fma(-cur[s][e], yp, y[e]);
+        else if (lane == (p & 31)) y[e] = yp;
+#pragma unroll
+        for (int f = e + 1; f < E; ++f) y[f] = fma(-cur[s][f], yp, y[f]);
+      }
+    }
+  }
+  const int last = (nn - 1) & ~(kInvAhead - 1);
+  fetch(last);
+#pragma unroll
+  for (int e = E - 1; e >= 0; --e) {
+    for (int q0 = min(32 * e + 32 - kInvAhead, last); q0 >= 32 * e; q0 -= kInvAhead) {
+      take();
+      fetch(q0 - kInvAhead);
+#pragma unroll
+      for (int s = kInvAhead - 1; s >= 0; --s) {
+        const int q = q0 + s;
+        if (q >= nn) continue;
+        const double m = y[e] * ri[e], xq = __shfl_sync(0xffffffffu, m, q & 31);
+        if (lane < (q & 31)) y[e] = fma(-cur[s][e], xq, y[e]);
+        else if (lane == (q & 31)) y[e] = xq;
+#pragma unroll
+        for (int f = 0; f < e; ++f) y[f] = fma(-cur[s][f], xq, y[f]);
+      }
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < E; ++e)
+    if (lane + 32 * e < nn) Ainv[(int64_t)(lane + 32 * e) * ldi + c] = y[e];
+}
+
+// A^{-1} for nn <= kInvMax, a block of one warp per column; larger ones are left to k_inv.  Each
+// warp runs the form with the fewest registers' worth of rows that hold nn.  The same numbers as
+// k_inv's, bit for bit.
+__global__ void __launch_bounds__(32) k_inv_small(const double* A, int64_t ld, const int* nn_dev, int nn_fixed,
+                                                  const double* rinv, double* Ainv, int64_t ldi) {
+  const int nn = dev_nn(nn_dev, nn_fixed);
+  if (nn > kInvMax) return;
+  for (int c = blockIdx.x; c < nn; c += gridDim.x) {
+    if (nn <= 32) inv_column<1>(A, ld, nn, rinv, Ainv, ldi, c);
+    else if (nn <= 64) inv_column<2>(A, ld, nn, rinv, Ainv, ldi, c);
+    else if (nn <= 128) inv_column<4>(A, ld, nn, rinv, Ainv, ldi, c);
+    else inv_column<8>(A, ld, nn, rinv, Ainv, ldi, c);
+  }
+}
+
+// The same for nn > kInvMax, one block per column at a time, two barriers a step.
 __global__ void k_inv(const double* A, int64_t ld, const int* nn_dev, int nn_fixed, const double* rinv, double* Ainv,
                       int64_t ldi) {
   extern __shared__ double y[];
   const int nn = nn_dev ? *nn_dev : nn_fixed;
+  if (nn <= kInvMax) return;
   for (int c = blockIdx.x; c < nn; c += gridDim.x) {
     for (int i = threadIdx.x; i < nn; i += blockDim.x) y[i] = (i == c) ? 1.0 : 0.0;
     __syncthreads();
@@ -795,7 +884,8 @@ cudaError_t launch_stiff_factor(const Dev& d, cudaStream_t st) {
   cudaError_t e = launch_chol<double>(d.G, cap, ns, 0, cap, d.chol_diag, d.chol_rinv, d.chol_tiles,
                                       &d.sc->chol_fail, st);
   if (e != cudaSuccess) return e;
-  k_inv<<<std::min(cap, 4 * 152), 256, rowbytes, st>>>(d.G, cap, ns, 0, d.chol_rinv, d.Ginv, cap);
+  k_inv_small<<<std::min(cap, kInvMax), 32, 0, st>>>(d.G, cap, ns, 0, d.chol_rinv, d.Ginv, cap);
+  if (cap > kInvMax) k_inv<<<std::min(cap, 4 * 152), 256, rowbytes, st>>>(d.G, cap, ns, 0, d.chol_rinv, d.Ginv, cap);
   return cudaGetLastError();
 }
 
