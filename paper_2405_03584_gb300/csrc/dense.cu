@@ -36,7 +36,12 @@ namespace ipmk {
 __device__ __forceinline__ double r_mul(double a, double b) { return a * b; }
 __device__ __forceinline__ double r_fms(double c, double a, double b) { return fma(-a, b, c); }   // c - a b
 __device__ __forceinline__ double r_rsqrt(double p) { return rsqrt(p); }
-__device__ __forceinline__ bool r_above(double a, double b) { return a > b; }
+// a > b for b > 0, by the order of the bits (a float64 comparison takes as long as a multiplication
+// and would lie on the chain from pivot to pivot); false where a or b is NaN.
+__device__ __forceinline__ bool r_above(double a, double b) {
+  const long long ia = __double_as_longlong(a);
+  return ia > __double_as_longlong(b) && ia <= 0x7ff0000000000000ll;
+}
 __device__ __forceinline__ double r_shfl(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
 __device__ __forceinline__ double r_to_double(double v) { return v; }
 __device__ __forceinline__ double r_floor(double fl) { return fl + 1e-300; }
@@ -114,10 +119,12 @@ __global__ void k_chol_save_diag(const R* A, int64_t ld, const int* nn_dev, int 
 // and factors it at once (pivot by shuffle, reciprocal square root, scaling), while the
 // other warps apply step k to the rest of the trailing block, the entries (i, j) with
 // k + 1 < j <= i.  Listed by j descending (then i), those are the first (30 - k)(31 - k) / 2
-// entries of one table of pairs, so the threads take them densely (one each with 512
-// threads) instead of one row per warp with most lanes idle.  (Measured on GB300: about
-// 20000 cycles per tile; a whole tile in one warp's registers, with no barrier, took 44000:
-// one warp then issues every multiply-add of the tile.)
+// entries of one table of pairs, so the threads take them densely instead of one row per warp
+// with most lanes idle.  Only warps of the other three quarters of the SM take part: every
+// float64 instruction holds its quarter's pipe for 64 cycles, and those of a warp beside warp 0
+// would hold up the chain.  (A tile with the rows below it 14.4 us; 12.5 us
+// so, with the floor's test on integers and one scaling a column.  A whole tile in one warp's registers, with no
+// barrier, takes twice as long: one warp then issues every multiply-add of the tile.)
 constexpr int kPanelThreads = 512;
 constexpr int kTriPairs = kT * (kT - 1) / 2;   // 496 pairs (i, j), 1 <= j <= i < 32
 
@@ -133,7 +140,8 @@ __device__ __forceinline__ R tile_column(R (*t)[kT + 1], R* rs, R x, R flc, int 
     if (nfloor && lane == 0) atomicAdd(nfloor, 1);
   }
   const R r = r_rsqrt(piv);
-  const R col = lane == c ? r_mul(piv, r) : (lane > c ? r_mul(x, r) : r_const<R>(0.0));
+  const R m = r_mul(lane == c ? piv : x, r);
+  const R col = lane >= c ? m : r_const<R>(0.0);
   if (lane >= c) t[lane][c] = col;
   if (lane == c) rs[c] = r;
   return col;
@@ -169,9 +177,9 @@ __device__ void tile_potrf(R (*t)[kT + 1], R* rs, const R* A, int64_t ld, int nn
       const R lck = r_shfl(colk, c);           // L_ck
       if (tx >= c) x = r_fms(x, colk, lck);    // step k on column c
       colk = tile_column<R>(t, rs, x, r_shfl(fl, c), c, base + c < nn, nfloor);
-    } else {
+    } else if (ty & 3) {
       const int cnt = (kT - 2 - k) * (kT - 1 - k) / 2;
-      for (int e = threadIdx.x - 32; e < cnt; e += blockDim.x - 32) {
+      for (int e = (ty - 1 - (ty >> 2)) * 32 + tx; e < cnt; e += kPanelThreads * 3 / 4) {
         const int i = pairs[e] / kT, j = pairs[e] % kT;
         t[i][j] = r_fms(t[i][j], t[i][k], t[j][k]);
       }
