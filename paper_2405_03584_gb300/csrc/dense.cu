@@ -122,8 +122,8 @@ __global__ void k_chol_save_diag(const R* A, int64_t ld, const int* nn_dev, int 
 // entries of one table of pairs, so the threads take them densely instead of one row per warp
 // with most lanes idle.  Only warps of the other three quarters of the SM take part: every
 // float64 instruction holds its quarter's pipe for 64 cycles, and those of a warp beside warp 0
-// would hold up the chain.  (A tile with the rows below it 14.4 us; 12.5 us
-// so, with the floor's test on integers and one scaling a column.  A whole tile in one warp's registers, with no
+// would hold up the chain.  (A tile with the rows below it 14.4 us; 12.5 us so, with the floor's
+// test on integers and one scaling a column.  A whole tile in one warp's registers, with no
 // barrier, takes twice as long: one warp then issues every multiply-add of the tile.)
 constexpr int kPanelThreads = 512;
 constexpr int kTriPairs = kT * (kT - 1) / 2;   // 496 pairs (i, j), 1 <= j <= i < 32

@@ -342,7 +342,7 @@ __device__ void cons_resid(const Dev& d, double* part, int b, int nb) {
 // neighbouring threads.  The two dot products share one tree (each half of a group carries one
 // of them after the first exchange).  The maxima are reduced as integers.  n = 7001 at 16 lanes:
 // 31 us as one kernel of one-lane epilogues and twelve float64 block reductions (and 7 us for
-// the constraint rows), 11 us now for both.
+// the constraint rows), 9.8 us for both so.
 template <int G>
 __global__ void __launch_bounds__(256, 4) k_cols_resid(Dev d, double* part, int gcols) {
   if ((int)blockIdx.x >= gcols) {
@@ -457,7 +457,8 @@ static __device__ void control_step(const Dev& d, double cg_rel, cudaGraphCondit
 // All its quotients are formed by one division, a lane each.
 // MODE RSM_START: also the complementarity mean (the start points' mu); RSM_CONTROL: also the
 // iteration's control step.  (24.6 us with every thread over all 19 quantities in turn and one
-// thread's chain of nine divisions, plus 4.4 us and a launch for the control; 5 us now.)
+// thread's chain of nine divisions, plus 4.4 us and a launch for the control; 5 us so, 8 to 12 us
+// with the control step.)
 constexpr int kFinalThreads = 640;
 template <int MODE>
 __global__ void __launch_bounds__(kFinalThreads) k_resid_final(Dev d, int gR, int gM, int gN, const double* part,

@@ -12,22 +12,23 @@
 // however many lanes it serves: an instruction that every warp of a block executes for a value
 // they all share costs more than a barrier.  As separate kernels (update, A_s z, G^{-1} u,
 // correction, p), each with its own last-block sum, the half took 27 us an iteration at n =
-// 1500 and 30 us at n = 50000.  One thread-block cluster runs it instead: its CTAs are resident
-// together, so a global sum is one exchange through distributed shared memory and one cluster
-// barrier, the vectors stay in registers from the update to the new p, and the loads of a phase
-// are issued before the barrier that precedes it.  Scalars are formed by one warp and handed
+// 1500 and 30 us at n = 50000 (9.9 us and 20.8 us here).  One thread-block cluster runs it
+// instead: its CTAs are resident together, so a global sum is one exchange through distributed
+// shared memory and one cluster barrier, the vectors stay in registers from the update to the
+// new p, and the loads of a phase are issued before the barrier that precedes it.  Scalars are formed by one warp and handed
 // out through shared memory; warps without unknowns skip the vector arithmetic; the trees of a
 // sum are formed from shared memory by 8 lanes per 32 values (6 float64 instructions for four
 // trees a warp, against 20 by shuffles alone).
 //
-// Every sum that feeds the iteration (p^T q, r^T z, the stiff rows' products) has the order of
-// the whole-chip kernels (blocks of 256 values as warp trees, then the blocks' parts as one
-// such block), so which of the two forms runs does not show in the result, bit for bit; only
-// ||r||^2, which is compared with tolerances alone, is added in an order of its own.
+// Every sum that feeds the iteration (p^T q, r^T z, the stiff rows' products) has one fixed order
+// (blocks of 256 values as warp trees, then the blocks' parts as one such block) for every shape
+// of the cluster, so the shape does not show in the result, bit for bit; only ||r||^2, which is
+// compared with tolerances alone, is added in an order of its own.
 //
 // One cluster of 16 SMs streams about 2 TB/s and has a tenth of the chip's float64 rate, so
-// the kernel stops paying where the vectors outgrow it: tail_runs() declines above kTailMaxN
-// unknowns and the caller takes the whole-chip kernels.
+// the kernel stops paying where the vectors outgrow it: above kTailMaxN unknowns (kTailPlainN
+// without the stiff rows' correction) tail_runs() declines and the caller takes the whole-chip
+// kernels.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -38,14 +39,18 @@ namespace ipmk {
 
 namespace {
 
-#ifndef IPM_TAIL_SMALL
-#define IPM_TAIL_SMALL 512
-#endif
 constexpr int kTailThreads = 512;
 constexpr int kTailWarps = kTailThreads / 32;
 constexpr int kTailCtas = 16;          // CTAs of the largest cluster (16 needs the non-portable opt-in)
+constexpr int64_t kTailSmall = 512;    // unknowns up to which the cluster has 8 CTAs
 constexpr int kTailMaxE = 7;           // unknowns per thread
 constexpr int64_t kTailMaxN = (int64_t)kTailCtas * kTailThreads * kTailMaxE;
+// Without the stiff rows' correction the whole-chip form is two kernels, and the shorter one from
+// about 20000 unknowns on: whole solves with H's low-rank term alone take 3.33 ms by the cluster
+// and 3.43 by the chip at n = 16384, 3.54 and 3.44 at 24000, 3.92 and 3.68 at 45000 (with the
+// correction it is five, and the cluster the shorter one at every size it holds).  The reduced
+// storages stay with the cluster: their results are rounded by its sums.
+constexpr int64_t kTailPlainN = (int64_t)kTailCtas * kTailThreads * 2;
 constexpr int kStiffCapMax = 1024;     // options.stiff_max's limit
 constexpr int kPre = 8;                // entries per lane fetched before a barrier
 
@@ -590,8 +595,9 @@ cudaError_t allow_e() {
 }
 
 // CTAs of the cluster: a small problem's barriers are cheaper among fewer CTAs, and a small
-// cluster finds room beside other solves sooner.
-int tail_ctas(int64_t nsys) { return nsys <= IPM_TAIL_SMALL ? 8 : 16; }
+// cluster finds room beside other solves sooner (with 512 unknowns each of 8 CTAs still has a
+// thread for every one of its own).
+int tail_ctas(int64_t nsys) { return nsys <= kTailSmall ? 8 : 16; }
 
 cudaError_t launch_tail(const Dev& d, int precond, int mode, int npart, cudaGraphConditionalHandle h, bool set_cond,
                         cudaStream_t st) {
@@ -613,7 +619,9 @@ cudaError_t launch_tail(const Dev& d, int precond, int mode, int npart, cudaGrap
 }  // namespace
 
 bool tail_runs(const Dev& d, int precond) {
-  return (precond == PC_JACOBI || precond == PC_JACOBI_LR) && d.nsys <= kTailMaxN;
+  if (precond != PC_JACOBI && precond != PC_JACOBI_LR) return false;
+  const bool lr = precond == PC_JACOBI_LR && d.m > 0;
+  return d.nsys <= (lr || d.storage != ST_F64 ? kTailMaxN : kTailPlainN);
 }
 
 cudaError_t prepare_tail() {

@@ -2,7 +2,8 @@
 splits change, against the oracle's formulas with the problem's matrices kept sparse.
 
 * the iteration's vector half: one cluster of 8 or 16 blocks with 1, 2, 4 or 7 unknowns a
-  thread (512 threads a block) up to 57344 unknowns, whole-chip kernels beyond;
+  thread (512 threads a block) up to 57344 unknowns (16384 without the stiff rows' correction),
+  whole-chip kernels beyond;
 * the low-rank correction by m stiff rows: chosen, ordered, their Gram matrix factored and
   inverted (a warp a column up to 256 rows, a block a column beyond), rows longer than 256
   entries;
