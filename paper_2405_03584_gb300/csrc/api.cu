@@ -2278,6 +2278,11 @@ static void batch_free(ipm_batch* b) {
 
 extern "C" {
 
+// Solves in one launch beyond which each takes the whole-chip form of the PCG's vector half: a
+// cluster of 16 SMs waits for room beside that many others, and holds it while it waits at its
+// barriers (F32, n = 12000: 20 solves 56.0 ms by clusters and 45.1 by the chip; n = 20000: 30
+// solves 125 and 99; 64 QPs of 2000 to 40000: 58.9 and 62.5 solves/s; up to 12 the clusters win or tie).
+constexpr int kCrowd = 12;
 int ipm_batch_create(ipm_handle* const* handles, int count, int flags, ipm_batch** out) {
   if (!handles || count < 1 || !out || flags != IPM_COLD) return IPM_ERR_ARG;
   *out = nullptr;
@@ -2312,7 +2317,9 @@ int ipm_batch_create(ipm_handle* const* handles, int count, int flags, ipm_batch
     e = cudaStreamWaitEvent(h->st, b->fork, 0);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->d.sc, h->hs, sizeof(Scal), cudaMemcpyHostToDevice, h->st);
     gr.solve_c[0] = LoopCounts{};
+    h->d.crowd = count > kCrowd ? 1 : 0;
     if (e == cudaSuccess) e = emit_solve(h, pc, false, h->st, &gr.solve_c[0]);
+    h->d.crowd = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->hs, h->d.sc, sizeof(Scal), cudaMemcpyDeviceToHost, h->st);
     if (e == cudaSuccess && h->trace_cap)
       e = cudaMemcpyAsync(h->htrace, h->d.trace, sizeof(double) * kTraceCols * (size_t)h->trace_cap,

@@ -928,7 +928,7 @@ __device__ __forceinline__ int half_octave(double y) {
 template <int G>
 __global__ void k_stiff_select(Dev d) {
   __shared__ unsigned int h[kHistBins];
-  __shared__ int list[2048];
+  __shared__ int list[1024];                       // stiff_max's limit
   __shared__ int s_cnt;
   __shared__ double s_thr;
   __shared__ bool s_last;
@@ -987,11 +987,11 @@ __global__ void k_stiff_select(Dev d) {
     const int32_t k = __ldcg(&d.cand[i]);
     if (__ldcg(&d.ratio[k]) >= thr) {
       const int at = atomicAdd(&s_cnt, 1);
-      if (at < 2048) list[at] = k;
+      if (at < 1024) list[at] = k;
     }
   }
   __syncthreads();
-  const int total = min(s_cnt, 2048), ns = min(total, d.stiff_cap);
+  const int total = min(s_cnt, 1024), ns = min(total, d.stiff_cap);
   for (int i = tid; i < total; i += blockDim.x) {
     const int k = list[i];
     int rank = 0;
@@ -1468,15 +1468,20 @@ static void launch_op_cols(const Dev& d, const Geo& g, int mode, cudaStream_t st
 // ZM 2 (dense): z is left to the dense apply.
 template <int ZM>
 __global__ void __launch_bounds__(256) k_cg_update(Dev d, int npart) {
-  __shared__ double sm[2 * kBlock];
+  __shared__ double sm[ZM == 0 ? 2 * kBlock : 1];
   __shared__ double sh[32];
   __shared__ double s_alpha;
   Scal* sc = d.sc;
   if (sc->cg_done) return;
-  double t1[1] = {0.0}, pq1[1];
-  for (int b = threadIdx.x; b < npart; b += blockDim.x) t1[0] += __ldcg(d.partials + 16 * kMaxRedBlocks + b);
-  block_sums<1>(t1, sm, pq1);
-  const double pq = pq1[0];
+  double pq;
+  if (ZM == 0) {
+    double t1[1] = {0.0}, pq1[1];
+    for (int b = threadIdx.x; b < npart; b += blockDim.x) t1[0] += __ldcg(d.partials + 16 * kMaxRedBlocks + b);
+    block_sums<1>(t1, sm, pq1);
+    pq = pq1[0];
+  } else {
+    pq = sum_pq_parts(d, npart, sh);   // the cluster kernel's order: either form gives the same bits
+  }
   const bool good = pq > 0.0 && isfinite(pq);      // else breakdown: keep the last iterate
   if (threadIdx.x == 0) s_alpha = good ? sc->rz / pq : 0.0;
   __syncthreads();
@@ -2165,8 +2170,16 @@ cudaError_t launch_dense_build(const Dev& d, cudaStream_t st);       // dense.cu
 cudaError_t launch_stiff_factor(const Dev& d, cudaStream_t st);      // dense.cu
 
 cudaError_t prepare_steps() {
-  return cudaFuncSetAttribute(k_gram_G, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              kGramSlots * 8 * kGramEntries * 6);
+  cudaError_t e = cudaFuncSetAttribute(k_gram_G, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       kGramSlots * 8 * kGramEntries * 6);
+  // Shared memory (percent) for two blocks an SM, not for all that fit: an SM changes its split of
+  // L1 and shared memory only when idle, so beside other solves the split of one kernel stays for
+  // all, and the operator passes live on their L1 (64 QPs in one launch: 49.0 solves/s with the
+  // default, 62.5 with one block's share, 63.1 with two; alone one block's share costs 4 us in 15).
+  constexpr int kGramCarveout = 44;
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_gram_G, cudaFuncAttributePreferredSharedMemoryCarveout, kGramCarveout);
+  return e;
 }
 
 // Before the right-hand side: stiff-row selection (JACOBI_LR).

@@ -580,6 +580,9 @@ cudaError_t allow_mode() {
   cudaError_t e = cudaSuccess;
   auto one = [&](auto* f) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    // one CTA an SM: no more shared memory taken from the L1 than it needs (see k_gram_G's)
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxL1);
   };
   one(k_pcg_tail<E, LR, TAIL_ITER>);
   one(k_pcg_tail<E, LR, TAIL_INIT>);
@@ -621,6 +624,7 @@ cudaError_t launch_tail(const Dev& d, int precond, int mode, int npart, cudaGrap
 bool tail_runs(const Dev& d, int precond) {
   if (precond != PC_JACOBI && precond != PC_JACOBI_LR) return false;
   const bool lr = precond == PC_JACOBI_LR && d.m > 0;
+  if (d.crowd && lr) return false;
   return d.nsys <= (lr || d.storage != ST_F64 ? kTailMaxN : kTailPlainN);
 }
 

@@ -15,6 +15,7 @@ struct Dev {
   int64_t n, m, nR;            // variables, constraint rows, rows of R = [F; A_csr]
   int64_t nsys;                // PCG unknowns: n (condensed system), n + m (doubly augmented)
   int aug;                     // 1: PCG on the doubly augmented system (Section 4, eq:2x2_augmented)
+  int crowd;                   // captured beside many other solves: see ipm_batch_create
   int64_t nnzR, nnzHs;
   int g_rows, g_cols;          // lanes per row of the kernels over R and over R^T (4, 8, 16, 32)
   int g_at;                    // lanes per row of the kernels over A^T alone

@@ -11,7 +11,8 @@ splits change, against the oracle's formulas with the problem's matrices kept sp
   time, alone (its own column kernel) and beside matrix rows;
 * the triangular solves of the dense preconditioner, in blocks of 32 with the rows of a block
   two to a thread, even and odd sizes;
-* the limit on PCG iterations with two iterations per pass of the loop.
+* the limit on PCG iterations with two iterations per pass of the loop;
+* many solves in one launch.
 
 A Newton direction is taken at eta = 1e-9: PCG stops at a residual of 1e-9 ||rhs|| by its own
 recursion, and the true residual of the returned step may differ from the recursion's by what
@@ -136,3 +137,24 @@ def test_iteration_limit(limit):
         s.set_iterate(x, sl, y, zl, zu, MU)
         rep = s.newton_direction(eta=1e-14)["report"]
     assert rep["iters"] == limit and rep["converged"] == 0
+
+
+# more than 12 solves in one launch take the whole-chip form of the vector half
+@pytest.mark.parametrize("storage", ["f64", "f32"])
+def test_many_solves_in_one_launch(storage):
+    """13 uneven QPs in one launch give each member the bits of its solve alone."""
+    solvers, ref = [], []
+    for i in range(13):
+        p = W.rt_qp(n=200 + 37 * i, seed=60 + i, density=0.02, n_organ=60 + 5 * i)
+        s = ipm.Solver(precond="jacobi_lr", storage=storage)
+        s.set_qp_rt(p)
+        assert s.solve() == ipm.IPM_OK
+        ref.append(s.get()["x"])
+        solvers.append(s)
+    b = ipm.Batch(solvers)
+    assert b.solve() == [ipm.IPM_OK] * 13
+    for s, x in zip(solvers, ref):
+        assert np.array_equal(s.get()["x"], x)
+    b.close()
+    for s in solvers:
+        s.close()
