@@ -8,12 +8,12 @@
 // recovery -> ratio test -> update -> residual summary -> mu test / stop rule (which sets the
 // outer condition and appends a trace row).  The host launches the graph and waits once.
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <chrono>
 #include <map>
 #include <memory>
 #include <mutex>
-#include <tuple>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -447,10 +447,11 @@ int operator_group(double avg_nnz, int64_t rows, bool columns) {
   return g;
 }
 
-// Autotuner results per matrix signature (n, rows of R, non-zeros), process-wide, so that a
-// QP loaded again in the same process runs the same schedule (and gives the same bits).
+// Autotuner results, process-wide, so that a QP loaded again in the same process runs the same
+// schedule (and gives the same bits).  The key is everything that picks the timed kernels or
+// their work: sizes, non-zeros of R and Hs, columns of U, storage, arithmetic and formats.
 std::mutex g_tune_mu;
-std::map<std::tuple<int64_t, int64_t, int64_t>, std::pair<int, int>> g_tune_cache;
+std::map<std::array<int64_t, 8>, std::pair<int, int>> g_tune_cache;
 
 // Operator formats decided once R and R^T are on the device: the double-float copies of the
 // values (asked for by options.op_arith, kept only when every value is in the float32 range
@@ -675,9 +676,12 @@ int prepare_block_segments(ipm_handle* h, const std::vector<int64_t>& Rp, const 
 
 // Times the two operator kernels for every lane-group size on the loaded matrices (three
 // launches each after one warm-up, CUDA events on the handle's stream) and keeps the fastest.
+// Where H has the low-rank term alone the column pass has one width only (k_op_cols_lr): timing
+// it would let noise pick the width of the other column kernels, so load_qp's choice stays.
 int autotune_groups(ipm_handle* h) {
   Dev& d = h->d;
-  const auto key = std::make_tuple(d.n, d.nR, d.nnzR);
+  const std::array<int64_t, 8> key = {d.n,     d.nR,      d.nnzR, d.nnzHs,
+                                      d.ucols, d.storage, d.df + 2 * d.mx + 4 * d.runs + 8 * d.gap, d.aug};
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune_cache.find(key);
@@ -701,7 +705,7 @@ int autotune_groups(ipm_handle* h) {
   CUDA_TRY(h, cudaEventCreate(&e1));
   const int cand[4] = {4, 8, 16, 32};
   for (int which = 0; which < 2; ++which) {
-    if (which == 0 && d.nR == 0) continue;
+    if (which == 0 ? d.nR == 0 : lr_alone(d)) continue;
     float best = 1e30f;
     int bestg = which == 0 ? d.g_rows : d.g_cols;
     for (int gsz : cand) {

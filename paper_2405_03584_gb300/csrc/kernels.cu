@@ -1435,10 +1435,6 @@ __global__ void __launch_bounds__(256, kOpColsMinBlocks) k_op_cols_lr(Dev d) {
   if (MODE == 0) store_pq_part(d, pq, sh);
 }
 
-static bool lr_alone(const Dev& d) {
-  return d.storage == ST_F64 && d.ucols && !(d.ucols & 1) && !d.nnzR && !d.Hs_ptr && !d.aug;
-}
-
 // Its blocks: as many tiles each as the most loaded block of a resident wave has, on fewer blocks.
 static int lr_blocks(const Dev& d, const Geo& g) {
   const int64_t tiles = (d.n + kLrTile - 1) / kLrTile, each = (tiles + g.gN64 - 1) / g.gN64;

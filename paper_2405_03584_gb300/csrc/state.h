@@ -339,6 +339,11 @@ cudaError_t launch_update(const Dev& d, const Geo& g, cudaStream_t st);
 cudaError_t launch_apply(const Dev& d, const Geo& g, cudaStream_t st);
 // ---- the two operator kernels alone (measurement) ----
 cudaError_t launch_op_rows_only(const Dev& d, const Geo& g, cudaStream_t st);
+// H has the low-rank term alone, in float64 and with an even number of columns: the column pass
+// is a kernel of its own (k_op_cols_lr), with the same lanes whatever g_cols is
+inline bool lr_alone(const Dev& d) {
+  return d.storage == ST_F64 && d.ucols && !(d.ucols & 1) && !d.nnzR && !d.Hs_ptr && !d.aug && !d.df && !d.mx;
+}
 cudaError_t launch_op_cols_only(const Dev& d, const Geo& g, cudaStream_t st);
 // ---- full Jacobi diagonal into Minv's storage as M (not inverted) ----
 cudaError_t launch_jacobi_full(const Dev& d, const Geo& g, double* out, cudaStream_t st);
