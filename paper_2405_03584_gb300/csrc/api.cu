@@ -429,21 +429,31 @@ int heuristic_group(double avg_nnz) {
   return g;
 }
 
-// The same for the float64 operator passes, measured on GB300 at every width over RT, dense and
-// VMAT-shaped matrices.  Two costs pull apart: a row's sum takes log2 G float64 instructions a
+// The same for the float64 operator passes, measured on GB300 at every width over RT, dense, wide
+// and VMAT-shaped matrices.  Two costs pull apart: a row's sum takes log2 G float64 instructions a
 // warp (each holds a quarter of an SM for 64 cycles), and few rows times few lanes leave the
-// chip without loads in flight.
-//  * rows of R (many, short): 4 lanes up to 64 entries (n = 7001, 42 a row: 7.4 us at 4, 8.0 at
-//    8, 10.9 at 16), 8 beyond (RT n = 50000, 250 a row: 141 us at 4, 121 at 8, 143 at 16; VMAT
-//    134 a row: 37.6, 31.9, 35.2);
-//  * columns (few, long): 16 lanes from 32 entries (n = 7001, 168 a column: 13.0 us at 4, 8.4 at
-//    8, 8.3 at 16, 11.7 at 32; n = 50000, 1000 a column: 207, 137, 123, 149), else 8;
-//  * so few rows that 32768 lanes are not reached: wider while 8 entries a lane remain (dense n =
-//    500, m = 1000: rows 13.8 us at 8, 5.8 at 32; columns 17.0 at 16, 12.9 at 32).
+// chip without loads in flight.  In us at 4 / 8 / 16 / 32 lanes:
+//  * rows of R (many, short): 4 lanes up to 112 entries (n = 7001, 42 a row: 7.4, 8.0, 10.9, -; 40000
+//    rows of 100: 17, 18, 25, 33), 8 beyond (RT n = 50000, 250 a row: 141, 121, 143, -; VMAT 134 a
+//    row: 38, 32, 35, -);
+//  * columns (few, long): 16 lanes from 160 entries (n = 7001, 168 a column: 13.0, 8.4, 8.3, 11.7; n =
+//    50000, 1000 a column: 207, 137, 123, 149), 8 from 80 (20000 columns of 100: 13.1, 12.6, 15.2,
+//    20.7), else 4 (50000 columns of 50: 13.5, 16.4, 22.7, 33.1);
+//  * so few that 32768 lanes are not reached: wider while 8 entries a lane remain, columns up to 16
+//    lanes while 2 remain (dense n = 500, m = 1000: rows 20.7, 14.2, 10.1, 8.1; 1500 columns of 36: 8.4,
+//    8.2, 7.6, 8.1);
+//  * so few that 98304 are not reached: wider while 16 entries a lane remain (4096 rows of 2048: 128,
+//    82, 47, 29, its columns 189, 96, 52, 31; 8192 rows of 512: 34, 25, 18, 19, its 4096 columns of 1024:
+//    85, 43, 25, 21; 16000 rows of 500 are enough at 8: 49, 31, 34, 30).
 // Reduced storages keep heuristic_group's widths: their float32 sums depend on it.
 int operator_group(double avg_nnz, int64_t rows, bool columns) {
-  int g = columns ? (avg_nnz >= 32.0 ? 16 : 8) : (avg_nnz > 64.0 ? 8 : 4);
-  while (g < 32 && rows * g < 32768 && avg_nnz >= 16.0 * g) g *= 2;
+  int g = columns ? (avg_nnz >= 160.0 ? 16 : (avg_nnz >= 80.0 ? 8 : 4)) : (avg_nnz > 112.0 ? 8 : 4);
+  while (g < 32) {
+    const int64_t lanes = rows * g;
+    const double left = avg_nnz / (2 * g);       // entries a lane at twice the width
+    if (!(lanes < 32768 && left >= (columns && g < 16 ? 2.0 : 8.0)) && !(lanes < 98304 && left >= 16.0)) break;
+    g *= 2;
+  }
   return g;
 }
 
