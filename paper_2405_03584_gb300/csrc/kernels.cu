@@ -80,7 +80,9 @@ Geo make_geo(const Dev& d) {
 // threads load neighbouring ones) and walks every rg-th row of its block's chunk, rg = 256 / ceil(ucols / 8) rows of
 // threads side by side: of 256 threads 250 carry columns at 200 columns, where 32 lanes over
 // 128-column slices carried 200 of 256 values, and every float64 instruction of a warp costs the
-// same.  (n = 77373, 200 columns: 41 us before.)
+// same.  (n = 77373, 200 columns: 41 us before.)  The rg partial sums of a column are added by as
+// many threads as there are for it: by one thread a column they were a serial chain of 256 at up to
+// 8 columns (both kernels at n = 20000, 7 columns: 20.9 -> 15.0 us; n = 1000, one column: 20.9 -> 10.8).
 constexpr int kLrCols = 8;
 constexpr int kLrTile = kBlock / 4;              // rows of U a block of the column pass takes at a time
 constexpr int kLrSlice = 256 * kLrCols;          // columns a block covers at a time
@@ -148,12 +150,17 @@ __global__ void __launch_bounds__(256) k_lr_part(Dev d, const double* __restrict
 #pragma unroll
     for (int k = 0; k < kLrCols; ++k) sh[tid][k] = acc[k];
     __syncthreads();
-    for (int t = tid; t < w; t += 256) {
+    // column t by L neighbouring threads (L w <= 256), then a tree over them
+    const int L = nch > 16 ? 1 : 1 << (31 - __clz(32 / nch));
+    for (int t = tid / L; t - (tid & 31) / L < w; t += 256 / L) {   // whole warps: the shuffles need them
       // the thread and accumulator of column t
       const int i = VEC ? t / 2 : t, th = i % nch, k = VEC ? 2 * (i / nch) + (t & 1) : i / nch;
       double s = 0.0;
-      for (int q = 0; q < rg; ++q) s += sh[q * nch + th][k];
-      d.upart[(r0 + t) * (int64_t)d.ublocks + blockIdx.x] = s;   // column-major: the final sum reads runs
+      if (t < w)
+        for (int q = tid & (L - 1); q < rg; q += L) s += sh[q * nch + th][k];
+      for (int o = L / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (t < w && (tid & (L - 1)) == 0)
+        d.upart[(r0 + t) * (int64_t)d.ublocks + blockIdx.x] = s;   // column-major: the final sum reads runs
     }
     __syncthreads();
   }
