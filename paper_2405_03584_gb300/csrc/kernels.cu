@@ -1348,7 +1348,7 @@ cudaError_t launch_op_rows_runs(const Dev& d, const Geo& g, int mode, cudaStream
 // MODE 0: inside PCG; MODE 1: a single operator apply (no scalars touched); MODE 2: as 1,
 // when the reduced-precision PCG asks for a residual replacement.
 // EXT: with any of a sparse block of H, the low-rank term and the augmented system; without, the
-// pass keeps its registers for the loads (six blocks an SM allow 40; with them 24 bytes spill).
+// pass keeps its registers for the loads (six blocks an SM allow 40; no form spills).
 // The block's 256 / G variables are finished by that many neighbouring threads: the last
 // float64 instructions of a variable cost a warp the same for one lane as for 32 (n = 50000,
 // 49.9 million entries: 132 -> 119 us with both; the entries' multiply-adds alone take 84 us of
@@ -1372,7 +1372,7 @@ __global__ void __launch_bounds__(256, kOpColsMinBlocks) k_op_cols(Dev d) {
       const int64_t hb = ok ? d.Hs_ptr[j] : 0, he = ok ? d.Hs_ptr[j + 1] : 0;
       acc += group_row_dot<G, false>(hb, he, gl, d.Hs_idx, d.Hs_val, d.p);
     }
-    if (EXT && d.ucols) acc += lr_row<G>(d, j, ok, gl);
+    if (EXT && d.ucols) acc += lr_row<G, true>(d, j, ok, gl);
     if (gl == 0) st[buf][tid / G] = acc;
     __syncthreads();
     const int64_t jj = j0 + tid;

@@ -132,10 +132,34 @@ struct Dev {
 // An even column count makes every row start on 16 bytes: two columns a load then, of U and of
 // the weights alike (the loads' issue slots, not their bytes, held this pass at twice the
 // float64 pipe's time).
-template <int G>
+// LEAN: two accumulators instead of four, for k_op_cols with its 40 registers a thread (six blocks an
+// SM): with four it spilled 16 to 108 bytes (-Xptxas -v), with two it spills none (VMAT column pass
+// 41.1 -> 38.4 us, n = 77373 with 33 columns 20.7 -> 15.9).  The reduced storages' column pass spills
+// too (28 to 136 bytes), but there the loads in flight are worth more: n = 20000, 200 columns, F32
+// 37 us with four, 52 with two.
+template <int G, bool LEAN = false>
 __device__ __forceinline__ double lr_row(const Dev& d, const int64_t j, const bool ok, const int gl) {
   double a = 0.0;
-  if (ok) {
+  if (LEAN) {
+    if (ok) {
+      const double* row = d.U + j * d.ucols;
+      const int uc = (int)d.ucols;
+      double a1 = 0.0;
+      if ((uc & 1) == 0) {
+#pragma unroll 2
+        for (int v = 2 * gl; v < uc; v += 2 * G) {
+          const double2 u = __ldg(reinterpret_cast<const double2*>(row + v));
+          const double2 s = __ldg(reinterpret_cast<const double2*>(d.lrs + v));
+          a = fma(u.x, s.x, a);
+          a1 = fma(u.y, s.y, a1);
+        }
+      } else {
+#pragma unroll 2
+        for (int r = gl; r < uc; r += G) a = fma(__ldg(row + r), __ldg(d.lrs + r), a);
+      }
+      a += a1;
+    }
+  } else if (ok) {
     const double* row = d.U + j * d.ucols;
     double a1 = 0.0, a2 = 0.0, a3 = 0.0;
     if ((d.ucols & 1) == 0) {
