@@ -2297,11 +2297,24 @@ static void batch_free(ipm_batch* b) {
 
 extern "C" {
 
-// Solves in one launch beyond which each takes the whole-chip form of the PCG's vector half: a
-// cluster of 16 SMs waits for room beside that many others, and holds it while it waits at its
-// barriers (F32, n = 12000: 20 solves 56.0 ms by clusters and 45.1 by the chip; n = 20000: 30
-// solves 125 and 99; 64 QPs of 2000 to 40000: 58.9 and 62.5 solves/s; up to 12 the clusters win or tie).
-constexpr int kCrowd = 12;
+// Solves in one launch beyond which a condensed system's PCG takes the whole-chip form of its vector
+// half (more kernels, the same bits): a CTA of the cluster kernel takes all registers of an SM, so
+// a cluster waits for 16 SMs without a block of another solve, and holds them while it waits at
+// its barriers.  By clusters / by the chip, ms, with the stiff rows' correction:
+//   n = 1500, F64   8: 8.5 / 9.9   12: 10.0 / 10.7   16: 11.9 / 11.4   20: 14.4 / 12.4
+//   n = 3000, F64   8: 11.0 / 12.1   12: 14.0 / 13.9   16: 17.7 / 15.6
+//   n = 5000, F64   8: 17.3 / 17.6   10: 20.3 / 19.4   12: 23.7 / 21.5
+//   n = 12000, F64  6: 27.8 / 28.6   8: 35.0 / 33.9   10: 42.8 / 39.5   12: 51.2 / 45.5
+//   n = 12000, F32  6: 29.5 / 31.4   8: 36.5 / 36.5   10: 44.6 / 41.9   12: 52.4 / 47.1
+//   n = 30000, F64  6: 68.4 / 67.1   8: 89.4 / 85.0   12: 132.6 / 123.2
+// and without it, where that form is shorter:
+//   n = 1500, F64   16: 1.7 / 1.9   20: 2.0 / 2.0      n = 3000, F64   12: 2.0 / 2.0   16: 2.5 / 2.3
+//   n = 12000, F64  8: 5.9 / 5.7   12: 8.7 / 8.1       n = 12000, F32  8: 5.7 / 5.8   12: 8.5 / 7.9
+// (64 QPs of 2000 to 40000, F32: 58.9 solves/s by clusters and 62.5 by the chip.)
+static int crowd_limit(const Dev& d, int pc) {
+  if (d.nsys > 4096) return 8;
+  return d.nsys <= 2048 && !(pc == PC_JACOBI_LR && d.m > 0) ? 20 : 12;
+}
 int ipm_batch_create(ipm_handle* const* handles, int count, int flags, ipm_batch** out) {
   if (!handles || count < 1 || !out || flags != IPM_COLD) return IPM_ERR_ARG;
   *out = nullptr;
@@ -2336,7 +2349,7 @@ int ipm_batch_create(ipm_handle* const* handles, int count, int flags, ipm_batch
     e = cudaStreamWaitEvent(h->st, b->fork, 0);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->d.sc, h->hs, sizeof(Scal), cudaMemcpyHostToDevice, h->st);
     gr.solve_c[0] = LoopCounts{};
-    h->d.crowd = count > kCrowd ? 1 : 0;
+    h->d.crowd = count > crowd_limit(h->d, pc) ? 1 : 0;
     if (e == cudaSuccess) e = emit_solve(h, pc, false, h->st, &gr.solve_c[0]);
     h->d.crowd = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->hs, h->d.sc, sizeof(Scal), cudaMemcpyDeviceToHost, h->st);

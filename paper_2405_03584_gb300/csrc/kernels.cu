@@ -1465,7 +1465,7 @@ static void launch_op_cols(const Dev& d, const Geo& g, int mode, cudaStream_t st
 }
 
 // The whole-chip form of the iteration's vector half (pcg.cu's cluster kernel where that does
-// not run: BLOCK32 and DENSE preconditioners, systems beyond its size).
+// not run: BLOCK32 and DENSE preconditioners, systems beyond its size, batches of many solves).
 // alpha = rz / p^T q (npart block parts); dx += alpha p; r -= alpha q; ||r||^2 -> convergence test.
 // ZM 0 (Jacobi): z = r / M, r^T z, beta.  ZM 1 (Jacobi + low rank): z0 = r / M only.
 // ZM 2 (dense): z is left to the dense apply.
@@ -1922,6 +1922,10 @@ cudaError_t launch_cg_body(const Dev& d, const Geo& g, int precond, cudaGraphCon
     const int gs = (d.stiff_cap + 7) / 8;
     k_stiff_u<<<gs, kBlock, 0, st>>>(d, 0);
     k_stiff_t<<<gs, kBlock, 0, st>>>(d, 0);
+    k_stiff_corr<<<g.eN, kBlock, 0, st>>>(d, 0);
+  } else if (d.crowd && !d.aug) {
+    // in a crowded batch for the cluster kernel: its order of r^T z, so its bits (no stiff rows here)
+    k_cg_update<1><<<gU, kBlock, 0, st>>>(d, npart);
     k_stiff_corr<<<g.eN, kBlock, 0, st>>>(d, 0);
   } else {
     k_cg_update<0><<<gU, kBlock, 0, st>>>(d, npart);

@@ -624,7 +624,7 @@ cudaError_t launch_tail(const Dev& d, int precond, int mode, int npart, cudaGrap
 bool tail_runs(const Dev& d, int precond) {
   if (precond != PC_JACOBI && precond != PC_JACOBI_LR) return false;
   const bool lr = precond == PC_JACOBI_LR && d.m > 0;
-  if (d.crowd && lr) return false;
+  if (d.crowd && !d.aug) return false;
   return d.nsys <= (lr || d.storage != ST_F64 ? kTailMaxN : kTailPlainN);
 }
 
