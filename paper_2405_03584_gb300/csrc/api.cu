@@ -17,6 +17,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <initializer_list>
 #include <new>
 #include <string>
 #include <thread>
@@ -355,18 +356,30 @@ int dev_alloc(ipm_handle* h, void** p, size_t bytes, const char* what) {
   return IPM_OK;
 }
 
-// Pinned buffers: the trace rows copied back after each solve, and a stage that holds the largest
-// stretch of results a call copies out at once (rd .. dzu).
+// Vectors of host calls up to these sizes go through the pinned stage (vectors_out, apply_kkt).  A copy
+// into pageable memory is synchronous and takes 10 to 12 us whatever its size; through the stage a
+// vector costs its bytes at 22 GB/s, the plain copy that follows (three vectors of 32 / 64 / 96 / 128
+// KB: 45 / 45 / 44 / 46 us by pageable copies, 35 / 42 / 47 / 54 through the stage; one vector of 16 /
+// 64 / 256 KB: 12.7 / 13.6 / 14.8 and 12.4 / 16.0 / 28.7; an operand on its way in: n = 16000 / 32000
+// applications 63 / 74 us by pageable copies, 56 / 78 through the stage).
+constexpr size_t kStageVec = 64 << 10;     // one of several vectors of a call
+constexpr size_t kStageOne = 16 << 10;     // a call's only vector
+constexpr size_t kStageIn = 128 << 10;     // an operand
+constexpr size_t kStageGap = 16 << 10;     // staged vectors this close in the arena come in one copy
+
+// Pinned buffers: the trace rows copied back after each solve, and the stage: no more than five
+// staged vectors, the scalars and the gaps between them.
 int alloc_trace(ipm_handle* h) {
   h->trace_cap = h->opt.max_ipm;
   const size_t tb = sizeof(double) * kTraceCols * (size_t)h->trace_cap;
   const Dev& d = h->d;
   const size_t step = (size_t)((const char*)(d.dzu + d.n) - (const char*)d.rd);
   const size_t iter = (size_t)((const char*)(d.zu + d.n) - (const char*)d.x);
-  if (cudaMallocHost(&h->htrace, tb + std::max(step, iter)) != cudaSuccess) {
+  const size_t stage = std::min(std::max(step, iter), 5 * kStageVec + 6 * kStageGap + sizeof(Scal));
+  if (cudaMallocHost(&h->htrace, tb + stage) != cudaSuccess) {
     cudaGetLastError();
     h->htrace = nullptr;
-    return fail(h, IPM_ERR_OOM, "pinned trace buffer");
+    return fail(h, IPM_ERR_OOM, "pinned trace and result buffers");
   }
   h->stage = (char*)h->htrace + tb;
   return IPM_OK;
@@ -1083,33 +1096,56 @@ int copy_in(ipm_handle* h, double* dst, const double* src, int64_t n, int mem) {
   return IPM_OK;
 }
 
-// Results for host memory go through the pinned stage: one copy of a stretch of the arena, one
-// synchronisation, then plain copies to the caller's arrays.  (A copy into pageable memory is
-// staged by the runtime, one at a time and synchronously: five of them and two of the scalars were
-// 100 us of a Newton step at n = 24.)
-struct Staged {
-  const char* begin;
-  char* at;
+// Results for host memory: the requested vectors, in the order they lie in the arena, and (scal) the
+// device scalars into h->hs.  Small ones go through the pinned stage, neighbours in one copy; large
+// ones straight to the caller.  One synchronisation; done on return.
+struct OutVec {
+  double* dst;
+  const double* src;
+  int64_t n;
 };
-int stage_out(ipm_handle* h, const void* begin, const void* end, size_t offset, Staged* s) {
-  s->begin = (const char*)begin;
-  s->at = h->stage + offset;
-  CUDA_TRY(h, cudaMemcpyAsync(s->at, begin, (size_t)((const char*)end - (const char*)begin), cudaMemcpyDeviceToHost, h->st));
+int vectors_out(ipm_handle* h, std::initializer_list<OutVec> vecs, bool scal) {
+  struct Part {
+    const char* src;
+    void* dst;
+    size_t bytes, at;
+  };
+  Part parts[8];
+  int np = 0;
+  auto add = [&](const void* src, void* dst, size_t bytes) {
+    int i = np++;
+    for (; i > 0 && parts[i - 1].src > (const char*)src; --i) parts[i] = parts[i - 1];
+    parts[i] = {(const char*)src, dst, bytes, 0};
+  };
+  int asked = scal ? 1 : 0;
+  for (const OutVec& v : vecs) asked += v.dst && v.n > 0 ? 1 : 0;
+  const size_t limit = asked > 1 ? kStageVec : kStageOne;
+  for (const OutVec& v : vecs)
+    if (v.dst && v.n > 0 && sizeof(double) * (size_t)v.n <= limit) add(v.src, v.dst, sizeof(double) * (size_t)v.n);
+  if (scal) add(h->d.sc, h->hs, sizeof(Scal));
+  size_t used = 0;
+  for (int i = 0; i < np;) {                 // runs of staged parts
+    const char* beg = parts[i].src;
+    const char* end = beg;
+    for (; i < np && (size_t)(parts[i].src - end) <= kStageGap; ++i) {
+      parts[i].at = used + (size_t)(parts[i].src - beg);
+      end = parts[i].src + parts[i].bytes;
+    }
+    CUDA_TRY(h, cudaMemcpyAsync(h->stage + used, beg, (size_t)(end - beg), cudaMemcpyDeviceToHost, h->st));
+    used += (size_t)(end - beg);
+  }
+  for (const OutVec& v : vecs) {
+    if (!v.dst || v.n <= 0 || sizeof(double) * (size_t)v.n <= limit) continue;
+    CUDA_TRY(h, cudaMemcpyAsync(v.dst, v.src, sizeof(double) * (size_t)v.n, cudaMemcpyDeviceToHost, h->st));
+  }
+  CUDA_TRY(h, cudaStreamSynchronize(h->st));
+  for (int i = 0; i < np; ++i) std::memcpy(parts[i].dst, h->stage + parts[i].at, parts[i].bytes);
   return IPM_OK;
-}
-void unstage(const Staged& s, double* dst, const double* src, int64_t n) {
-  if (dst && n > 0) std::memcpy(dst, s.at + ((const char*)src - s.begin), sizeof(double) * (size_t)n);
 }
 
 // One vector to the caller; host memory: done on return.
 int copy_vector_out(ipm_handle* h, double* dst, const double* src, int64_t n, int mem) {
-  if (mem != IPM_MEM_HOST) return copy_out(h, dst, src, n, mem);
-  Staged t;
-  int rc;
-  if ((rc = stage_out(h, src, src + n, 0, &t))) return rc;
-  CUDA_TRY(h, cudaStreamSynchronize(h->st));
-  unstage(t, dst, src, n);
-  return IPM_OK;
+  return mem == IPM_MEM_HOST ? vectors_out(h, {{dst, src, n}}, false) : copy_out(h, dst, src, n, mem);
 }
 
 // Scalar fields of the device struct (written from the host between graph launches).
@@ -2044,23 +2080,16 @@ int ipm_get_xyz(ipm_handle* h, double* x, double* y, double* zl, double* zu, dou
   if ((rc = enter(h, stream))) return rc;
   const Dev& d = h->d;
   if (mem == IPM_MEM_HOST) {
-    Staged t;
-    if ((rc = stage_out(h, d.x, d.zu + d.n, 0, &t))) return rc;
-    CUDA_TRY(h, cudaStreamSynchronize(h->st));
-    unstage(t, x, d.x, d.n);
-    unstage(t, zl, d.zl, d.n);
-    unstage(t, zu, d.zu, d.n);
-    if (!h->stacked) {
-      unstage(t, y, d.y, d.m);
-      unstage(t, s, d.s, d.m);
-    }
+    const int64_t m1 = h->stacked ? 0 : d.m;   // two-sided rows: below
+    if ((rc = vectors_out(h, {{x, d.x, d.n}, {s, d.s, m1}, {y, d.y, m1}, {zl, d.zl, d.n}, {zu, d.zu, d.n}}, false)))
+      return rc;
   } else {
     if ((rc = copy_out(h, x, d.x, d.n, mem))) return rc;
     if ((rc = copy_out(h, zl, d.zl, d.n, mem))) return rc;
     if ((rc = copy_out(h, zu, d.zu, d.n, mem))) return rc;
   }
   if (!h->stacked && mem == IPM_MEM_HOST) {
-    // unstaged above
+    // copied above
   } else if (!h->stacked) {
     if ((rc = copy_out(h, y, d.y, d.m, mem))) return rc;
     if ((rc = copy_out(h, s, d.s, d.m, mem))) return rc;
@@ -2145,15 +2174,8 @@ int ipm_residuals(ipm_handle* h, double* rd, double* rp, double* rs, double* rl,
   // complementarity residuals into scratch vectors (ds: r_s, dzl: r_l, dzu: r_u)
   CUDA_TRY(h, launch_comp_resid(d, h->g, h->st));
   if (mem == IPM_MEM_HOST) {
-    Staged t;
-    if ((rc = stage_out(h, d.rd, d.dzu + d.n, 0, &t))) return rc;
-    CUDA_TRY(h, cudaStreamSynchronize(h->st));
-    unstage(t, rd, d.rd, d.n);
-    unstage(t, rp, d.rp, d.m);
-    unstage(t, rs, d.ds, d.m);
-    unstage(t, rl, d.dzl, d.n);
-    unstage(t, ru, d.dzu, d.n);
-    std::memcpy(h->hs, t.at + ((const char*)d.sc - t.begin), sizeof(Scal));
+    if ((rc = vectors_out(h, {{rd, d.rd, d.n}, {rp, d.rp, d.m}, {rs, d.ds, d.m}, {rl, d.dzl, d.n}, {ru, d.dzu, d.n}}, true)))
+      return rc;
   } else {
     if ((rc = copy_out(h, rd, d.rd, d.n, mem))) return rc;
     if ((rc = copy_out(h, rp, d.rp, d.m, mem))) return rc;
@@ -2179,7 +2201,7 @@ int ipm_apply_kkt(ipm_handle* h, const double* p, double* q, int mem, void* stre
   if ((rc = enter(h, stream))) return rc;
   const Dev& d = h->d;
   CUDA_TRY(h, launch_diag_update(d, h->g, h->st));
-  if (mem == IPM_MEM_HOST) {
+  if (mem == IPM_MEM_HOST && sizeof(double) * (size_t)d.n <= kStageIn) {
     std::memcpy(h->stage, p, sizeof(double) * (size_t)d.n);
     CUDA_TRY(h, cudaMemcpyAsync(d.p, h->stage, sizeof(double) * (size_t)d.n, cudaMemcpyHostToDevice, h->st));
   } else if ((rc = copy_in(h, d.p, p, d.n, mem))) {
@@ -2216,15 +2238,8 @@ int ipm_newton_direction(ipm_handle* h, double eta, double* dx, double* ds, doub
   CUDA_TRY(h, launch_ask_eta(d, eta > 0 ? eta : 0.0, h->st));
   CUDA_TRY(h, cudaGraphLaunch(h->graphs[h->precond].dir, h->st));
   if (mem == IPM_MEM_HOST) {
-    Staged t;
-    if ((rc = stage_out(h, d.sc, d.dzu + d.n, 0, &t))) return rc;
-    CUDA_TRY(h, cudaStreamSynchronize(h->st));
-    unstage(t, dx, d.dx, d.n);
-    unstage(t, ds, d.ds, d.m);
-    unstage(t, dy, d.dy, d.m);
-    unstage(t, dzl, d.dzl, d.n);
-    unstage(t, dzu, d.dzu, d.n);
-    std::memcpy(h->hs, t.at, sizeof(Scal));
+    if ((rc = vectors_out(h, {{dx, d.dx, d.n}, {ds, d.ds, d.m}, {dy, d.dy, d.m}, {dzl, d.dzl, d.n}, {dzu, d.dzu, d.n}}, true)))
+      return rc;
   } else {
     if ((rc = copy_out(h, dx, d.dx, d.n, mem))) return rc;
     if ((rc = copy_out(h, ds, d.ds, d.m, mem))) return rc;
