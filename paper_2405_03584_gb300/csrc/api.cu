@@ -1241,7 +1241,7 @@ int ipm_create(const ipm_options* opt, ipm_handle** out) {
     delete h;
     return IPM_ERR_CUDA;
   }
-  if (prepare_tail() != cudaSuccess || prepare_steps() != cudaSuccess) {   // per device: cheap to set again
+  if (prepare_steps() != cudaSuccess) {   // per device: cheap to set again
     cudaGetLastError();
     ipm_destroy(h);
     return IPM_ERR_CUDA;
@@ -1641,6 +1641,7 @@ static int load_qp(ipm_handle* h, const ipm_qp* qp, int64_t m_ar, void* stream) 
   h->loaded = true;
   h->have_iterate = false;
   h->precond = choose_precond(h);
+  h->d.cluster = tail_places(h->d, h->precond) ? 1 : 0;
   h->info = ipm_info{};
   return leave(h, stream);
 }
@@ -1881,6 +1882,7 @@ int ipm_share_qp(ipm_handle* h, ipm_handle* src, void* stream) {
   h->loaded = true;
   h->have_iterate = false;
   h->precond = choose_precond(h);
+  h->d.cluster = tail_places(h->d, h->precond) ? 1 : 0;
   h->info = ipm_info{};
   return leave(h, stream);
 }

@@ -27,8 +27,8 @@
 //
 // One cluster of 16 SMs streams about 2 TB/s and has a tenth of the chip's float64 rate, so
 // the kernel stops paying where the vectors outgrow it: above kTailMaxN unknowns (kTailPlainN
-// without the stiff rows' correction) tail_runs() declines and the caller takes the whole-chip
-// kernels.
+// without the stiff rows' correction), and where the device has no room for such a cluster,
+// tail_runs() declines and the caller takes the whole-chip kernels.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -548,20 +548,41 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_pcg_tail(Dev d, int npart, 
   }
 }
 
-template <int E, bool LR, int MODE>
-cudaError_t launch_one(const Dev& d, int ctas, int npart, cudaGraphConditionalHandle h, int set_cond, cudaStream_t st) {
+// A cluster of `ctas` CTAs; the attribute lives as long as the configuration is used.
+cudaLaunchConfig_t tail_config(int ctas, cudaStream_t st, cudaLaunchAttribute* at) {
   cudaLaunchConfig_t c{};
   c.gridDim = dim3((unsigned)ctas);
   c.blockDim = dim3(kTailThreads);
   c.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)ctas;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = (unsigned)ctas;
+  at->val.clusterDim.y = 1;
+  at->val.clusterDim.z = 1;
   c.attrs = at;
   c.numAttrs = 1;
+  return c;
+}
+
+template <int E, bool LR, int MODE>
+cudaError_t launch_one(const Dev& d, int ctas, int npart, cudaGraphConditionalHandle h, int set_cond, cudaStream_t st) {
+  cudaLaunchAttribute at;
+  const cudaLaunchConfig_t c = tail_config(ctas, st, &at);
   return cudaLaunchKernelEx(&c, k_pcg_tail<E, LR, MODE>, d, npart, h, set_cond);
+}
+
+// Sets a form's attributes on the current device and asks whether a cluster of it finds room there.
+template <int E, bool LR, int MODE>
+bool places_one(int ctas) {
+  auto* f = k_pcg_tail<E, LR, MODE>;
+  cudaLaunchAttribute at;
+  const cudaLaunchConfig_t c = tail_config(ctas, 0, &at);
+  int clusters = 0;
+  const bool ok = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                  // one CTA an SM: no more shared memory taken from the L1 than it needs (see k_gram_G's)
+                  cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxL1) == cudaSuccess &&
+                  cudaOccupancyMaxActiveClusters(&clusters, f, &c) == cudaSuccess;
+  if (!ok) cudaGetLastError();
+  return ok && clusters > 0;
 }
 
 template <int E, bool LR>
@@ -575,65 +596,53 @@ cudaError_t launch_mode(const Dev& d, int mode, int ctas, int npart, cudaGraphCo
   }
 }
 
-template <int E, bool LR>
-cudaError_t allow_mode() {
-  cudaError_t e = cudaSuccess;
-  auto one = [&](auto* f) {
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    // one CTA an SM: no more shared memory taken from the L1 than it needs (see k_gram_G's)
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxL1);
-  };
-  one(k_pcg_tail<E, LR, TAIL_ITER>);
-  one(k_pcg_tail<E, LR, TAIL_INIT>);
-  one(k_pcg_tail<E, LR, TAIL_RU>);
-  one(k_pcg_tail<E, LR, TAIL_RU2>);
-  return e;
-}
-
-template <int E>
-cudaError_t allow_e() {
-  const cudaError_t e = allow_mode<E, false>();
-  return e == cudaSuccess ? allow_mode<E, true>() : e;
-}
-
 // CTAs of the cluster: a small problem's barriers are cheaper among fewer CTAs, and a small
 // cluster finds room beside other solves sooner (with 512 unknowns each of 8 CTAs still has a
 // thread for every one of its own).
 int tail_ctas(int64_t nsys) { return nsys <= kTailSmall ? 8 : 16; }
 
-cudaError_t launch_tail(const Dev& d, int precond, int mode, int npart, cudaGraphConditionalHandle h, bool set_cond,
-                        cudaStream_t st) {
+// f(integral_constant E, bool_constant LR, CTAs) for the form that covers a system.
+template <typename F>
+auto tail_form(const Dev& d, int precond, F f) {
   const int ctas = tail_ctas(d.nsys);
   const int64_t cta_n = ((d.nsys + ctas - 1) / ctas + 255) & ~(int64_t)255;
   const int64_t per = (cta_n + kTailThreads - 1) / kTailThreads;
   const bool lr = precond == PC_JACOBI_LR && d.m > 0;
-  auto go = [&](auto ec) -> cudaError_t {
-    constexpr int E = decltype(ec)::value;
-    return lr ? launch_mode<E, true>(d, mode, ctas, npart, h, set_cond ? 1 : 0, st)
-              : launch_mode<E, false>(d, mode, ctas, npart, h, set_cond ? 1 : 0, st);
-  };
+  auto go = [&](auto ec) { return lr ? f(ec, std::true_type{}, ctas) : f(ec, std::false_type{}, ctas); };
   if (per <= 1) return go(std::integral_constant<int, 1>{});
   if (per <= 2) return go(std::integral_constant<int, 2>{});
   if (per <= 4) return go(std::integral_constant<int, 4>{});
   return go(std::integral_constant<int, kTailMaxE>{});
 }
 
-}  // namespace
+cudaError_t launch_tail(const Dev& d, int precond, int mode, int npart, cudaGraphConditionalHandle h, bool set_cond,
+                        cudaStream_t st) {
+  return tail_form(d, precond, [&](auto ec, auto lr, int ctas) {
+    return launch_mode<decltype(ec)::value, decltype(lr)::value>(d, mode, ctas, npart, h, set_cond ? 1 : 0, st);
+  });
+}
 
-bool tail_runs(const Dev& d, int precond) {
+// The cluster form covers a system of this size and preconditioner.
+bool tail_covers(const Dev& d, int precond) {
   if (precond != PC_JACOBI && precond != PC_JACOBI_LR) return false;
   const bool lr = precond == PC_JACOBI_LR && d.m > 0;
-  if (d.crowd && !d.aug) return false;
   return d.nsys <= (lr || d.storage != ST_F64 ? kTailMaxN : kTailPlainN);
 }
 
-cudaError_t prepare_tail() {
-  cudaError_t e = allow_e<1>();
-  if (e == cudaSuccess) e = allow_e<2>();
-  if (e == cudaSuccess) e = allow_e<4>();
-  if (e == cudaSuccess) e = allow_e<kTailMaxE>();
-  return e;
+}  // namespace
+
+bool tail_runs(const Dev& d, int precond) { return d.cluster && !(d.crowd && !d.aug) && tail_covers(d, precond); }
+
+// 16 SMs of one processing cluster are not a given: a process may be confined to fewer, and then every
+// launch would fail where the whole-chip kernels run.
+bool tail_places(const Dev& d, int precond) {
+  if (!tail_covers(d, precond)) return false;
+  return tail_form(d, precond, [&](auto ec, auto lr, int ctas) {
+    constexpr int E = decltype(ec)::value;
+    constexpr bool LR = decltype(lr)::value;
+    return places_one<E, LR, TAIL_ITER>(ctas) && places_one<E, LR, TAIL_INIT>(ctas) &&
+           (d.storage == ST_F64 || (places_one<E, LR, TAIL_RU>(ctas) && places_one<E, LR, TAIL_RU2>(ctas)));
+  });
 }
 
 cudaError_t launch_tail_init(const Dev& d, int precond, cudaGraphConditionalHandle h, cudaStream_t st) {

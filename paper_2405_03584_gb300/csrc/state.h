@@ -16,6 +16,7 @@ struct Dev {
   int64_t nsys;                // PCG unknowns: n (condensed system), n + m (doubly augmented)
   int aug;                     // 1: PCG on the doubly augmented system (Section 4, eq:2x2_augmented)
   int crowd;                   // captured beside many other solves: see ipm_batch_create
+  int cluster;                 // the device has room for the cluster kernel's form for this system
   int64_t nnzR, nnzHs;
   int g_rows, g_cols;          // lanes per row of the kernels over R and over R^T (4, 8, 16, 32)
   int g_at;                    // lanes per row of the kernels over A^T alone
@@ -311,9 +312,9 @@ cudaError_t launch_cg_init(const Dev& d, const Geo& g, int precond, cudaStream_t
 cudaError_t launch_cg_body(const Dev& d, const Geo& g, int precond, cudaGraphConditionalHandle h, cudaStream_t st,
                            bool in_graph = true, bool lowp = false);
 // ---- the vector half of a PCG iteration as one cluster kernel (pcg.cu) ----
-bool tail_runs(const Dev& d, int precond);   // the cluster kernel covers this system
-cudaError_t prepare_tail();                  // kernel attributes, per device
-cudaError_t prepare_steps();                 // the same for kernels.cu
+bool tail_runs(const Dev& d, int precond);   // the cluster kernel takes this system (Dev::cluster and its size)
+bool tail_places(const Dev& d, int precond); // sets its attributes and asks the device for room: Dev::cluster
+cudaError_t prepare_steps();                 // kernel attributes of kernels.cu, per device
 cudaError_t launch_tail_init(const Dev& d, int precond, cudaGraphConditionalHandle h, cudaStream_t st);
 cudaError_t launch_tail_iter(const Dev& d, int precond, int npart, cudaGraphConditionalHandle h, bool in_graph,
                              cudaStream_t st);
