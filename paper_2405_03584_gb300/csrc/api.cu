@@ -1931,7 +1931,7 @@ static int solve_launch(ipm_handle* h, int flags, int64_t* direct_launches) {
   return IPM_OK;
 }
 
-static int fill_info(ipm_handle* h, int64_t direct_launches);
+static int fill_info(ipm_handle* h, int64_t direct_launches, const LoopCounts& lc);
 
 // Waits for the launched solve (bounded by timeout_ms) and fills h->info and h->trace.
 static int solve_collect(ipm_handle* h, int64_t direct_launches) {
@@ -1951,16 +1951,16 @@ static int solve_collect(ipm_handle* h, int64_t direct_launches) {
   } else {
     CUDA_TRY(h, cudaEventSynchronize(h->ev));
   }
-  return fill_info(h, direct_launches);
+  return fill_info(h, direct_launches, h->graphs[h->pending_pc].solve_c[h->pending_warm ? 1 : 0]);
 }
 
-// Result bookkeeping after a finished solve: info from the pinned scalars and trace rows.
-static int fill_info(ipm_handle* h, int64_t direct_launches) {
+// Result bookkeeping after a finished solve: info from the pinned scalars and trace rows, launches from
+// the counts of the graph that ran (lc).
+static int fill_info(ipm_handle* h, int64_t direct_launches, const LoopCounts& lc) {
   const auto t0 = h->t_launch;
   h->pending = 0;
   const Scal& s = *h->hs;
   const int pc = h->pending_pc;
-  const LoopCounts& lc = h->graphs[pc].solve_c[h->pending_warm ? 1 : 0];
   const int rows = std::min(s.trace_rows, h->trace_cap);
   h->trace.assign(h->htrace, h->htrace + (size_t)rows * kTraceCols);
   int64_t launches = direct_launches;
@@ -2296,6 +2296,7 @@ int ipm_step_lengths(ipm_handle* h, const double* dx, const double* ds, const do
 struct ipm_batch {
   std::vector<ipm_handle*> hs;
   std::vector<uint64_t> gens;       // each member's ipm_handle::gen when the graph was captured
+  std::vector<LoopCounts> counts;   // launches of each member's branch (a crowded one runs other kernels than alone)
   cudaStream_t st = nullptr;
   cudaEvent_t ev = nullptr, fork = nullptr;
   std::vector<cudaEvent_t> join;
@@ -2345,6 +2346,7 @@ int ipm_batch_create(ipm_handle* const* handles, int count, int flags, ipm_batch
   b->hs.assign(handles, handles + count);
   for (int i = 0; i < count; ++i) b->gens.push_back(handles[i]->gen);
   b->join.assign(count, nullptr);
+  b->counts.assign(count, LoopCounts{});
   auto bad = [&](ipm_handle* h, const std::string& m) {
     if (h) h->err = m;
     cudaGetLastError();
@@ -2362,12 +2364,10 @@ int ipm_batch_create(ipm_handle* const* handles, int count, int flags, ipm_batch
   for (int i = 0; i < count && e == cudaSuccess; ++i) {
     ipm_handle* h = b->hs[i];
     const int pc = h->precond;
-    Graphs& gr = h->graphs[pc];
     e = cudaStreamWaitEvent(h->st, b->fork, 0);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->d.sc, h->hs, sizeof(Scal), cudaMemcpyHostToDevice, h->st);
-    gr.solve_c[0] = LoopCounts{};
     h->d.crowd = count > crowd_limit(h->d, pc) ? 1 : 0;
-    if (e == cudaSuccess) e = emit_solve(h, pc, false, h->st, &gr.solve_c[0]);
+    if (e == cudaSuccess) e = emit_solve(h, pc, false, h->st, &b->counts[i]);
     h->d.crowd = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(h->hs, h->d.sc, sizeof(Scal), cudaMemcpyDeviceToHost, h->st);
     if (e == cudaSuccess && h->trace_cap)
@@ -2416,7 +2416,7 @@ int ipm_batch_solve(ipm_batch* b, void* stream, int* statuses) {
     h->pending_pc = h->precond;
     h->pending_warm = 0;
     h->t_launch = t0;
-    const int st = fill_info(h, 0);
+    const int st = fill_info(h, 0, b->counts[i]);
     if (statuses) statuses[i] = st;
     if (st != IPM_OK && worst == IPM_OK) worst = st;
   }

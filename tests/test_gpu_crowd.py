@@ -64,3 +64,26 @@ def test_same_bits_as_alone(precond, count, n, storage):
     b.close()
     for s in solvers:
         s.close()
+
+
+def test_launch_counts():
+    """A member's kernel_launches are those of the graph that ran: its own, or the batch's branch."""
+    p = W.rt_qp(n=4400, density=0.003, seed=5)
+    solvers = [ipm.Solver(precond="jacobi_lr") for _ in range(9)]
+    for s in solvers:
+        s.set_qp_rt(p)
+    launches = lambda: [s.info()["kernel_launches"] for s in solvers]
+    solvers[0].solve()
+    alone = solvers[0].info()["kernel_launches"]
+    b = ipm.Batch(solvers)
+    b.solve()
+    crowded = launches()
+    assert len(set(crowded)) == 1 and crowded[0] > alone      # the whole-chip form has more launches
+    for s in solvers:
+        s.solve()
+    assert launches() == [alone] * 9
+    b.solve()
+    assert launches() == crowded
+    b.close()
+    for s in solvers:
+        s.close()
