@@ -14,6 +14,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "order_bits.h"
+
 namespace ipmk {
 
 constexpr int kWarp = 32;
@@ -28,7 +30,6 @@ constexpr int kBlock = 256;          // threads per block of the streaming kerne
 constexpr int kOpRowsMinBlocks = IPM_OP_ROWS_MINB;
 constexpr int kOpColsMinBlocks = IPM_OP_COLS_MINB;
 constexpr int kMaxRedBlocks = 2048;  // upper bound of blocks that write reduction partials
-constexpr long long kInfBits = 0x7ff0000000000000ll;   // INFINITY's bits
 constexpr int kHistBins = 64;        // stiff-row ratio histogram bins (two per octave)
 
 // Device scalars of one handle.
@@ -66,7 +67,7 @@ struct Scal {
   int refine_total, max_cg_step, trace_rows, trace_cap;
   // step
   double alpha_p, alpha_d;
-  long long step_min[2];             // least ratios of the step's ratio test (bits; primal, dual)
+  long long step_min[2];             // least ratios of the step's ratio test (min_key; primal, dual)
   // residual summary at the current iterate (written by k_resid_final)
   double rel_kkt, res_primal, res_dual, res_gap, pobj, dobj, rnorm_mu, comp_mean;
   double rp_inf, rd_inf, rc_inf;

@@ -37,7 +37,8 @@ __device__ __forceinline__ double r_mul(double a, double b) { return a * b; }
 __device__ __forceinline__ double r_fms(double c, double a, double b) { return fma(-a, b, c); }   // c - a b
 __device__ __forceinline__ double r_rsqrt(double p) { return rsqrt(p); }
 // a > b for b > 0, by the order of the bits (a float64 comparison takes as long as a multiplication
-// and would lie on the chain from pivot to pivot); false where a or b is NaN.
+// and would lie on the chain from pivot to pivot); false where a is NaN.  (b is the floor of the pivot
+// a, kFloorRel times the diagonal entry that a started from: it is NaN only where a is.)
 __device__ __forceinline__ bool r_above(double a, double b) {
   const long long ia = __double_as_longlong(a);
   return ia > __double_as_longlong(b) && ia <= 0x7ff0000000000000ll;

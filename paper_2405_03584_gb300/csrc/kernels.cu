@@ -2007,13 +2007,14 @@ cudaError_t launch_apply_ru(const Dev& d, const Geo& g, cudaStream_t st) {
 
 // ------------------------------------------------------------------------------ recovery
 
-// The ratio test's quotient -v / dv of a positive v that falls (INFINITY otherwise) as the bits
-// of the float64: for the quotients met here (>= 0) their order as integers is the numbers', so
-// block and grid minima run on the integer pipe and one atomic a block; NaN never wins.
+// The ratio test's quotient -v / dv of a v that falls (INFINITY otherwise), as the key that orders
+// quotients on the integer pipe: block and grid minima run there, with one atomic a warp, and come
+// out as fmin's would (NaN is passed over; a negative quotient, of a v that rounding put past its
+// bound, counts as the number it is).
 __device__ __forceinline__ void keep_ratio(long long& m, double v, double dv) {
   if (dv < 0.0) {
-    const long long b = __double_as_longlong(-v / dv);
-    m = b < m ? b : m;
+    const long long k = min_key(__double_as_longlong(-v / dv));
+    m = k < m ? k : m;
   }
 }
 
@@ -2033,8 +2034,8 @@ __device__ __forceinline__ void block_ratio(const Dev& d, long long ap, long lon
 
 // alpha = min(1, tau times the minimum ratio), separate for (x, s) and (y, z) or their minimum.
 __device__ __forceinline__ void step_lengths(const Scal* sc, double& a_p, double& a_d) {
-  a_p = fmin(1.0, sc->tau * __longlong_as_double(sc->step_min[0]));
-  a_d = fmin(1.0, sc->tau * __longlong_as_double(sc->step_min[1]));
+  a_p = fmin(1.0, sc->tau * __longlong_as_double(min_key_bits(sc->step_min[0])));
+  a_d = fmin(1.0, sc->tau * __longlong_as_double(min_key_bits(sc->step_min[1])));
   if (sc->equal_steps) a_p = a_d = fmin(a_p, a_d);
 }
 
