@@ -1634,7 +1634,10 @@ static int load_qp(ipm_handle* h, const ipm_qp* qp, int64_t m_ar, void* stream) 
   CUDA_TRY(h, cudaMemcpyAsync(d.sc, h->hs, sizeof(Scal), cudaMemcpyHostToDevice, h->st));
   CUDA_TRY(h, launch_diagH(d, h->st));
   CUDA_TRY(h, launch_quantize(d, h->st));
+  CUDA_TRY(h, launch_find_repeats(d, h->st));
+  CUDA_TRY(h, cudaMemcpyAsync(&h->hs->repeats, &d.sc->repeats, sizeof(int), cudaMemcpyDeviceToHost, h->st));
   CUDA_TRY(h, cudaStreamSynchronize(h->st));   // host staging buffers go out of scope
+  h->d.repeats = h->hs->repeats;
   if ((rc = prepare_operator_formats(h))) return rc;
   if (nblk && (rc = prepare_block_segments(h, q.Rp, q.arow))) return rc;
   if (h->opt.autotune && !h->opt.lanes_rows && !h->opt.lanes_cols && (rc = autotune_groups(h))) return rc;

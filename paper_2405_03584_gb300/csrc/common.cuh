@@ -49,6 +49,7 @@ struct Scal {
   double stiff_gamma, stiff_thresh;
   int n_stiff, stiff_max, max_stiff_seen, chol_fail;
   int n_cand, sc_used;               // rows above gamma so far, stiff entries placed
+  int repeats;                       // a constraint row repeats a column (once a QP)
   // FP64 refinement of a reduced-precision Newton step
   double tol2_outer, rr_outer, refine_eta;
   // primal infeasibility certificate (Farkas): with (y, z) scaled by its largest entry,

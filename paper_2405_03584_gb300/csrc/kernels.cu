@@ -218,6 +218,20 @@ __global__ void k_diagH(Dev d) {
   }
 }
 
+// repeats = 1 where a constraint row repeats a column (rows increase within a column of A^T, so the
+// entries lie side by side).
+__global__ void k_find_repeats(Dev d) {
+  for (int64_t j = gwarp(); j < d.n; j += nwarps())
+    for (int64_t e = d.AT_ptr[j] + 1 + (threadIdx.x & 31); e < d.AT_ptr[j + 1]; e += 32)
+      if (d.AT_idx[e] == d.AT_idx[e - 1]) d.sc->repeats = 1;
+}
+
+cudaError_t launch_find_repeats(const Dev& d, cudaStream_t st) {
+  if (!d.m || !d.nnzA) return cudaSuccess;
+  k_find_repeats<<<(int)std::min<int64_t>((d.n + 7) / 8, 4096), kBlock, 0, st>>>(d);
+  return cudaGetLastError();
+}
+
 __global__ void k_fill_rowk(Dev d) {
   for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < d.nR; r += (int64_t)gridDim.x * blockDim.x)
     d.rowk[r] = -1;
@@ -1026,7 +1040,8 @@ __global__ void k_stiff_select(Dev d) {
 // one-block scan and a second pass took 21 us at n = 7001 and 53 us at n = 50000): each entry
 // (slot a, variable j) sets bit a of j's mask; the masks' counts give every variable a run of
 // the list; an entry's place in its run is the number of lower bits, so a run holds its slots in
-// increasing order.  (Runs are handed out in any order; nothing depends on where a run lies.)
+// increasing order.  (Runs are handed out in any order; nothing depends on where a run lies.)  A column
+// that a row repeats has one place, with the entries' sum, as the operator has it (Dev::repeats).
 __global__ void k_sc_mask(Dev d) {
   const int ns = d.sc->n_stiff, lane = threadIdx.x & 31;
   for (int a = gwarp(); a < ns; a += nwarps())
@@ -1051,7 +1066,12 @@ __global__ void k_sc_runs(Dev d) {
     int base = 0;
     if (lane == 31 && cum) base = atomicAdd(&d.sc->sc_used, cum);
     base = __shfl_sync(0xffffffffu, base, 31) + cum - cnt;
-    if (j < d.n) d.sc_run[j] = make_int2(base, base + cnt <= d.sc_cap ? cnt : 0);
+    if (j < d.n) {
+      const int run = base + cnt <= d.sc_cap ? cnt : 0;
+      d.sc_run[j] = make_int2(base, run);
+      if (d.repeats)
+        for (int t = 0; t < run; ++t) d.sc_val[base + t] = 0.0;
+    }
   }
 }
 
@@ -1066,7 +1086,8 @@ __global__ void k_sc_fill(Dev d) {
       for (int w = 0; w < (a >> 5); ++w) at += __popc(m[w]);
       if (at < run.y) {
         d.sc_slot[run.x + at] = a;
-        d.sc_val[run.x + at] = d.R_val[e];
+        if (d.repeats) atomicAdd(&d.sc_val[run.x + at], d.R_val[e]);
+        else d.sc_val[run.x + at] = d.R_val[e];
       }
     }
 }

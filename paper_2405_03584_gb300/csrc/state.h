@@ -60,6 +60,7 @@ struct Dev {
   unsigned* sc_mask;           // n x sc_words: the stiff rows of each variable, one bit a slot (shares
                                // dzl, dzu, z, p, q where these are large enough: it is dead by then)
   int sc_words;
+  int repeats;                 // a constraint row repeats a column (found at ipm_set_qp)
   int2* sc_run;                // n: first of a variable's stiff entries in sc_slot, sc_val, and their number
   int32_t* sc_slot; double* sc_val;  // sc_cap
   int64_t sc_cap;
@@ -285,6 +286,7 @@ cudaError_t launch_lr(const Dev& d, const double* v, int quad, cudaStream_t st);
 // ---- setup and start point ----
 cudaError_t launch_diagH(const Dev& d, cudaStream_t st);
 cudaError_t launch_fill_rowk(const Dev& d, cudaStream_t st);
+cudaError_t launch_find_repeats(const Dev& d, cudaStream_t st);   // sets the scalar `repeats`
 cudaError_t launch_densify_R(const Dev& d, cudaStream_t st);   // dense.cu: Rd from R (once per QP)
 cudaError_t launch_start_point(const Dev& d, const Geo& g, cudaStream_t st);
 // ---- residual summary at the current iterate and mu ----
