@@ -450,26 +450,29 @@ int heuristic_group(double avg_nnz) {
 //    rows of 100: 17, 18, 25, 33), 8 beyond (RT n = 50000, 250 a row: 141, 121, 143, -; VMAT 134 a
 //    row: 38, 32, 35, -);
 //  * columns (few, long): 16 lanes from 160 entries (n = 7001, 168 a column: 13.0, 8.4, 8.3, 11.7; n =
-//    50000, 1000 a column: 207, 137, 123, 149), 8 from 80 (20000 columns of 100: 13.1, 12.6, 15.2,
-//    20.7), else 4 (50000 columns of 50: 13.5, 16.4, 22.7, 33.1).  8 also for 160 to 256 entries where
-//    that makes 65536 lanes and R^T lies in one die's half of the L2: alone as fast as 16 (RT solves
-//    at n = 10007 / 12000 / 16000: 12.4 / 12.3 / 15.0 ms at 16, 12.2 / 12.1 / 15.0 at 8), and beside
-//    other solves, which share the float64 pipe with it, faster (16 in one launch at n = 12000: 66 ms
-//    and 57); beyond, the loads take longer and 16 lanes win alone (n = 20000: 18.4 ms and 19.1);
+//    50000, 1000 a column: 207, 137, 123, 149), 8 from 64 (20000 columns of 100: 13.1, 12.6, 15.2,
+//    20.7; n = 9000, 80 a column: 14.4, 10.7, 10.5, 12.6), else 4 (50000 columns of 50: 13.5, 16.4, 22.7,
+//    33.1).  8 also for 160 to 256 entries where that makes 65536 lanes and R^T lies in one die's half
+//    of the L2: alone as fast as 16 (RT solves at n = 10007 / 12000 / 16000: 12.4 / 12.3 / 15.0 ms at
+//    16, 12.2 / 12.1 / 15.0 at 8), and beside other solves, which share the float64 pipe with it, faster
+//    (16 in one launch at n = 12000: 66 ms and 57); beyond, the loads take longer and 16 lanes win
+//    alone (n = 20000: 18.4 ms and 19.1);
 //  * so few that 32768 lanes are not reached: wider while 8 entries a lane remain, columns up to 16
-//    lanes while 2 remain (dense n = 500, m = 1000: rows 20.7, 14.2, 10.1, 8.1; 1500 columns of 36: 8.4,
-//    8.2, 7.6, 8.1);
+//    lanes while 2 remain and, below 65536, up to 8 while 1 remains (dense n = 500, m = 1000: rows
+//    20.7, 14.2, 10.1, 8.1; 1500 columns of 36: 8.4, 8.2, 7.6, 8.1; 1100 of 16: 8.2, 7.5, 7.8, -);
 //  * so few that 98304 are not reached: wider while 16 entries a lane remain (4096 rows of 2048: 128,
 //    82, 47, 29, its columns 189, 96, 52, 31; 8192 rows of 512: 34, 25, 18, 19, its 4096 columns of 1024:
 //    85, 43, 25, 21; 16000 rows of 500 are enough at 8: 49, 31, 34, 30).
 // Reduced storages keep heuristic_group's widths: their float32 sums depend on it.
 int operator_group(double avg_nnz, int64_t rows, bool columns) {
-  int g = columns ? (avg_nnz >= 160.0 ? 16 : (avg_nnz >= 80.0 ? 8 : 4)) : (avg_nnz > 112.0 ? 8 : 4);
+  int g = columns ? (avg_nnz >= 160.0 ? 16 : (avg_nnz >= 64.0 ? 8 : 4)) : (avg_nnz > 112.0 ? 8 : 4);
   if (columns && g == 16 && avg_nnz <= 256.0 && 8 * rows >= 65536 && (double)rows * avg_nnz <= 4e6) return 8;
   while (g < 32) {
     const int64_t lanes = rows * g;
     const double left = avg_nnz / (2 * g);       // entries a lane at twice the width
-    if (!(lanes < 32768 && left >= (columns && g < 16 ? 2.0 : 8.0)) && !(lanes < 98304 && left >= 16.0)) break;
+    const bool few = columns && g < 16 ? (g == 4 ? lanes < 65536 && left >= 1.0 : lanes < 32768 && left >= 2.0)
+                                       : lanes < 32768 && left >= 8.0;
+    if (!few && !(lanes < 98304 && left >= 16.0)) break;
     g *= 2;
   }
   return g;

@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("rows,n,per_row,lanes_rows,lanes_cols", [
     (4096, 2048, 2048, 32, 32), (8192, 4096, 512, 16, 32), (8192, 4096, 1024, 16, 32), (2048, 1024, 1024, 32, 32),
     (1000, 50000, 2500, 32, 4), (500, 20000, 4000, 32, 8), (40000, 10000, 100, 4, 16),
-    (28004, 7001, 42, 4, 16), (48000, 12000, 60, 4, 8), (80000, 20000, 60, 4, 16), (6000, 1500, 9, 4, 16), (1000, 500, 500, 32, 32), (16000, 1000, 500, 8, 32)])
+    (28004, 7001, 42, 4, 16), (48000, 12000, 60, 4, 8), (80000, 20000, 60, 4, 16), (36000, 9000, 20, 4, 8), (4400, 1100, 4, 4, 8), (6000, 1500, 9, 4, 16), (1000, 500, 500, 32, 32), (16000, 1000, 500, 8, 32)])
 def test_widths(rows, n, per_row, lanes_rows, lanes_cols):
     rng = np.random.default_rng(1)
     first = rng.integers(0, n - per_row + 1, rows)
