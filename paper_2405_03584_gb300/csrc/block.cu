@@ -154,9 +154,8 @@ __global__ void __launch_bounds__(128) k_block_apply(Dev d, int init) {
     __syncwarp();
   }
   double v[1] = {rz};
-  const int ops[1] = {0};
   double out[1];
-  if (grid_reduce<1>(v, ops, d.partials + 28 * kMaxRedBlocks, &d.sc->ticket[T_CORR], out, sh)) {
+  if (grid_reduce<1>(v, d.partials + 28 * kMaxRedBlocks, &d.sc->ticket[T_CORR], out, sh)) {
     if (threadIdx.x == 0) {
       Scal* sc = d.sc;
       if (init) {

@@ -77,7 +77,7 @@ struct Scal {
   unsigned int ticket[8];
 };
 
-enum ScalTicket { T_PQ = 0, T_UPD = 1, T_CORR = 2, T_INIT = 3, T_HIST = 4, T_STEP = 5, T_MISC = 6, T_REF = 7 };
+enum ScalTicket { T_UPD = 0, T_CORR = 1, T_INIT = 2, T_HIST = 3, T_REF = 4 };
 
 // Storage of the matrix values used inside PCG (mirrors enum ipm_storage).
 enum Storage { ST_F64 = 0, ST_F32 = 1, ST_BF16 = 2, ST_FP8 = 3 };
@@ -96,25 +96,19 @@ __device__ __forceinline__ double warp_max(double v) {
   for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
-__device__ __forceinline__ double warp_min(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
 
 // Block-wide reductions in a fixed order (warp tree, then warp 0 over the warp results).
 // Every thread of the block must call them; the result is valid in every thread.
-template <int OP>  // 0 sum, 1 max, 2 min
+template <int OP>  // 0 sum, 1 max
 __device__ __forceinline__ double block_reduce(double v, double* sh /* >= 32 doubles */) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  v = OP == 0 ? warp_sum(v) : (OP == 1 ? warp_max(v) : warp_min(v));
+  v = OP == 0 ? warp_sum(v) : warp_max(v);
   __syncthreads();
   if (lane == 0) sh[wid] = v;
   __syncthreads();
   if (wid == 0) {
-    const double id = OP == 0 ? 0.0 : (OP == 1 ? -INFINITY : INFINITY);
-    double t = lane < nw ? sh[lane] : id;
-    t = OP == 0 ? warp_sum(t) : (OP == 1 ? warp_max(t) : warp_min(t));
+    double t = lane < nw ? sh[lane] : (OP == 0 ? 0.0 : -INFINITY);
+    t = OP == 0 ? warp_sum(t) : warp_max(t);
     if (lane == 0) sh[0] = t;
   }
   __syncthreads();
@@ -137,17 +131,15 @@ __device__ __forceinline__ double block_sum0(double v, double* sh /* >= 32 doubl
   return v;
 }
 
-// Last-block-done grid reduction.  Each block stores its partial for each of NQ quantities
-// at partials[q * kMaxRedBlocks + blockIdx.x]; the last block to arrive reduces them in
+// Last-block-done grid sums.  Each block stores its partial for each of NQ quantities
+// at partials[q * kMaxRedBlocks + blockIdx.x]; the last block to arrive adds them in
 // block-index order and returns true (in all of its threads) with the totals in out[].
-// Deterministic for a fixed grid size.  ops[q]: 0 sum, 1 max, 2 min.
+// Deterministic for a fixed grid size.
 template <int NQ>
-__device__ bool grid_reduce(const double (&v)[NQ], const int (&ops)[NQ], double* partials,
-                            unsigned int* ticket, double (&out)[NQ], double* sh) {
+__device__ bool grid_reduce(const double (&v)[NQ], double* partials, unsigned int* ticket, double (&out)[NQ], double* sh) {
   double r[NQ];
 #pragma unroll
-  for (int q = 0; q < NQ; ++q)
-    r[q] = ops[q] == 0 ? block_reduce<0>(v[q], sh) : (ops[q] == 1 ? block_reduce<1>(v[q], sh) : block_reduce<2>(v[q], sh));
+  for (int q = 0; q < NQ; ++q) r[q] = block_reduce<0>(v[q], sh);
   __shared__ bool s_last;
   if (threadIdx.x == 0) {
 #pragma unroll
@@ -161,13 +153,9 @@ __device__ bool grid_reduce(const double (&v)[NQ], const int (&ops)[NQ], double*
   __threadfence();
 #pragma unroll
   for (int q = 0; q < NQ; ++q) {
-    const double id = ops[q] == 0 ? 0.0 : (ops[q] == 1 ? -INFINITY : INFINITY);
-    double acc = id;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
-      double pv = __ldcg(partials + q * kMaxRedBlocks + b);
-      acc = ops[q] == 0 ? acc + pv : (ops[q] == 1 ? fmax(acc, pv) : fmin(acc, pv));
-    }
-    out[q] = ops[q] == 0 ? block_reduce<0>(acc, sh) : (ops[q] == 1 ? block_reduce<1>(acc, sh) : block_reduce<2>(acc, sh));
+    double acc = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) acc += __ldcg(partials + q * kMaxRedBlocks + b);
+    out[q] = block_reduce<0>(acc, sh);
   }
   if (threadIdx.x == 0) *ticket = 0u;
   return true;

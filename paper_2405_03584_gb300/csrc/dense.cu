@@ -91,16 +91,16 @@ __device__ __forceinline__ float2 r_floor(float2 fl) { return make_float2(fmaxf(
 //   * the panel: every block factors the diagonal tile in shared memory (the same code on the
 //     same data, so each gets the same factor; block 0 stores it in tiles[kb], which the last
 //     pass installs), then the others each solve 16 rows of the tiles below,
-//     X = A_ib,kb L_kb,kb^{-T}, one warp per row;
+//     X = A_ib,kb L_kb,kb^{-T}, four rows a warp;
 //   * the trailing update A_ib,jb -= L_ib,kb L_jb,kb^T (kb < jb <= ib) on 16 x 16 quarter tiles.
-// Each pivot takes one reciprocal square root and the rest multiplies by it (no division on
-// the chain), and the arithmetic of a tile column is spread over as many SMs as it has row
-// blocks.  The reciprocal pivots go to rinv[] for the triangular solves.  nn is read on the
+// Each pivot takes one reciprocal square root (float64) or one reciprocal (pairs, whose square
+// roots follow at the tile's end) and the rest multiplies by it, and the arithmetic of a tile
+// column is spread over as many SMs as it has row blocks.  The reciprocal pivots go to rinv[] for the triangular solves.  nn is read on the
 // device (it may be the number of stiff rows).  A pivot below floor_rel * (original diagonal)
 // is raised to that floor (a modified factor; still symmetric positive definite, which is all
 // a preconditioner needs); the count goes to *nfloor.
 constexpr int kT = 32;
-constexpr int kPanelRows = 16;  // rows of the panel below the diagonal tile per block 
+constexpr int kPanelRows = 16;  // rows below the diagonal tile that a panel block solves
 constexpr double kFloorRel = 1e-13;
 
 __device__ __forceinline__ int dev_nn(const int* nn_dev, int nn_fixed) { return nn_dev ? *nn_dev : nn_fixed; }

@@ -6,8 +6,9 @@
 // where R = [F; A_csr] and omega = w_R + theta placed on the constraint rows, so that
 // R^T diag(omega) R = F^T W F + A^T Theta A.  One PCG iteration is two streaming passes:
 // k_op_rows (row gather over R) and k_op_cols (row gather over the stored transpose R^T).
-// All reductions are block-tree + last-block sums in block order: results are bitwise
-// reproducible for a fixed problem size.
+// Sums over the grid are block parts added in block order, by the last block to arrive or by every
+// block of the kernel that needs them; maxima and minima, where the order does not matter, are
+// taken on the integer pipe.  Results are bitwise reproducible for a fixed problem size.
 #include <algorithm>
 #include <cmath>
 
@@ -77,10 +78,10 @@ Geo make_geo(const Dev& d) {
 // both passes read rows of U contiguously.
 //
 // A thread owns 8 columns (in 16-byte loads of two where rows start on 16 bytes; neighbouring
-// threads load neighbouring ones) and walks every rg-th row of its block's chunk, rg = 256 / ceil(ucols / 8) rows of
-// threads side by side: of 256 threads 250 carry columns at 200 columns, where 32 lanes over
-// 128-column slices carried 200 of 256 values, and every float64 instruction of a warp costs the
-// same.  (n = 77373, 200 columns: 41 us before.)  The rg partial sums of a column are added by as
+// threads load neighbouring ones) and walks every rg-th row of its block's chunk, rg = 256 /
+// ceil(ucols / 8) rows of threads side by side: of 256 threads 250 carry columns at 200 columns,
+// where 32 lanes over 128-column slices carried 200 of 256 values, and every float64 instruction of
+// a warp costs the same.  (n = 77373, 200 columns: 41 us before.)  The rg partial sums of a column are added by as
 // many threads as there are for it: by one thread a column they were a serial chain of 256 at up to
 // 8 columns (both kernels at n = 20000, 7 columns: 20.9 -> 15.0 us; n = 1000, one column: 20.9 -> 10.8).
 constexpr int kLrCols = 8;
@@ -1546,9 +1547,8 @@ __global__ void __launch_bounds__(256) k_cg_update(Dev d, int npart) {
     return;
   }
   const double v[1] = {rr};
-  const int ops[1] = {0};
   double out[1];
-  if (grid_reduce<1>(v, ops, d.partials + 17 * kMaxRedBlocks, &sc->ticket[T_UPD], out, sh)) {
+  if (grid_reduce<1>(v, d.partials + 17 * kMaxRedBlocks, &sc->ticket[T_UPD], out, sh)) {
     if (threadIdx.x == 0) {
       sc->pq = pq;
       sc->alpha = alpha;
@@ -1669,9 +1669,8 @@ __global__ void k_stiff_corr(Dev d, int init) {
     rz = fma(d.r[j], zj, rz);
   }
   double v[1] = {rz};
-  const int ops[1] = {0};
   double out[1];
-  if (grid_reduce<1>(v, ops, d.partials + 19 * kMaxRedBlocks, &d.sc->ticket[T_CORR], out, sh)) {
+  if (grid_reduce<1>(v, d.partials + 19 * kMaxRedBlocks, &d.sc->ticket[T_CORR], out, sh)) {
     if (threadIdx.x == 0) {
       Scal* sc = d.sc;
       if (init) {
@@ -1863,9 +1862,8 @@ __global__ void k_cg_init_diag(Dev d) {
     rz = fma(d.r[j], zj, rz);
   }
   double v[1] = {rz};
-  const int ops[1] = {0};
   double out[1];
-  if (grid_reduce<1>(v, ops, d.partials + 21 * kMaxRedBlocks, &d.sc->ticket[T_CORR], out, sh)) {
+  if (grid_reduce<1>(v, d.partials + 21 * kMaxRedBlocks, &d.sc->ticket[T_CORR], out, sh)) {
     if (threadIdx.x == 0) d.sc->rz = out[0];
   }
 }

@@ -529,9 +529,8 @@ __global__ void k_refine_resid(Dev d, cudaGraphConditionalHandle h, int set_cond
     rr = fma(rj, rj, rr);
   }
   double v[1] = {rr};
-  const int ops[1] = {0};
   double out[1];
-  if (grid_reduce<1>(v, ops, d.partials + 27 * kMaxRedBlocks, &d.sc->ticket[T_REF], out, sh)) {
+  if (grid_reduce<1>(v, d.partials + 27 * kMaxRedBlocks, &d.sc->ticket[T_REF], out, sh)) {
     if (threadIdx.x == 0) {
       Scal* sc = d.sc;
       sc->refine_it += 1;
@@ -618,16 +617,15 @@ __global__ void k_ru_update(Dev d, int npart) {
   const double alpha = good ? d.sc->rz / pq : 0.0;
   double rr = 0.0;
   if (good)
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < d.n; j += (int64_t)gridDim.x * blockDim.x) {
-    d.dx[j] = fma(alpha, d.p[j], d.dx[j]);
-    const double rj = fma(-alpha, d.q[j], d.r[j]);
-    d.r[j] = rj;
-    rr = fma(rj, rj, rr);
-  }
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < d.n; j += (int64_t)gridDim.x * blockDim.x) {
+      d.dx[j] = fma(alpha, d.p[j], d.dx[j]);
+      const double rj = fma(-alpha, d.q[j], d.r[j]);
+      d.r[j] = rj;
+      rr = fma(rj, rj, rr);
+    }
   double v[1] = {rr};
-  const int ops[1] = {0};
   double out[1];
-  if (grid_reduce<1>(v, ops, d.partials + 17 * kMaxRedBlocks, &d.sc->ticket[T_UPD], out, sh)) {
+  if (grid_reduce<1>(v, d.partials + 17 * kMaxRedBlocks, &d.sc->ticket[T_UPD], out, sh)) {
     if (threadIdx.x == 0) {
       Scal* sc = d.sc;
       sc->pq = pq;
@@ -663,9 +661,8 @@ __global__ void k_ru_resid(Dev d) {
     rr = fma(rj, rj, rr);
   }
   double v[1] = {rr};
-  const int ops[1] = {0};
   double out[1];
-  if (grid_reduce<1>(v, ops, d.partials + 27 * kMaxRedBlocks, &d.sc->ticket[T_REF], out, sh)) {
+  if (grid_reduce<1>(v, d.partials + 27 * kMaxRedBlocks, &d.sc->ticket[T_REF], out, sh)) {
     if (threadIdx.x == 0) {
       Scal* sc = d.sc;
       sc->refine_it += 1;
@@ -704,9 +701,8 @@ __global__ void k_ru_z(Dev d) {
   }
   if (ZM == 1) return;
   double v[1] = {rz};
-  const int ops[1] = {0};
   double out[1];
-  if (grid_reduce<1>(v, ops, d.partials + 29 * kMaxRedBlocks, &d.sc->ticket[T_CORR], out, sh)) {
+  if (grid_reduce<1>(v, d.partials + 29 * kMaxRedBlocks, &d.sc->ticket[T_CORR], out, sh)) {
     if (threadIdx.x == 0) {
       Scal* sc = d.sc;
       sc->beta = out[0] / sc->rz;

@@ -12,11 +12,11 @@
 // however many lanes it serves: an instruction that every warp of a block executes for a value
 // they all share costs more than a barrier.  As separate kernels (update, A_s z, G^{-1} u,
 // correction, p), each with its own last-block sum, the half took 27 us an iteration at n =
-// 1500 and 30 us at n = 50000 (9.9 us and 20.8 us here).  One thread-block cluster runs it
+// 1500 and 34 us at n = 50000 (9 us and 22 us here).  One thread-block cluster runs it
 // instead: its CTAs are resident together, so a global sum is one exchange through distributed
 // shared memory and one cluster barrier, the vectors stay in registers from the update to the
-// new p, and the loads of a phase are issued before the barrier that precedes it.  Scalars are formed by one warp and handed
-// out through shared memory; warps without unknowns skip the vector arithmetic; the trees of a
+// new p, and the loads of a phase are issued before the barrier that precedes it.  Scalars are
+// formed by one warp and handed out through shared memory; warps without unknowns skip the vector arithmetic; the trees of a
 // sum are formed from shared memory by 8 lanes per 32 values (6 float64 instructions for four
 // trees a warp, against 20 by shuffles alone).
 //
