@@ -80,6 +80,9 @@ def _moved(f, tmp_path):
 
 def test_bytes_moved(tmp_path):
     n, m, scalars = 30000, 2000, 4096
+    t = torch.zeros(1000, device="cuda")
+    if _moved(lambda: t.cpu(), tmp_path) != 4000:
+        pytest.skip("the profiler records no copies here")
     s = _solver(n, m)
     assert _moved(lambda: _call("get", s, ["x"], False), tmp_path) == 8 * n
     assert _moved(lambda: _call("get", s, [], False), tmp_path) == 0
